@@ -29,6 +29,12 @@ void set_err(const char *fmt, ...) {
 constexpr int kMaxLev = 16;
 constexpr int kMaxCoarse = 3072;
 constexpr int kProfSlots = 64;
+// Top levels of at most this many nodes run their V-cycles in one cluster of
+// 16 SMs.  FP32: whatever fits its shared memory (up to about 60000 nodes) is
+// faster there than in separate launches.  FP64: 2 operations a clock and SM
+// make 16 SMs slower than the chip on a 32^3 level (77 against 9 us of pure
+// issue a sweep), not on a 16^3 one.
+constexpr long kSmallNodes64 = 8192, kSmallNodes32 = 100000;
 constexpr int kMaxInner = 10;  // cap on FP32 V-cycles per refinement step
 
 // n FP32 V-cycles (from e = 0) captured once and replayed; the event pairs
@@ -74,6 +80,10 @@ struct mg_ctx {
     int split0;            // finest FP32 arrays in parity-split column order
     double *Ainv;
     int ncoarse;
+    // V-cycles of the levels from top64 / top32 down in one launch (-1: none)
+    SmallPlan<double> s64;
+    SmallPlan<float> s32;
+    int top64, top32;
     double *partials, *dsum, *hsum;
     // cross-CTA state of the fused finest-level sweep (when it applies)
     SweepSync sync;
@@ -89,7 +99,7 @@ struct mg_ctx {
     long pend_sweeps[kProfSlots], pend_launches[kProfSlots];
     int npend;
     // FP32 inner V-cycles as CUDA graphs, one per cycle count
-    InnerGraph *graphs[kMaxInner + 1];
+    InnerGraph *graphs[2][kMaxInner + 1];  // [profiling][cycles]
     cudaStream_t cap;  // private stream used only to capture them
     InnerGraph *capturing;
     double prof_ms;
@@ -476,8 +486,8 @@ mg_status prof_push(mg_ctx *ctx, cudaEvent_t e0, cudaEvent_t e1, long sweeps, lo
 template <typename T>
 mg_status smooth(mg_ctx *ctx, int l, const T *b, T *x, int sweeps_n, bool descending) {
     InnerGraph *G = ctx->capturing;
-    const bool timed = l == 0 && sweeps_n > 0 &&
-                       (G ? G->nev < 2 * kMaxInner : ctx->prof_on);
+    const bool timed = l == 0 && sweeps_n > 0 && ctx->prof_on &&
+                       (!G || G->nev < 2 * kMaxInner);
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     if (timed && !G) {
         if (ctx->npend == kProfSlots) {
@@ -580,9 +590,29 @@ mg_status residual_restrict_level<float>(mg_ctx *ctx, int l, const float *b, con
     return MG_OK;
 }
 
-// one V-cycle for A_l x = b on level l (section 3.6)
+// the level from which V-cycles run as one launch, or -1.  With profiling
+// on, level 0 keeps separate launches, whose smoothing the timers bracket.
+template <typename T>
+int small_top(const mg_ctx *ctx);
+template <>
+int small_top<double>(const mg_ctx *ctx) {
+    return ctx->prof_on && ctx->top64 == 0 ? -1 : ctx->top64;
+}
+template <>
+int small_top<float>(const mg_ctx *ctx) {
+    return ctx->prof_on && ctx->top32 == 0 ? -1 : ctx->top32;
+}
+inline const SmallPlan<double> &small_plan_of(const mg_ctx *ctx, double) { return ctx->s64; }
+inline const SmallPlan<float> &small_plan_of(const mg_ctx *ctx, float) { return ctx->s32; }
+
+// one V-cycle for A_l x = b on level l (section 3.6); below level 0 x is
+// taken as zero on entry
 template <typename T>
 mg_status vcycle(mg_ctx *ctx, int l, const T *b, T *x) {
+    if (l == small_top<T>(ctx)) {
+        CK(small_cycle<T>(small_plan_of(ctx, T()), b, x, l > 0, 1, ctx->st));
+        return MG_OK;
+    }
     T *r = Bufs<T>::r(ctx, l);
     if (l == ctx->nlev - 1) {
         CKS(residual_level<T>(ctx, l, b, x, r));
@@ -592,7 +622,8 @@ mg_status vcycle(mg_ctx *ctx, int l, const T *b, T *x) {
     CKS(smooth<T>(ctx, l, b, x, ctx->opts.nu1, false));
     T *bc = Bufs<T>::b(ctx, l + 1), *xc = Bufs<T>::x(ctx, l + 1);
     CKS(residual_restrict_level<T>(ctx, l, b, x, r, bc));
-    CK(cudaMemsetAsync(xc, 0, corner_count(ctx->L[l + 1]) * sizeof(T), ctx->st));
+    if (l + 1 != small_top<T>(ctx))
+        CK(cudaMemsetAsync(xc, 0, corner_count(ctx->L[l + 1]) * sizeof(T), ctx->st));
     CKS(vcycle<T>(ctx, l + 1, bc, xc));
     CK(prolong_add_any(ctx->L[l], xc, x, ctx->st, split_of<T>(ctx, l)));
     CKS(smooth<T>(ctx, l, b, x, ctx->opts.nu2, true));
@@ -666,6 +697,10 @@ int inner_count(const mg_ctx *ctx, double rel, double tol, double kappa) {
 
 // n FP32 V-cycles on the finest correction equation from e = 0
 mg_status inner_cycles_direct(mg_ctx *ctx, int n) {
+    if (small_top<float>(ctx) == 0) {
+        CK(small_cycle<float>(ctx->s32, ctx->b32[0], ctx->x32[0], true, n, ctx->st));
+        return MG_OK;
+    }
     CK(cudaMemsetAsync(ctx->x32[0], 0, corner_count(ctx->L[0]) * sizeof(float), ctx->st));
     for (int c = 0; c < n; c++) CKS(vcycle<float>(ctx, 0, ctx->b32[0], ctx->x32[0]));
     return MG_OK;
@@ -674,11 +709,14 @@ mg_status inner_cycles_direct(mg_ctx *ctx, int n) {
 // the same as one CUDA graph: captured on the private stream at first use,
 // replayed on the context's stream
 mg_status inner_cycles(mg_ctx *ctx, int n) {
-    if (ctx->opts.flags & MG_FLAG_NO_GRAPH) return inner_cycles_direct(ctx, n);
-    InnerGraph *G = ctx->graphs[n];
+    if ((ctx->opts.flags & MG_FLAG_NO_GRAPH) || small_top<float>(ctx) == 0)
+        return inner_cycles_direct(ctx, n);
+    // timed graphs carry event records around the finest smoothing
+    InnerGraph *&slot = ctx->graphs[ctx->prof_on ? 1 : 0][n];
+    InnerGraph *G = slot;
     if (!G) {
         G = new InnerGraph();
-        ctx->graphs[n] = G;
+        slot = G;
         for (int i = 0; i < 2 * kMaxInner; i++) {
             CK(cudaEventCreate(&G->ev[i][0]));
             CK(cudaEventCreate(&G->ev[i][1]));
@@ -836,8 +874,8 @@ void mg_free(mg_ctx *ctx) {
             cudaEventDestroy(ctx->ev[i][0]);
             cudaEventDestroy(ctx->ev[i][1]);
         }
-    for (int n = 0; n <= kMaxInner; n++) {
-        InnerGraph *G = ctx->graphs[n];
+    for (int n = 0; n < 2 * (kMaxInner + 1); n++) {
+        InnerGraph *G = ctx->graphs[n / (kMaxInner + 1)][n % (kMaxInner + 1)];
         if (!G) continue;
         if (G->exec) cudaGraphExecDestroy(G->exec);
         for (int i = 0; i < 2 * kMaxInner; i++) {
@@ -945,6 +983,7 @@ mg_status mg_setup(const mg_grid *grid, const mg_moduli *moduli, const mg_bc *bc
     {
         cudaError_t e = smoother_init();
         if (e == cudaSuccess) e = plane_init();
+        if (e == cudaSuccess) e = small_init();
         if (e != cudaSuccess) {
             set_err("mg_setup: %s", cudaGetErrorString(e));
             delete ctx;
@@ -1017,6 +1056,20 @@ mg_status mg_setup(const mg_grid *grid, const mg_moduli *moduli, const mg_bc *bc
         s = MG_ERR_CUDA;
         goto fail;
     }
+    ctx->top64 = ctx->top32 = -1;
+    for (int l = 0; l + 1 < ctx->nlev; l++) {
+        const int f = opts->flags;
+        if (ctx->top64 < 0 && small_plan(ctx->L + l, ctx->c64 + l, ctx->nlev - l, ctx->ncoarse,
+                                         ctx->Ainv, opts->nu1, opts->nu2, kSmallNodes64, ctx->s64))
+            ctx->top64 = l;
+        // the flags that choose how FP32 sweeps or finest transfers run are obeyed
+        if (ctx->top32 < 0 && !(f & MG_FLAG_COLOUR_PASSES) &&
+            !(l == 0 && (f & (MG_FLAG_FUSED_SWEEP | MG_FLAG_UNFUSED_TRANSFERS))) &&
+            small_plan(ctx->L + l, ctx->c32 + l, ctx->nlev - l, ctx->ncoarse, ctx->Ainv,
+                       opts->nu1, opts->nu2, kSmallNodes32, ctx->s32))
+            ctx->top32 = l;
+    }
+    if (ctx->top32 == 0) ctx->split0 = 0;  // its arrays are in natural order
     *out = ctx;
     return MG_OK;
 fail:

@@ -126,6 +126,35 @@ cudaError_t gs_colour_coarse(const Dims &d, const Coarse<double> &c, const doubl
 cudaError_t gs_colour_coarse(const Dims &d, const Coarse<float> &c, const float *b, float *x,
                              int colour, cudaStream_t s);
 
+// V-cycle of the small levels in one launch (small_cycle.cu).  Offsets are
+// in elements of the CTA's shared memory; m* are division multipliers.
+constexpr int kSmallLevels = 6, kSmallCoarse = 768;
+struct SmallLevel {
+    int nx, ny, nz, np, ppc;  // np = nx ny; ppc: interior planes per CTA
+    int hx, w, pl;            // nx / 2 (0: coarsest), row pitch, plane size
+    unsigned mnx, mnp, mhx, mnh, mppc, mpl;
+    int x, b, p;  // x, right-hand side, x-y restricted residual
+};
+template <typename T>
+struct SmallPlan {
+    int nlev, nu1, nu2, ncoarse;
+    int plmax, scratch;  // the largest plane; offset of the scratch
+    int threads, nodes;  // threads of a CTA, nodes of a plane a thread may own
+    size_t smem;
+    const double *Ainv;
+    SmallLevel lev[kSmallLevels];
+    Coarse<T> op[kSmallLevels];
+};
+cudaError_t small_init();
+template <typename T>
+bool small_plan(const Dims *d, const Coarse<T> *op, int nlev, int ncoarse, const double *Ainv,
+                int nu1, int nu2, long max_nodes, SmallPlan<T> &g);
+// `cycles` V-cycles for A x = b on the plan's top level; from_zero: x is
+// taken as zero on entry (its wall planes too) and only its interior is written
+template <typename T>
+cudaError_t small_cycle(const SmallPlan<T> &g, const T *b, T *x, bool from_zero, int cycles,
+                        cudaStream_t s);
+
 // one-time kernel attribute set-up of the sweeps (call before any capture):
 // smoother_init for the row-strip kernels, plane_init for the whole-plane one
 cudaError_t smoother_init();
