@@ -12,6 +12,24 @@ namespace qsmg {
 namespace {
 
 constexpr int kThreads = 256;
+constexpr int kLinThreads = 128;  // most threads of the linear-order kernels
+
+// threads of a block for np nodes a plane, `planes` planes: fewer on small
+// levels, so that every SM gets some
+inline int lin_threads(long np, long planes) {
+    int nt = kLinThreads;
+    while (nt > 32 && (np + nt - 1) / nt * planes < 608) nt /= 2;
+    return nt;
+}
+// multiplier m for t / d = umulhi(t, m) with t < n; 0 where that is not exact
+inline unsigned magic(int d, long n) {
+    return d == 1 || n * d >= (1L << 32) ? 0u : (unsigned)((1ull << 32) / (unsigned)d + 1);
+}
+__device__ __forceinline__ int fdiv(int t, int d, unsigned m) {
+    return m ? (int)__umulhi((unsigned)t, m) : t / d;
+}
+// FP32 prolongation takes one component a thread up to this many coarse cells
+constexpr long kProlongSplit = 1L << 17;
 
 inline unsigned nblocks(long n, int t = kThreads) { return (unsigned)((n + t - 1) / t); }
 
@@ -257,39 +275,37 @@ __global__ void __launch_bounds__(1024) k_sum_partials(const double *__restrict_
 }
 
 // restriction R = T^T (full weighting, weights 1, 1/2, 1/4, 1/8 by the
-// number of odd offsets), coarse interior nodes
+// number of odd offsets), coarse interior nodes; one thread a node component,
+// nodes of a plane dealt in linear order so that small planes fill their
+// warps (a level of 16^3 takes 4 us against 9.5 in FP64 with three
+// components a thread and 32 x 8 blocks: half its lanes and most SMs idle)
 template <typename T>
-__global__ void k_restrict(Dims f, Dims c, const T *__restrict__ r, T *__restrict__ bc,
-                           int split) {
-    int I, J, K;
-    if (!node_ijk(c, I, J, K)) return;
-    T s0 = 0, s1 = 0, s2 = 0;
+__global__ void __launch_bounds__(kLinThreads)
+    k_restrict(Dims f, Dims c, unsigned mnx, const T *__restrict__ r, T *__restrict__ bc,
+               int split) {
+    const int m = blockIdx.x * blockDim.x + threadIdx.x;
+    if (m >= c.nx * c.ny) return;
+    const int J = fdiv(m, c.nx, mnx), I = m - J * c.nx;
+    const int K = blockIdx.y + 1, a = blockIdx.z;
+    const T h = T(0.5);
+    const int i0 = colmap(2 * I, f.nx, split), ip = colmap(2 * I + 1, f.nx, split),
+              im = colmap(I ? 2 * I - 1 : f.nx - 1, f.nx, split);
+    const T *ra = r + a * f.cs;
+    T z[3];
 #pragma unroll
     for (int ez = -1; ez <= 1; ez++) {
-        const T wz = ez ? T(0.5) : T(1);
         const long pl = (long)(2 * K + ez) * f.ny;
+        T y[3];
 #pragma unroll
         for (int ey = -1; ey <= 1; ey++) {
-            const T wy = ey ? T(0.5) : T(1);
             int jj = 2 * J + ey;
-            jj = jj < 0 ? jj + f.ny : (jj >= f.ny ? jj - f.ny : jj);
-            const long row = (pl + jj) * f.nx;
-#pragma unroll
-            for (int ex = -1; ex <= 1; ex++) {
-                const T w = (ex ? T(0.5) : T(1)) * wy * wz;
-                int ii = 2 * I + ex;
-                ii = ii < 0 ? ii + f.nx : (ii >= f.nx ? ii - f.nx : ii);
-                const long q = row + colmap(ii, f.nx, split);
-                s0 += w * r[q];
-                s1 += w * r[q + f.cs];
-                s2 += w * r[q + 2 * f.cs];
-            }
+            jj = jj < 0 ? jj + f.ny : jj;
+            const T *row = ra + (pl + jj) * f.nx;
+            y[ey + 1] = row[i0] + h * (row[im] + row[ip]);
         }
+        z[ez + 1] = y[1] + h * (y[0] + y[2]);
     }
-    const long p = ((long)K * c.ny + J) * c.nx + I;
-    bc[p] = s0;
-    bc[p + c.cs] = s1;
-    bc[p + 2 * c.cs] = s2;
+    bc[a * c.cs + (long)K * c.ny * c.nx + m] = z[1] + h * (z[0] + z[2]);
 }
 
 // z part of the full weighting, after the fused fine residual of
@@ -383,6 +399,53 @@ __global__ void k_prolong(Dims f, Dims c, const T *__restrict__ xc, T *__restric
                 }
             }
         }
+}
+
+// the same one component a thread, cells of a plane in linear order: for
+// levels too small to fill the chip with three components a thread, and in
+// FP64, where every instruction of a half-empty warp costs a full one
+template <typename T>
+__global__ void __launch_bounds__(kLinThreads)
+    k_prolong_c(Dims f, Dims c, unsigned mnx, const T *__restrict__ xc, T *__restrict__ x,
+                int split) {
+    const int m = blockIdx.x * blockDim.x + threadIdx.x;
+    if (m >= c.nx * c.ny) return;
+    const int J = fdiv(m, c.nx, mnx), I = m - J * c.nx;
+    const int K = blockIdx.y, a = blockIdx.z;
+    const int I1 = I + 1 < c.nx ? I + 1 : 0, J1 = J + 1 < c.ny ? J + 1 : 0;
+    const long cps = (long)c.nx * c.ny, fps = (long)f.nx * f.ny;
+    const int fcol[2] = {colmap(2 * I, f.nx, split), colmap(2 * I + 1, f.nx, split)};
+    const T h = T(0.5);
+    const T *X = xc + a * c.cs + (long)K * cps;
+    T *xf = x + a * f.cs + (long)(2 * K) * fps + (long)(2 * J) * f.nx;
+    T w[2][2][2], old[2][2][2];  // [z][fine b][fine e]
+    const int cz0 = K == 0 ? 1 : 0;  // fine plane 0 is a wall
+#pragma unroll
+    for (int z = 0; z < 2; z++) {
+        const T v00 = X[z * cps + (long)J * c.nx + I], v01 = X[z * cps + (long)J * c.nx + I1];
+        const T v10 = X[z * cps + (long)J1 * c.nx + I], v11 = X[z * cps + (long)J1 * c.nx + I1];
+        const T a0 = h * (v00 + v01), a1 = h * (v10 + v11);
+        w[z][0][0] = v00;
+        w[z][0][1] = a0;
+        w[z][1][0] = h * (v00 + v10);
+        w[z][1][1] = h * (a0 + a1);
+    }
+#pragma unroll
+    for (int z = 0; z < 2; z++)
+#pragma unroll
+        for (int b = 0; b < 2; b++)
+#pragma unroll
+            for (int e = 0; e < 2; e++)
+                if (z >= cz0) old[z][b][e] = xf[z * fps + (long)b * f.nx + fcol[e]];
+#pragma unroll
+    for (int z = 0; z < 2; z++)
+#pragma unroll
+        for (int b = 0; b < 2; b++)
+#pragma unroll
+            for (int e = 0; e < 2; e++)
+                if (z >= cz0)
+                    xf[z * fps + (long)b * f.nx + fcol[e]] =
+                        old[z][b][e] + (z ? h * (w[0][b][e] + w[1][b][e]) : w[0][b][e]);
 }
 
 // x += Ainv r on the coarsest level; one warp per unknown, fixed-order sums.
@@ -585,7 +648,9 @@ template <typename T>
 static cudaError_t restrict_t(const Dims &f, const T *r, T *bc, cudaStream_t s, int split) {
     const Dims c = make_dims(f.nx / 2, f.ny / 2, f.nz / 2);
     if (c.nz < 2) return cudaSuccess;
-    k_restrict<T><<<node_grid(c.nx, c.ny, c.nz - 1), kBlock, 0, s>>>(f, c, r, bc, split);
+    const int nt = lin_threads((long)c.nx * c.ny, 3L * (c.nz - 1));
+    const dim3 grid((c.nx * c.ny + nt - 1) / nt, c.nz - 1, 3);
+    k_restrict<T><<<grid, nt, 0, s>>>(f, c, magic(c.nx, (long)c.nx * c.ny), r, bc, split);
     count_launch();
     return cudaGetLastError();
 }
@@ -608,7 +673,13 @@ cudaError_t restrict_z(const Dims &fine, const float *part, float *bc, cudaStrea
 template <typename T>
 static cudaError_t prolong_t(const Dims &f, const T *xc, T *x, cudaStream_t s, int split) {
     const Dims c = make_dims(f.nx / 2, f.ny / 2, f.nz / 2);
-    k_prolong<T><<<node_grid(c.nx, c.ny, c.nz), kBlock, 0, s>>>(f, c, xc, x, split);
+    if (sizeof(T) == 8 || (long)c.nx * c.ny * c.nz <= kProlongSplit) {
+        const int nt = lin_threads((long)c.nx * c.ny, 3L * c.nz);
+        const dim3 grid((c.nx * c.ny + nt - 1) / nt, c.nz, 3);
+        k_prolong_c<T><<<grid, nt, 0, s>>>(f, c, magic(c.nx, (long)c.nx * c.ny), xc, x, split);
+    } else {
+        k_prolong<T><<<node_grid(c.nx, c.ny, c.nz), kBlock, 0, s>>>(f, c, xc, x, split);
+    }
     count_launch();
     return cudaGetLastError();
 }

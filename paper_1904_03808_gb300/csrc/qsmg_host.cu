@@ -31,10 +31,11 @@ constexpr int kMaxCoarse = 3072;
 constexpr int kProfSlots = 64;
 // Top levels of at most this many nodes run their V-cycles in one cluster of
 // 16 SMs.  FP32: whatever fits its shared memory (up to about 60000 nodes) is
-// faster there than in separate launches.  FP64: 2 operations a clock and SM
-// make 16 SMs slower than the chip on a 32^3 level (77 against 9 us of pure
-// issue a sweep), not on a 16^3 one.
-constexpr long kSmallNodes64 = 8192, kSmallNodes32 = 100000;
+// faster there than in separate launches.  FP64: with 2 operations a clock and
+// SM, 16 SMs take longer over a 16^3 level than row strips on the whole chip
+// (64^3 gradient 68.1 against 65.1 ms with the limit at 8192 and 1000 nodes),
+// not over an 8^3 one.
+constexpr long kSmallNodes64 = 2048, kSmallNodes32 = 100000;
 constexpr int kMaxInner = 10;  // cap on FP32 V-cycles per refinement step
 
 // n FP32 V-cycles (from e = 0) captured once and replayed; the event pairs
@@ -101,6 +102,7 @@ struct mg_ctx {
     // FP32 inner V-cycles as CUDA graphs, one per cycle count
     InnerGraph *graphs[2][kMaxInner + 1];  // [profiling][cycles]
     cudaStream_t cap;  // private stream used only to capture them
+    InnerGraph *graph64;  // the FP64 V-cycle from level 1 down, on own arrays
     InnerGraph *capturing;
     double prof_ms;
     long prof_sweeps, prof_launches;
@@ -451,9 +453,29 @@ mg_status sweeps_colour(mg_ctx *ctx, int l, const T *b, T *x, int sweeps, bool d
     return MG_OK;
 }
 
+// FP64: row strips in two launches a sweep where the rows fit, ping-ponging
+// with the level's residual buffer, else colour launches
 template <typename T>
 mg_status sweeps(mg_ctx *ctx, int l, const T *b, T *x, int n, bool descending) {
-    return sweeps_colour<T>(ctx, l, b, x, n, descending);
+    const Dims &d = ctx->L[l];
+    if (!strip_fits(d, l == 0)) return sweeps_colour<T>(ctx, l, b, x, n, descending);
+    T *a = x, *o = ctx->r64[l];
+    for (int s = 0; s < n; s++) {
+        if (l == 0)
+            CK(gs_sweep_strip(d, ctx->f64, b, a, x, o, descending, ctx->st));
+        else
+            CK(gs_sweep_strip(d, ctx->c64[l], b, a, x, o, descending, ctx->st));
+        T *t = a;
+        a = o;
+        o = t;
+    }
+    if (a != x) {  // interior planes back
+        const size_t plane = (size_t)d.ny * d.nx;
+        for (int c = 0; c < 3; c++)
+            CK(cudaMemcpyAsync(x + c * d.cs + plane, a + c * d.cs + plane,
+                               (d.nz - 1) * plane * sizeof(T), cudaMemcpyDeviceToDevice, ctx->st));
+    }
+    return MG_OK;
 }
 
 // FP32: the two-phase kernels (row strips where the rows fit, else tiles),
@@ -532,10 +554,15 @@ int split_of<float>(const mg_ctx *ctx, int l) {
 
 template <typename T>
 mg_status residual_level(mg_ctx *ctx, int l, const T *b, const T *x, T *r) {
+    const Dims &d = ctx->L[l];
+    // the coarsest level may have odd sizes, and is never smoothed
+    const bool strip = l + 1 < ctx->nlev && strip_fits(d, l == 0);
     if (l == 0)
-        CK(residual_fine(ctx->L[0], Bufs<T>::fine(ctx), b, x, r, ctx->st));
+        CK(strip ? residual_strip(d, ctx->f64, b, x, r, ctx->st)
+                 : residual_fine(d, Bufs<T>::fine(ctx), b, x, r, ctx->st));
     else
-        CK(residual_coarse(ctx->L[l], Bufs<T>::coarse(ctx, l), b, x, r, ctx->st));
+        CK(strip ? residual_strip(d, ctx->c64[l], b, x, r, ctx->st)
+                 : residual_coarse(d, Bufs<T>::coarse(ctx, l), b, x, r, ctx->st));
     return MG_OK;
 }
 
@@ -590,6 +617,31 @@ mg_status residual_restrict_level<float>(mg_ctx *ctx, int l, const float *b, con
     return MG_OK;
 }
 
+// what `body` issues on the context's stream, captured on the private stream
+// into G instead
+template <class Body>
+mg_status capture_graph(mg_ctx *ctx, InnerGraph *G, const Body &body) {
+    cudaStream_t user = ctx->st;
+    const long k0 = g_launches.load();
+    CK(cudaStreamBeginCapture(ctx->cap, cudaStreamCaptureModeThreadLocal));
+    ctx->st = ctx->cap;
+    const mg_status s = body();
+    ctx->st = user;
+    cudaGraph_t graph = nullptr;
+    const cudaError_t ee = cudaStreamEndCapture(ctx->cap, &graph);
+    G->kernels = g_launches.load() - k0;
+    g_launches.fetch_sub(G->kernels);  // counted when replayed, not when captured
+    if (s != MG_OK) {
+        if (graph) cudaGraphDestroy(graph);
+        return s;
+    }
+    CK(ee);
+    const cudaError_t ei = cudaGraphInstantiate(&G->exec, graph, 0);
+    cudaGraphDestroy(graph);
+    CK(ei);
+    return MG_OK;
+}
+
 // the level from which V-cycles run as one launch, or -1.  With profiling
 // on, level 0 keeps separate launches, whose smoothing the timers bracket.
 template <typename T>
@@ -604,6 +656,37 @@ int small_top<float>(const mg_ctx *ctx) {
 }
 inline const SmallPlan<double> &small_plan_of(const mg_ctx *ctx, double) { return ctx->s64; }
 inline const SmallPlan<float> &small_plan_of(const mg_ctx *ctx, float) { return ctx->s32; }
+
+template <typename T>
+mg_status vcycle(mg_ctx *ctx, int l, const T *b, T *x);
+
+// the V-cycle on level l + 1 from xc = 0
+template <typename T>
+mg_status coarse_cycle_direct(mg_ctx *ctx, int l, const T *bc, T *xc) {
+    if (l + 1 != small_top<T>(ctx))
+        CK(cudaMemsetAsync(xc, 0, corner_count(ctx->L[l + 1]) * sizeof(T), ctx->st));
+    return vcycle<T>(ctx, l + 1, bc, xc);
+}
+mg_status coarse_cycle(mg_ctx *ctx, int l, const float *bc, float *xc) {
+    return coarse_cycle_direct<float>(ctx, l, bc, xc);
+}
+
+// FP64 below the finest level: one CUDA graph on the context's own arrays
+// (the finest level works on the caller's), captured at its first use; a
+// launch of its own costs the host 2.6 us, one inside a graph the device 0.5
+mg_status coarse_cycle(mg_ctx *ctx, int l, const double *bc, double *xc) {
+    if (l != 0 || small_top<double>(ctx) == 1 || ctx->nlev < 3 ||
+        (ctx->opts.flags & MG_FLAG_NO_GRAPH))
+        return coarse_cycle_direct<double>(ctx, l, bc, xc);
+    if (!ctx->graph64) {
+        InnerGraph *G = new InnerGraph();
+        ctx->graph64 = G;
+        CKS(capture_graph(ctx, G, [&] { return coarse_cycle_direct<double>(ctx, l, bc, xc); }));
+    }
+    CK(cudaGraphLaunch(ctx->graph64->exec, ctx->st));
+    count_launch(ctx->graph64->kernels);
+    return MG_OK;
+}
 
 // one V-cycle for A_l x = b on level l (section 3.6); below level 0 x is
 // taken as zero on entry
@@ -622,9 +705,7 @@ mg_status vcycle(mg_ctx *ctx, int l, const T *b, T *x) {
     CKS(smooth<T>(ctx, l, b, x, ctx->opts.nu1, false));
     T *bc = Bufs<T>::b(ctx, l + 1), *xc = Bufs<T>::x(ctx, l + 1);
     CKS(residual_restrict_level<T>(ctx, l, b, x, r, bc));
-    if (l + 1 != small_top<T>(ctx))
-        CK(cudaMemsetAsync(xc, 0, corner_count(ctx->L[l + 1]) * sizeof(T), ctx->st));
-    CKS(vcycle<T>(ctx, l + 1, bc, xc));
+    CKS(coarse_cycle(ctx, l, bc, xc));
     CK(prolong_add_any(ctx->L[l], xc, x, ctx->st, split_of<T>(ctx, l)));
     CKS(smooth<T>(ctx, l, b, x, ctx->opts.nu2, true));
     return MG_OK;
@@ -721,26 +802,10 @@ mg_status inner_cycles(mg_ctx *ctx, int n) {
             CK(cudaEventCreate(&G->ev[i][0]));
             CK(cudaEventCreate(&G->ev[i][1]));
         }
-        cudaStream_t user = ctx->st;
-        const long k0 = g_launches.load();
-        CK(cudaStreamBeginCapture(ctx->cap, cudaStreamCaptureModeThreadLocal));
-        ctx->st = ctx->cap;
         ctx->capturing = G;
-        const mg_status body = inner_cycles_direct(ctx, n);
+        const mg_status e = capture_graph(ctx, G, [&] { return inner_cycles_direct(ctx, n); });
         ctx->capturing = nullptr;
-        ctx->st = user;
-        cudaGraph_t graph = nullptr;
-        const cudaError_t ee = cudaStreamEndCapture(ctx->cap, &graph);
-        G->kernels = g_launches.load() - k0;
-        g_launches.fetch_sub(G->kernels);  // counted when replayed, not when captured
-        if (body != MG_OK) {
-            if (graph) cudaGraphDestroy(graph);
-            return body;
-        }
-        CK(ee);
-        const cudaError_t ei = cudaGraphInstantiate(&G->exec, graph, 0);
-        cudaGraphDestroy(graph);
-        CK(ei);
+        CKS(e);
     }
     CK(cudaGraphLaunch(G->exec, ctx->st));
     count_launch(G->kernels);
@@ -884,6 +949,10 @@ void mg_free(mg_ctx *ctx) {
         }
         delete G;
     }
+    if (ctx->graph64) {
+        if (ctx->graph64->exec) cudaGraphExecDestroy(ctx->graph64->exec);
+        delete ctx->graph64;
+    }
     if (ctx->cap) cudaStreamDestroy(ctx->cap);
     delete ctx;
 }
@@ -984,6 +1053,7 @@ mg_status mg_setup(const mg_grid *grid, const mg_moduli *moduli, const mg_bc *bc
         cudaError_t e = smoother_init();
         if (e == cudaSuccess) e = plane_init();
         if (e == cudaSuccess) e = small_init();
+        if (e == cudaSuccess) e = strip_init();
         if (e != cudaSuccess) {
             set_err("mg_setup: %s", cudaGetErrorString(e));
             delete ctx;

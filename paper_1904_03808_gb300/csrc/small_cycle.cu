@@ -17,7 +17,8 @@
 //     folded into the right-hand side, then the 4 in-plane colours run on the
 //     plane, so every node sees the neighbour values of the sequential order.
 //     The halos written in a phase are not those read in it;
-//   - one thread a node (or up to kMaxNodes on planes larger than a CTA).
+//   - one thread a node in FP32, one a node component in FP64 (or up to
+//     kMaxNodes of them on planes larger than a CTA).
 // Levels start from x = 0 below the top, so the first phase of their first
 // pre-sweep has no neighbour planes to fold.  Every level's operator, the
 // finest included, is used in its parity-class form (Coarse<T>).
@@ -27,9 +28,8 @@
 // before it -- and at 32^3 the shared-memory loads add to that.  One FP32
 // V-cycle from 32^3 (32^3, 16^3, 8^3 and the 4^3 solve) takes 81 us against
 // about 250 us as 40 launches in a CUDA graph, one from 16^3 29 against
-// 150 us; the FP64 one from 16^3 176 against 780 us (there a warp
-// instruction takes 64 clocks of its scheduler's FP64 pipe, so few SMs cost
-// more: see kSmallNodes64).  Slower forms measured on the way, per cycle
+// 150 us.  FP64 is bound by the pipe besides (kSmallNodes64): the cycle from
+// 16^3 takes 127 us (176 with three components a thread) against 780 us.  Slower forms measured on the way, per cycle
 // from 32^3: neighbour planes read remotely at the start of a phase 89 us,
 // one thread per component with the 116-operation form of the fold 123 us,
 // halos written by the single updates 92 us.
@@ -52,7 +52,7 @@ constexpr int kCta = 16;          // CTAs of the cluster
 // register file divided by what a thread needs
 template <typename T>
 constexpr int small_threads(int nodes) {
-    return sizeof(T) == 8 ? 512 : nodes == 1 ? 1024 : 640;
+    return sizeof(T) == 8 ? (nodes == 1 ? 768 : 512) : nodes == 1 ? 1024 : 640;
 }
 constexpr int kMaxNodes = 4;
 constexpr size_t kSmallSmem = 220 * 1024;
@@ -124,14 +124,58 @@ __device__ __forceinline__ void plane_at(const Coarse<T> &c, const T *P, const N
     coarse_plane_terms(c, u, o);
 }
 
-template <typename T, int NODES>
+// Component a alone of z_row and of plane_at: in FP64 a warp instruction takes
+// 64 clocks of its scheduler however few lanes it has, so three threads a node
+// (one a component) finish a pass over a small plane in a third of the time,
+// for a few repeated sums.  a = 0 and 1 share the code with x and y exchanged
+// (the warps of a component stay together, so the branch on a = 2 is uniform
+// but for one warp).
+template <typename T>
+__device__ __forceinline__ void z_row_c(const Coarse<T> &c, const T *lo, const T *hi,
+                                        const Node &n, int a, T &A, T &U, T &V) {
+    auto S = [&](int x, int b) { const int q = n.r[1] + n.c[x] + b; return hi[q] + lo[q]; };
+    auto D = [&](int x, int b) { const int q = n.r[1] + n.c[x] + b; return hi[q] - lo[q]; };
+    const T s0 = S(1, a), sx = S(0, a) + S(2, a);
+    A = c.cd[a][4] * s0 + c.cd[a][5] * sx;
+    T B = c.cd[a][6] * s0 + c.cd[a][7] * sx, G;
+    if (a == 1) {
+        G = c.g[2][1] * (S(2, 0) - S(0, 0)) + (c.g[0][0] * D(1, 2) + c.g[0][1] * (D(0, 2) + D(2, 2)));
+    } else {
+        const int b = 2 - a;  // the component whose x-difference couples
+        const T d = D(2, b) - D(0, b);
+        A += c.g[1][0] * d;
+        B += c.g[1][1] * d;
+        if (a == 0)
+            G = c.g[2][1] * (S(2, 1) - S(0, 1));
+        else
+            G = c.g[0][0] * D(1, 1) + c.g[0][1] * (D(0, 1) + D(2, 1));
+    }
+    U = B - G;
+    V = B + G;
+}
+template <typename T>
+__device__ __forceinline__ T plane_at_c(const Coarse<T> &c, const T *P, const Node &n, int a) {
+    auto u = [&](int dx, int dy, int b) { return P[n.r[dy + 1] + n.c[dx + 1] + b]; };
+    T o = c.cd[a][1] * (u(-1, 0, a) + u(1, 0, a)) + c.cd[a][2] * (u(0, -1, a) + u(0, 1, a)) +
+          c.cd[a][3] * ((u(-1, -1, a) + u(1, 1, a)) + (u(1, -1, a) + u(-1, 1, a)));
+    if (a < 2) {
+        const int b = 1 - a;
+        o += c.g[2][0] * ((u(1, 1, b) - u(1, -1, b)) - (u(-1, 1, b) - u(-1, -1, b)));
+    }
+    return o;
+}
+
+// COMP: a thread owns one component of its nodes, else all three
+template <typename T, int NODES, bool COMP>
 struct Walker {
+    static constexpr int NC = COMP ? 1 : 3;
     const SmallPlan<T> &g;
     T *sm;
     cg::cluster_group cl;
     int rank, tid, nt;
     Node node[NODES];
-    int act;  // threads that own nodes on the current level (whole warps)
+    int comp[NODES];  // the component owned (COMP), else 0
+    int act;          // threads that own nodes on the current level (whole warps)
 
     // own planes of level l: [first, last)
     __device__ __forceinline__ int first(int l) const {
@@ -172,14 +216,17 @@ struct Walker {
     __device__ __forceinline__ void enter(int l) {
         const SmallLevel &L = g.lev[l];
         const int nh = L.np >> 2;
-        act = L.np < nt ? (L.np + 31) & ~31 : nt;
+        const int own = (3 / NC) * L.np;
+        act = own < nt ? (own + 31) & ~31 : nt;
 #pragma unroll
         for (int u = 0; u < NODES; u++) {
-            const int m = tid + u * nt;
+            const int t = tid + u * nt;
+            comp[u] = COMP && t < own ? fdiv(t, L.mnp) : 0;
+            const int m = t - comp[u] * L.np;
             const int q = fdiv(m, L.mnh), h = m - q * nh, jh = fdiv(h, L.mhx), ih = h - jh * L.hx;
             const int i = 2 * ih + (q & 1), j = 2 * jh + (q >> 1);
             Node &n = node[u];
-            n.colour = m < L.np ? q : -1;
+            n.colour = t < own ? q : -1;
             n.c[0] = col_of(L, i ? i - 1 : L.nx - 1);
             n.c[1] = col_of(L, i);
             n.c[2] = col_of(L, i + 1 < L.nx ? i + 1 : 0);
@@ -191,16 +238,19 @@ struct Walker {
 
     // r = right-hand side of plane k minus the dz = +-1 terms, at own nodes
     __device__ __forceinline__ void fold(const Coarse<T> &c, const T *b, const T *lo, const T *hi,
-                                         T (&r)[NODES][3]) const {
+                                         T (&r)[NODES][NC]) const {
         T *U = sm + g.scratch, *V = U + g.plmax;
 #pragma unroll
         for (int u = 0; u < NODES; u++) {
             if (node[u].colour < 0) continue;
-            T up[3], vp[3];
-            z_row(c, lo, hi, node[u], r[u], up, vp);
-            const int o = node[u].r[1] + node[u].c[1];
+            T up[NC], vp[NC];
+            if constexpr (COMP)
+                z_row_c(c, lo, hi, node[u], comp[u], r[u][0], up[0], vp[0]);
+            else
+                z_row(c, lo, hi, node[u], r[u], up, vp);
+            const int o = node[u].r[1] + node[u].c[1] + comp[u];
 #pragma unroll
-            for (int a = 0; a < 3; a++) {
+            for (int a = 0; a < NC; a++) {
                 U[o + a] = up[a];
                 V[o + a] = vp[a];
                 r[u][a] = b[o + a] - r[u][a];
@@ -210,10 +260,19 @@ struct Walker {
 #pragma unroll
         for (int u = 0; u < NODES; u++) {
             if (node[u].colour < 0) continue;
-            const int om = node[u].r[0] + node[u].c[1], op = node[u].r[2] + node[u].c[1];
+            const int om = node[u].r[0] + node[u].c[1] + comp[u],
+                      op = node[u].r[2] + node[u].c[1] + comp[u];
 #pragma unroll
-            for (int a = 0; a < 3; a++) r[u][a] -= U[om + a] + V[op + a];
+            for (int a = 0; a < NC; a++) r[u][a] -= U[om + a] + V[op + a];
         }
+    }
+    // the in-plane terms at own node u
+    __device__ __forceinline__ void in_plane(const Coarse<T> &c, const T *P, int u,
+                                             T (&o)[NC]) const {
+        if constexpr (COMP)
+            o[0] = plane_at_c(c, P, node[u], comp[u]);
+        else
+            plane_at(c, P, node[u], o);
     }
 
     // n sweeps on the level entered; zero: its x is still zero everywhere
@@ -229,7 +288,7 @@ struct Walker {
             if (tid < act)
 #pragma unroll 1
                 for (int q = (k0 ^ par) & 1; q < nk; q += 2) {
-                    T r[NODES][3];
+                    T r[NODES][NC];
                     T *const P = X0 + q * pl;
                     T *const h0 = q == 0 ? below : nullptr, *const h1 = q == ppc - 1 ? above : nullptr;
                     const T *b = B0 + q * pl;
@@ -237,10 +296,10 @@ struct Walker {
 #pragma unroll
                         for (int u = 0; u < NODES; u++)
 #pragma unroll
-                            for (int a = 0; a < 3; a++)
+                            for (int a = 0; a < NC; a++)
                                 r[u][a] = node[u].colour < 0
                                               ? T(0)
-                                              : b[node[u].r[1] + node[u].c[1] + a];
+                                              : b[node[u].r[1] + node[u].c[1] + comp[u] + a];
                     } else {
                         fold(c, b, P - pl, P + pl, r);
                     }
@@ -252,14 +311,12 @@ struct Walker {
 #pragma unroll
                         for (int u = 0; u < NODES; u++) {
                             if (node[u].colour != colour) continue;
-                            T o[3];
-                            plane_at(c, P, node[u], o);
-                            const int e = node[u].r[1] + node[u].c[1];
+                            T o[NC];
+                            in_plane(c, P, u, o);
+                            const int e = node[u].r[1] + node[u].c[1] + comp[u];
 #pragma unroll
-                            for (int a = 0; a < 3; a++) {
-                                o[a] = c.dinv[a] * (r[u][a] - o[a]);
-                                P[e + a] = o[a];
-                            }
+                            for (int a = 0; a < NC; a++)
+                                P[e + a] = c.dinv[comp[u] + a] * (r[u][a] - o[a]);
                         }
                     }
                     // 16 bytes at a time: the scattered stores of the single
@@ -289,19 +346,19 @@ struct Walker {
         if (tid < act)
 #pragma unroll 1
             for (int k = k0; k < k1; k++) {
-                T r[NODES][3];
+                T r[NODES][NC];
                 const T *P = own(l, L.x, k);
                 fold(c, own(l, L.b, k), P - L.pl, P + L.pl, r);
                 sync_act();
 #pragma unroll
                 for (int u = 0; u < NODES; u++) {
                     if (node[u].colour < 0) continue;
-                    T o[3];
-                    plane_at(c, P, node[u], o);
-                    const int q = node[u].r[1] + node[u].c[1];
+                    T o[NC];
+                    in_plane(c, P, u, o);
+                    const int q = node[u].r[1] + node[u].c[1] + comp[u];
 #pragma unroll
-                    for (int a = 0; a < 3; a++)
-                        R[q + a] = r[u][a] - (o[a] + c.cd[a][0] * P[q + a]);
+                    for (int a = 0; a < NC; a++)
+                        R[q + a] = r[u][a] - (o[a] + c.cd[comp[u] + a][0] * P[q + a]);
                 }
                 sync_act();
                 // x and y parts of the full weighting
@@ -430,8 +487,9 @@ __global__ void __launch_bounds__(small_threads<T>(NODES), 1)
     k_small_cycle(const __grid_constant__ SmallPlan<T> g, const T *__restrict__ b, T *x,
                   int from_zero, int cycles) {
     extern __shared__ __align__(16) unsigned char smem_small[];
-    Walker<T, NODES> w{g, reinterpret_cast<T *>(smem_small), cg::this_cluster(),
-                       (int)cg::this_cluster().block_rank(), (int)threadIdx.x, (int)blockDim.x};
+    Walker<T, NODES, sizeof(T) == 8> w{g, reinterpret_cast<T *>(smem_small), cg::this_cluster(),
+                                       (int)cg::this_cluster().block_rank(), (int)threadIdx.x,
+                                       (int)blockDim.x};
     const SmallLevel &L = g.lev[0];
     const long ps = L.np, cs = (long)(L.nz + 1) * ps;
     const int n3 = 3 * L.np, k0 = w.first(0), k1 = w.last(0);
@@ -564,7 +622,7 @@ bool small_plan(const Dims *d, const Coarse<T> *op, int nlev, int ncoarse, const
     // with the bank-conflict-free row pitch if that fits, else packed rows
     if (!small_layout(d, op, nlev, true, g) && !small_layout(d, op, nlev, false, g)) return false;
     // one thread a node where the CTA can be that large, else up to kMaxNodes
-    const int np = g.lev[0].np;
+    const int np = g.lev[0].np * (sizeof(T) == 8 ? 3 : 1);  // FP64: a thread a component
     g.nodes = np <= small_threads<T>(1) ? 1 : kMaxNodes;
     const int per = (np + g.nodes - 1) / g.nodes;
     g.threads = per < 128 ? 128 : (per + 31) / 32 * 32;
