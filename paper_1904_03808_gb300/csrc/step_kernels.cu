@@ -26,6 +26,29 @@ __device__ __forceinline__ bool cell_ijk(int nx, int ny, int &i, int &j, int &k)
     return i < nx && j < ny;
 }
 
+// Launch of a kernel that marches columns in z: blocks of `threads` over the
+// columns of a plane in linear order (the FP64 pipe is paid for by the warp
+// instruction, so lanes are packed whatever nx is), grid.y over chunks of
+// `chunk` planes.  A chunk repeats one plane's partial sums, so chunks are as
+// long as leaves the chip about four blocks an SM; then blocks shrink.
+struct March {
+    dim3 grid;
+    int threads, chunk;
+};
+inline March march(long columns, int planes) {
+    March m;
+    m.threads = 128;
+    m.chunk = 16;
+    auto blocks = [&] {
+        return ((columns + m.threads - 1) / m.threads) * ((planes + m.chunk - 1) / m.chunk);
+    };
+    while (m.chunk > 1 && blocks() < 608) m.chunk /= 2;
+    while (m.threads > 32 && blocks() < 608) m.threads /= 2;
+    m.grid = dim3((unsigned)((columns + m.threads - 1) / m.threads),
+                  (planes + m.chunk - 1) / m.chunk);
+    return m;
+}
+
 struct StzConst {
     double half_eDT_over_tau0;  // exp(-Delta/(kB T)) / (2 tau0)
     double beta;                // Omega eps0 / (kB T)
@@ -41,25 +64,57 @@ __host__ StzConst stz_const(const StepParams &p) {
     return c;
 }
 
+// exp(x + y) + exp(y - x), x > 0.  FP64 runs at 1/64 of the FP32 rate, and for
+// x > 12.5 the second term is below exp(-25) = 1.4e-11 of the first: there its
+// ratio r = exp(-2 x) in FP32 (relative error 4e-6 at most: the rounding of
+// 2 x <= 87, expf's own) changes the sum by less than 2^-54.
+__device__ __forceinline__ double exp_pair(double x, double y) {
+    const double ep = exp(x + y);
+    const float x2 = -2.0f * (float)x;
+    if (x2 < -25.0f) {
+        const float r = expf(x2);
+        return r > 0.0f ? fma(ep, (double)r, ep) : ep;  // (no inf * 0)
+    }
+    return ep + exp(y - x);
+}
+
 // athermal STZ rate magnitude, Eqs. (20)-(22):
 //   D = exp(-e_z/(kB chi)) exp(-Delta/(kB T)) cosh(Omega eps0 sbar/(kB T)) (1 - s_Y/sbar) / tau0,
-// 0 at or below yield (or for chi <= 0).  FP64 is slow on this part, so the
-// product exp(-e_z/chi) cosh(beta sbar) is taken as
-// (exp(beta sbar - e_z/chi) + exp(-beta sbar - e_z/chi)) / 2 (two exponentials,
-// no reciprocal) and 1/sbar is computed once by the caller.
+// 0 at or below yield (or for chi <= 0).  The product exp(-e_z/chi) cosh(beta
+// sbar) is taken as (exp(beta sbar - e_z/chi) + exp(-beta sbar - e_z/chi)) / 2
+// and 1/sbar is computed once by the caller.
 __device__ __forceinline__ double stz_rate(const StzConst &c, double sbar, double inv_sbar,
                                            double chi) {
     if (!(sbar > c.sY) || !(chi > 0.0)) return 0.0;
     const double y = -c.ez_K / chi, x = c.beta * sbar;
-    return (exp(x + y) + exp(y - x)) * c.half_eDT_over_tau0 * (1.0 - c.sY * inv_sbar);
+    return exp_pair(x, y) * c.half_eDT_over_tau0 * (1.0 - c.sY * inv_sbar);
+}
+
+// 1/2 sigma0 : sigma0, given the mean stress m
+__device__ __forceinline__ double j2_of(const double s[6], double m) {
+    const double d0 = s[0] - m, d1 = s[1] - m, d2 = s[2] - m;
+    return 0.5 * (d0 * d0 + d1 * d1 + d2 * d2) + (s[3] * s[3] + s[4] * s[4] + s[5] * s[5]);
+}
+
+// sbar = sqrt(q) and its reciprocal (0 for q = 0) from the reciprocal square
+// root, each corrected once to the accuracy of the square root and the
+// division, which take about twice the FP64 instructions
+__device__ __forceinline__ void sbar_inv(double q, double &sb, double &inv) {
+    const int hi = __double2hiint(q);
+    if (hi >= 0x00100000 && hi < 0x7ff00000) {  // positive, normal and finite
+        inv = rsqrt(q);
+        sb = q * inv;
+        sb = fma(fma(-sb, sb, q), 0.5 * inv, sb);
+        inv = fma(fma(-sb, inv, 1.0), inv, inv);
+    } else {
+        sb = sqrt(q);
+        inv = sb > 0.0 ? 1.0 / sb : 0.0;
+    }
 }
 
 // sbar with sbar^2 = 1/2 sigma0 : sigma0
 __device__ __forceinline__ double sbar_of(const double s[6]) {
-    const double m = (s[0] + s[1] + s[2]) * (1.0 / 3.0);
-    const double d0 = s[0] - m, d1 = s[1] - m, d2 = s[2] - m;
-    const double q = d0 * d0 + d1 * d1 + d2 * d2 + 2.0 * (s[3] * s[3] + s[4] * s[4] + s[5] * s[5]);
-    return sqrt(0.5 * q);
+    return sqrt(j2_of(s, (s[0] + s[1] + s[2]) * (1.0 / 3.0)));
 }
 
 // Eq. (31): G[a][b] = d v_a / d x_b at the centre of cell (i, j, k), from its
@@ -67,9 +122,9 @@ __device__ __forceinline__ double sbar_of(const double s[6]) {
 // Computed for a column of cells marching up in z: each corner plane's
 // contributions -- x-differences, y-differences and the sum over the 2 x 2
 // corners around the column -- are formed once and shared by the cells
-// below and above the plane (45 FP64 operations a cell instead of 72).
-constexpr int kCellChunk = 16;  // cells of one column per thread
-
+// below and above the plane.  The x- and y-differences come from the two
+// diagonals (their sum and difference): 39 FP64 operations a cell with the
+// scaling, instead of 72.
 struct GradPlane {
     double X[3], Y[3], Z[3];
 };
@@ -81,8 +136,9 @@ __device__ __forceinline__ GradPlane grad_plane(const double *__restrict__ v, lo
     for (int a = 0; a < 3; a++) {
         const double *g = v + a * cs + off;
         const double c00 = g[r0 + i], c10 = g[r0 + i1], c01 = g[r1 + i], c11 = g[r1 + i1];
-        P.X[a] = (c10 - c00) + (c11 - c01);
-        P.Y[a] = (c01 - c00) + (c11 - c10);
+        const double d1 = c11 - c00, d2 = c10 - c01;
+        P.X[a] = d1 + d2;
+        P.Y[a] = d1 - d2;
         P.Z[a] = (c00 + c10) + (c01 + c11);
     }
     return P;
@@ -99,19 +155,20 @@ __device__ __forceinline__ void grad_cell(const GradPlane &lo, const GradPlane &
     }
 }
 
-// column (i, j) of a chunk of kCellChunk cells; false if outside the grid
+// column (i, j) of a chunk of cells; false if outside the grid
 struct CellColumn {
     int i, j, i1, k0, k1;
     long pl, cs, r0, r1;
 };
-__device__ __forceinline__ bool cell_column(int nx, int ny, int nz, CellColumn &C) {
-    C.i = blockIdx.x * BX + threadIdx.x;
-    C.j = blockIdx.y * BY + threadIdx.y;
-    if (C.i >= nx || C.j >= ny) return false;
+__device__ __forceinline__ bool cell_column(int nx, int ny, int nz, int chunk, CellColumn &C) {
+    const int m = blockIdx.x * blockDim.x + threadIdx.x;
+    C.j = m / nx;
+    C.i = m - C.j * nx;
+    if (C.j >= ny) return false;
     C.i1 = C.i + 1 < nx ? C.i + 1 : 0;
     const int j1 = C.j + 1 < ny ? C.j + 1 : 0;
-    C.k0 = blockIdx.z * kCellChunk;
-    C.k1 = C.k0 + kCellChunk < nz ? C.k0 + kCellChunk : nz;
+    C.k0 = blockIdx.y * chunk;
+    C.k1 = C.k0 + chunk < nz ? C.k0 + chunk : nz;
     C.pl = (long)nx * ny;
     C.cs = (long)(nz + 1) * C.pl;
     C.r0 = (long)C.j * nx;
@@ -119,69 +176,95 @@ __device__ __forceinline__ bool cell_column(int nx, int ny, int nz, CellColumn &
     return true;
 }
 
+// constants of the predictor and the corrector: G of a cell enters both only
+// as dt G, so the scale of the gradient carries the time step
+struct CellConst {
+    double dt4h;     // dt / (4 h)
+    double lam, mu, mu2, mu2dt;
+};
+CellConst cell_const(const StepParams &p) {
+    return CellConst{p.dt * (0.25 / p.h), p.lam, p.mu, 2.0 * p.mu, 2.0 * p.mu * p.dt};
+}
+
 // Eq. (27) at cell q: sigma* = sigma + dt (L sigma + sigma L^T - tr(L) sigma
-// - 2 mu D^pl sigma0 / sbar) from the cell-centre gradient G of v^n and the
-// cell's sigma^n (s6) and chi^n; also stores D^pl and sbar
-__device__ __forceinline__ void predict_cell(const StepParams &p, const StzConst &c,
+// - 2 mu D^pl sigma0 / sbar) from dt times the cell-centre gradient of v^n (G)
+// and the cell's sigma^n (s6) and chi^n; also stores D^pl and sbar.  With
+// P = 2 mu dt D^pl / sbar and H = dt L - (tr(dt L) + P) / 2 I the update is
+// sigma + (H sigma + sigma H^T + P m I), m the mean stress: 49 instructions
+// where the terms one by one take 68.  The increment is summed before it is
+// added to sigma, which rounds the result once.
+__device__ __forceinline__ void predict_cell(const CellConst &w, const StzConst &c,
                                              const double (&G)[3][3], const double (&s6)[6],
                                              double chi_q, long q, long nc,
                                              double *__restrict__ sig_star,
                                              double *__restrict__ dpl,
                                              double *__restrict__ sbar_out) {
-    // full symmetric matrix
     const double S[3][3] = {{s6[0], s6[5], s6[4]}, {s6[5], s6[1], s6[3]}, {s6[4], s6[3], s6[2]}};
-    const double sb = sbar_of(s6);
-    const double inv_sb = sb > 0.0 ? 1.0 / sb : 0.0;
-    const double D = stz_rate(c, sb, inv_sb, chi_q);
-    const double trL = G[0][0] + G[1][1] + G[2][2];
     const double m = (s6[0] + s6[1] + s6[2]) * (1.0 / 3.0);
-    const double pl = (D > 0.0) ? 2.0 * p.mu * D * inv_sb : 0.0;
-    // (a, b) pairs of the 6 stored components
-    const int ia[6] = {0, 1, 2, 1, 0, 0}, ib[6] = {0, 1, 2, 2, 2, 1};
+    double sb, inv_sb;
+    sbar_inv(j2_of(s6, m), sb, inv_sb);
+    const double D = stz_rate(c, sb, inv_sb, chi_q);
+    const double P = w.mu2dt * D * inv_sb;
+    const double tr = 0.5 * (G[0][0] + G[1][1] + G[2][2] + P);
+    double H[3][3];
 #pragma unroll
-    for (int n = 0; n < 6; n++) {
+    for (int a = 0; a < 3; a++)
+#pragma unroll
+        for (int b = 0; b < 3; b++) H[a][b] = a == b ? G[a][b] - tr : G[a][b];
+#pragma unroll
+    for (int a = 0; a < 3; a++) {
+        double t = H[a][0] * S[0][a];
+        t = fma(H[a][1], S[1][a], t);
+        t = fma(H[a][2], S[2][a], t);
+        sig_star[a * nc + q] = S[a][a] + fma(2.0, t, P * m);
+    }
+    const int ia[3] = {1, 0, 0}, ib[3] = {2, 2, 1};
+#pragma unroll
+    for (int n = 0; n < 3; n++) {
         const int a = ia[n], b = ib[n];
-        double rate = -trL * S[a][b];
+        double t = H[a][0] * S[0][b];
 #pragma unroll
-        for (int e = 0; e < 3; e++) rate += G[a][e] * S[e][b] + S[a][e] * G[b][e];
-        rate -= pl * (S[a][b] - (a == b ? m : 0.0));
-        sig_star[n * nc + q] = S[a][b] + p.dt * rate;
+        for (int e = 0; e < 3; e++) {
+            if (e > 0) t = fma(H[a][e], S[e][b], t);
+            t = fma(S[a][e], H[b][e], t);
+        }
+        sig_star[(3 + n) * nc + q] = S[a][b] + t;
     }
     dpl[q] = D;
     sbar_out[q] = sb;
 }
 
 // Eq. (29) at one cell: sigma = sigma* + dt (lam tr(D) I + 2 mu D), D = sym G
-__device__ __forceinline__ void correct_cell(const StepParams &p, const double (&G)[3][3],
+// (G: dt times the gradient)
+__device__ __forceinline__ void correct_cell(const CellConst &w, const double (&G)[3][3],
                                              const double (&ss)[6], double (&s6)[6]) {
-    const double tr = G[0][0] + G[1][1] + G[2][2];
-    const double dt = p.dt, lam = p.lam, mu = p.mu;
-    s6[0] = ss[0] + dt * (lam * tr + 2.0 * mu * G[0][0]);
-    s6[1] = ss[1] + dt * (lam * tr + 2.0 * mu * G[1][1]);
-    s6[2] = ss[2] + dt * (lam * tr + 2.0 * mu * G[2][2]);
-    s6[3] = ss[3] + dt * mu * (G[1][2] + G[2][1]);
-    s6[4] = ss[4] + dt * mu * (G[0][2] + G[2][0]);
-    s6[5] = ss[5] + dt * mu * (G[0][1] + G[1][0]);
+    const double lt = w.lam * (G[0][0] + G[1][1] + G[2][2]);
+#pragma unroll
+    for (int a = 0; a < 3; a++) s6[a] = fma(w.mu2, G[a][a], ss[a] + lt);
+    s6[3] = fma(w.mu, G[1][2] + G[2][1], ss[3]);
+    s6[4] = fma(w.mu, G[0][2] + G[2][0], ss[4]);
+    s6[5] = fma(w.mu, G[0][1] + G[1][0], ss[5]);
 }
 
 // Eq. (27) over a column chunk of cells
-__global__ void k_stress_predict(StepParams p, StzConst c, const double *__restrict__ v,
-                                 const double *__restrict__ sig, const double *__restrict__ chi,
-                                 double *__restrict__ sig_star, double *__restrict__ dpl,
-                                 double *__restrict__ sbar_out, long nc) {
+__global__ void __launch_bounds__(128)
+    k_stress_predict(StepParams p, CellConst w, StzConst c, int chunk, const double *__restrict__ v,
+                     const double *__restrict__ sig, const double *__restrict__ chi,
+                     double *__restrict__ sig_star, double *__restrict__ dpl,
+                     double *__restrict__ sbar_out, long nc) {
     CellColumn C;
-    if (!cell_column(p.nx, p.ny, p.nz, C)) return;
+    if (!cell_column(p.nx, p.ny, p.nz, chunk, C)) return;
     GradPlane lo = grad_plane(v, C.cs, C.k0 * C.pl, C.r0, C.r1, C.i, C.i1);
     for (int k = C.k0; k < C.k1; k++) {
         const GradPlane hi = grad_plane(v, C.cs, (k + 1) * C.pl, C.r0, C.r1, C.i, C.i1);
         const long q = k * C.pl + C.r0 + C.i;
         double G[3][3];
-        grad_cell(lo, hi, 0.25 / p.h, G);
+        grad_cell(lo, hi, w.dt4h, G);
         lo = hi;
         double s6[6];
 #pragma unroll
         for (int a = 0; a < 6; a++) s6[a] = sig[a * nc + q];
-        predict_cell(p, c, G, s6, chi[q], q, nc, sig_star, dpl, sbar_out);
+        predict_cell(w, c, G, s6, chi[q], q, nc, sig_star, dpl, sbar_out);
     }
 }
 
@@ -189,119 +272,159 @@ __global__ void k_stress_predict(StepParams p, StzConst c, const double *__restr
 // diffusion: sum over the 6 faces of (D_P + D_N)/2 (chi_N - chi_P) / h^2;
 // z ghost cells carry linearly extrapolated sigma and chi, and their D is
 // the STZ rate of those extrapolated values
-__global__ void k_chi_update(StepParams p, StzConst c, const double *__restrict__ sig,
-                             const double *__restrict__ chi, const double *__restrict__ dpl,
-                             const double *__restrict__ sbar, double *__restrict__ chi_new,
-                             long nc) {
-    const int nx = p.nx, ny = p.ny, nz = p.nz;
-    int i, j, k;
-    if (!cell_ijk(nx, ny, i, j, k)) return;
-    const long q = ((long)k * ny + j) * nx + i;
-    const long pl = (long)nx * ny;
-    const int ip = (i + 1 < nx) ? i + 1 : 0, im = i ? i - 1 : nx - 1;
-    const int jp = (j + 1 < ny) ? j + 1 : 0, jm = j ? j - 1 : ny - 1;
-    const long base = (long)k * pl + (long)j * nx;
-    const double c0 = chi[q], D0 = dpl[q];
-    double acc = 0.0;
-    long nb[4] = {base + ip, base + im, (long)k * pl + (long)jp * nx + i,
-                  (long)k * pl + (long)jm * nx + i};
+// A thread marches a column in z: a z face's flux serves the cells below and
+// above it.  The products of constants are formed on the host -- three FP64
+// divisions a cell were half of this kernel.
+struct ChiConst {
+    double grow, diff;  // 2 dt / (c0 s_Y);  dt l^2 / (2 c0 h^2)
+    double chi_inf;
+};
+__global__ void __launch_bounds__(128)
+    k_chi_update(StepParams p, StzConst c, ChiConst w, int chunk, const double *__restrict__ sig,
+                 const double *__restrict__ chi, const double *__restrict__ dpl,
+                 const double *__restrict__ sbar, double *__restrict__ chi_new, long nc) {
+    CellColumn C;
+    if (!cell_column(p.nx, p.ny, p.nz, chunk, C)) return;
+    const int nz = p.nz;
+    const long pl = C.pl;
+    const long rm = (long)(C.j ? C.j - 1 : p.ny - 1) * p.nx + C.i, rp = C.r1 + C.i;
+    const long xm = C.r0 + (C.i ? C.i - 1 : p.nx - 1), xp = C.r0 + C.i1;
+    // (D_P + D_N) (chi_N - chi_P) of the z face on side +-1 of a wall cell q:
+    // the ghost's values are 2 * (this layer) - (next layer inward)
+    auto wall_flux = [&](long q, long in, double cP, double DP) {
+        double s6[6];
 #pragma unroll
-    for (int n = 0; n < 4; n++) acc += 0.5 * (D0 + dpl[nb[n]]) * (chi[nb[n]] - c0);
-    // z neighbours, with ghosts at the walls
-#pragma unroll
-    for (int side = 0; side < 2; side++) {
-        const int kn = side ? k + 1 : k - 1;
-        double cn, Dn;
-        if (kn >= 0 && kn < nz) {
-            cn = chi[q + (side ? pl : -pl)];
-            Dn = dpl[q + (side ? pl : -pl)];
+        for (int a = 0; a < 6; a++) s6[a] = 2.0 * sig[a * nc + q] - sig[a * nc + q + in];
+        const double cn = 2.0 * cP - chi[q + in], sbn = sbar_of(s6);
+        return (DP + stz_rate(c, sbn, sbn > 0.0 ? 1.0 / sbn : 0.0, cn)) * (cn - cP);
+    };
+    long q = C.k0 * pl + C.r0 + C.i;
+    double c0 = chi[q], D0 = dpl[q];
+    // flux across the face below the current cell, from the cell below
+    double below = C.k0 == 0 ? -wall_flux(q, pl, c0, D0)
+                             : (D0 + dpl[q - pl]) * (c0 - chi[q - pl]);
+    for (int k = C.k0; k < C.k1; k++, q += pl) {
+        const long kp = k * pl;
+        double above, c1 = 0.0, D1 = 0.0;
+        if (k + 1 < nz) {
+            c1 = chi[q + pl];
+            D1 = dpl[q + pl];
+            above = (D0 + D1) * (c1 - c0);
         } else {
-            // ghost: 2 * (this layer) - (next layer inward)
-            const long q1 = q + (side ? -pl : pl);
-            double s6[6];
-#pragma unroll
-            for (int a = 0; a < 6; a++) s6[a] = 2.0 * sig[a * nc + q] - sig[a * nc + q1];
-            cn = 2.0 * c0 - chi[q1];
-            const double sbn = sbar_of(s6);
-            Dn = stz_rate(c, sbn, sbn > 0.0 ? 1.0 / sbn : 0.0, cn);
+            above = wall_flux(q, -pl, c0, D0);
         }
-        acc += 0.5 * (D0 + Dn) * (cn - c0);
+        double acc = above - below;
+        const long nb[4] = {xp, xm, rp, rm};
+#pragma unroll
+        for (int n = 0; n < 4; n++) acc = fma(D0 + dpl[kp + nb[n]], chi[kp + nb[n]] - c0, acc);
+        const double growth = D0 * sbar[q] * (w.chi_inf - c0);
+        chi_new[q] = c0 + fma(w.grow, growth, w.diff * acc);
+        below = above;
+        c0 = c1;
+        D0 = D1;
     }
-    const double growth = 2.0 * D0 * sbar[q] / p.sY * (p.chi_inf - c0);
-    chi_new[q] = c0 + p.dt / p.c0 * (growth + (p.l * p.l) / (p.h * p.h) * acc);
 }
 
 // b = (h^2/(mu dt)) div sigma* at interior corners; the corner derivative is
-// Eq. (31) shifted by half a cell: cells (i-1..i, j-1..j, k-1..k)
-// corner divergence, marching up one (i, j) corner column over kDivChunk
-// corner planes: each cell layer's contributions -- x-differences of
-// sigma_a0, y-differences of sigma_a1 and the layer sum of sigma_a2 over the
-// 2 x 2 cells around the column -- are formed once and shared by the corners
-// below and above the layer (FP64 is add-bound here: about 42 adds a corner
-// instead of 72)
-constexpr int kDivChunk = 16;
-
+// Eq. (31) shifted by half a cell: cells (i-1..i, j-1..j, k-1..k).
+// Corner divergence, marching up one (i, j) corner column: each cell layer's
+// contributions -- the x-differences of sigma_a0 plus the y-differences of
+// sigma_a1, and the layer sum of sigma_a2 over the 2 x 2 cells around the
+// column -- are formed once and shared by the corners below and above the
+// layer (FP64 is add-bound here: 40 instructions a corner instead of 72)
 struct DivLayer {
-    double X[3], Y[3], Z[3];
+    double XY[3], Z[3];
 };
+
+// over the 2 x 2 cells f[y][x]
+__device__ __forceinline__ double sum4(const double (&f)[2][2]) {
+    return (f[0][0] + f[0][1]) + (f[1][0] + f[1][1]);
+}
+__device__ __forceinline__ double dif_x(const double (&f)[2][2]) {
+    return (f[0][1] - f[0][0]) + (f[1][1] - f[1][0]);
+}
+__device__ __forceinline__ double dif_y(const double (&f)[2][2]) {
+    return (f[1][0] - f[0][0]) + (f[1][1] - f[0][1]);
+}
 
 __device__ __forceinline__ DivLayer div_layer(const double *__restrict__ ss, long nc, long base,
                                               long rj0, long rj1, int im, int i) {
-    // stored component of sigma_ab: xx, yy, zz, yz, xz, xy
-    const int comp[3][3] = {{0, 5, 4}, {5, 1, 3}, {4, 3, 2}};
+    auto cells = [&](int n, double (&f)[2][2]) {
+        const double *g = ss + n * nc + base;
+        f[0][0] = g[rj0 + im];
+        f[0][1] = g[rj0 + i];
+        f[1][0] = g[rj1 + im];
+        f[1][1] = g[rj1 + i];
+    };
     DivLayer L;
-#pragma unroll
-    for (int a = 0; a < 3; a++) {
-        const double *fx = ss + comp[a][0] * nc + base, *fy = ss + comp[a][1] * nc + base,
-                     *fz = ss + comp[a][2] * nc + base;
-        L.X[a] = (fx[rj0 + i] - fx[rj0 + im]) + (fx[rj1 + i] - fx[rj1 + im]);
-        L.Y[a] = (fy[rj1 + im] - fy[rj0 + im]) + (fy[rj1 + i] - fy[rj0 + i]);
-        L.Z[a] = (fz[rj0 + im] + fz[rj0 + i]) + (fz[rj1 + im] + fz[rj1 + i]);
-    }
+    double f[2][2];
+    cells(5, f);  // xy: its x- and y-differences from the two diagonals
+    const double d1 = f[1][1] - f[0][0], d2 = f[0][1] - f[1][0];
+    L.XY[1] = d1 + d2;
+    L.XY[0] = d1 - d2;
+    cells(0, f);
+    L.XY[0] += dif_x(f);
+    cells(1, f);
+    L.XY[1] += dif_y(f);
+    cells(4, f);
+    L.XY[2] = dif_x(f);
+    L.Z[0] = sum4(f);
+    cells(3, f);
+    L.XY[2] += dif_y(f);
+    L.Z[1] = sum4(f);
+    cells(2, f);
+    L.Z[2] = sum4(f);
     return L;
 }
 
-__global__ void k_div_rhs(StepParams p, const double *__restrict__ ss, double *__restrict__ b,
-                          double scale) {
+// (its wall planes, not part of the system, are zeroed)
+__global__ void __launch_bounds__(128)
+    k_div_rhs(StepParams p, int chunk, const double *__restrict__ ss, double *__restrict__ b,
+              double scale) {
     const int nx = p.nx, ny = p.ny, nz = p.nz;
-    const int i = blockIdx.x * BX + threadIdx.x, j = blockIdx.y * BY + threadIdx.y;
-    if (i >= nx || j >= ny) return;
-    const int k0 = 1 + blockIdx.z * kDivChunk;
-    const int k1 = k0 + kDivChunk < nz ? k0 + kDivChunk : nz;  // corners k0 .. k1-1
+    const int m = blockIdx.x * blockDim.x + threadIdx.x, j = m / nx, i = m - j * nx;
+    if (j >= ny) return;
+    const int k0 = 1 + blockIdx.y * chunk;
+    const int k1 = k0 + chunk < nz ? k0 + chunk : nz;  // corners k0 .. k1-1
     const int im = i ? i - 1 : nx - 1, jm = j ? j - 1 : ny - 1;
     const long nc = (long)nx * ny * nz, pl = (long)nx * ny;
     const long rj0 = (long)jm * nx, rj1 = (long)j * nx;
     const long cs = (long)(nz + 1) * pl;
+#pragma unroll
+    for (int a = 0; a < 3; a++) {
+        if (k0 == 1) b[a * cs + m] = 0.0;
+        if (k1 == nz) b[a * cs + nz * pl + m] = 0.0;
+    }
     DivLayer lo = div_layer(ss, nc, (long)(k0 - 1) * pl, rj0, rj1, im, i);
     for (int k = k0; k < k1; k++) {
         const DivLayer hi = div_layer(ss, nc, (long)k * pl, rj0, rj1, im, i);
-        const long node = (long)k * pl + (long)j * nx + i;
+        const long node = (long)k * pl + m;
 #pragma unroll
         for (int a = 0; a < 3; a++)
-            b[a * cs + node] = scale * ((lo.X[a] + hi.X[a]) + (lo.Y[a] + hi.Y[a]) + (hi.Z[a] - lo.Z[a]));
+            b[a * cs + node] = scale * ((lo.XY[a] + hi.XY[a]) + (hi.Z[a] - lo.Z[a]));
         lo = hi;
     }
 }
 
 // Eq. (29) over a column chunk of cells; chi_dst <- chi_src on the way
 // (the step's new chi, when chi_dst is not null)
-__global__ void k_stress_correct(StepParams p, const double *__restrict__ v,
-                                 const double *__restrict__ ss, double *__restrict__ sig,
-                                 const double *__restrict__ chi_src, double *__restrict__ chi_dst,
-                                 long nc) {
+__global__ void __launch_bounds__(128)
+    k_stress_correct(StepParams p, CellConst w, int chunk, const double *__restrict__ v,
+                     const double *__restrict__ ss, double *__restrict__ sig,
+                     const double *__restrict__ chi_src, double *__restrict__ chi_dst, long nc) {
     CellColumn C;
-    if (!cell_column(p.nx, p.ny, p.nz, C)) return;
+    if (!cell_column(p.nx, p.ny, p.nz, chunk, C)) return;
     GradPlane lo = grad_plane(v, C.cs, C.k0 * C.pl, C.r0, C.r1, C.i, C.i1);
     for (int k = C.k0; k < C.k1; k++) {
         const GradPlane hi = grad_plane(v, C.cs, (k + 1) * C.pl, C.r0, C.r1, C.i, C.i1);
         const long q = k * C.pl + C.r0 + C.i;
         double G[3][3];
-        grad_cell(lo, hi, 0.25 / p.h, G);
+        grad_cell(lo, hi, w.dt4h, G);
         lo = hi;
         double s6[6], ss6[6];
 #pragma unroll
         for (int a = 0; a < 6; a++) ss6[a] = ss[a * nc + q];
-        correct_cell(p, G, ss6, s6);
+        correct_cell(w, G, ss6, s6);
 #pragma unroll
         for (int a = 0; a < 6; a++) sig[a * nc + q] = s6[a];
         if (chi_dst) chi_dst[q] = chi_src[q];
@@ -314,29 +437,30 @@ __global__ void k_stress_correct(StepParams p, const double *__restrict__ v,
 // through memory.  sig_star holds sigma* of step n on entry and of step n+1
 // on return (each cell reads and writes only its own entries); sig receives
 // sigma^{n+1}, chi_dst the step's new chi (chi_src).
-__global__ void k_correct_predict(StepParams p, StzConst c, const double *__restrict__ v,
-                                  double *__restrict__ sig_star, double *__restrict__ sig,
-                                  const double *__restrict__ chi_src,
-                                  double *__restrict__ chi_dst, double *__restrict__ dpl,
-                                  double *__restrict__ sbar_out, long nc) {
+__global__ void __launch_bounds__(128)
+    k_correct_predict(StepParams p, CellConst w, StzConst c, int chunk,
+                      const double *__restrict__ v, double *__restrict__ sig_star,
+                      double *__restrict__ sig, const double *__restrict__ chi_src,
+                      double *__restrict__ chi_dst, double *__restrict__ dpl,
+                      double *__restrict__ sbar_out, long nc) {
     CellColumn C;
-    if (!cell_column(p.nx, p.ny, p.nz, C)) return;
+    if (!cell_column(p.nx, p.ny, p.nz, chunk, C)) return;
     GradPlane lo = grad_plane(v, C.cs, C.k0 * C.pl, C.r0, C.r1, C.i, C.i1);
     for (int k = C.k0; k < C.k1; k++) {
         const GradPlane hi = grad_plane(v, C.cs, (k + 1) * C.pl, C.r0, C.r1, C.i, C.i1);
         const long q = k * C.pl + C.r0 + C.i;
         double G[3][3];
-        grad_cell(lo, hi, 0.25 / p.h, G);
+        grad_cell(lo, hi, w.dt4h, G);
         lo = hi;
         double s6[6], ss6[6];
 #pragma unroll
         for (int a = 0; a < 6; a++) ss6[a] = sig_star[a * nc + q];
-        correct_cell(p, G, ss6, s6);
+        correct_cell(w, G, ss6, s6);
 #pragma unroll
         for (int a = 0; a < 6; a++) sig[a * nc + q] = s6[a];
         const double chi_q = chi_src[q];
         chi_dst[q] = chi_q;
-        predict_cell(p, c, G, s6, chi_q, q, nc, sig_star, dpl, sbar_out);
+        predict_cell(w, c, G, s6, chi_q, q, nc, sig_star, dpl, sbar_out);
     }
 }
 
@@ -591,8 +715,9 @@ cudaError_t stress_predict(const StepParams &p, const double *v, const double *s
                            const double *chi, double *sig_star, double *dpl, double *sbar,
                            cudaStream_t s) {
     const long nc = (long)p.nx * p.ny * p.nz;
-    k_stress_predict<<<cell_grid(p.nx, p.ny, (p.nz + kCellChunk - 1) / kCellChunk), kBlock, 0, s>>>(p, stz_const(p), v, sig, chi,
-                                                                    sig_star, dpl, sbar, nc);
+    const March m = march((long)p.nx * p.ny, p.nz);
+    k_stress_predict<<<m.grid, m.threads, 0, s>>>(p, cell_const(p), stz_const(p), m.chunk, v, sig,
+                                                  chi, sig_star, dpl, sbar, nc);
     count_launch();
     return cudaGetLastError();
 }
@@ -600,25 +725,19 @@ cudaError_t stress_predict(const StepParams &p, const double *v, const double *s
 cudaError_t chi_update(const StepParams &p, const double *sig, const double *chi,
                        const double *dpl, const double *sbar, double *chi_new, cudaStream_t s) {
     const long nc = (long)p.nx * p.ny * p.nz;
-    k_chi_update<<<cell_grid(p.nx, p.ny, p.nz), kBlock, 0, s>>>(p, stz_const(p), sig, chi, dpl,
-                                                                sbar, chi_new, nc);
+    const March m = march((long)p.nx * p.ny, p.nz);
+    const ChiConst w{2.0 * p.dt / (p.c0 * p.sY),
+                     0.5 * (p.dt / p.c0) * ((p.l * p.l) / (p.h * p.h)), p.chi_inf};
+    k_chi_update<<<m.grid, m.threads, 0, s>>>(p, stz_const(p), w, m.chunk, sig, chi, dpl, sbar,
+                                              chi_new, nc);
     count_launch();
     return cudaGetLastError();
 }
 
 cudaError_t div_rhs(const StepParams &p, const double *sig_star, double *b, cudaStream_t s) {
-    const long pl = (long)p.nx * p.ny;
     const double scale = p.h * p.h / (p.mu * p.dt) * (0.25 / p.h);
-    cudaError_t e;
-    const long cs = (long)(p.nz + 1) * pl;
-    for (int a = 0; a < 3; a++) {  // wall planes of b are not part of the system
-        e = cudaMemsetAsync(b + a * cs, 0, pl * sizeof(double), s);
-        if (e != cudaSuccess) return e;
-        e = cudaMemsetAsync(b + a * cs + (long)p.nz * pl, 0, pl * sizeof(double), s);
-        if (e != cudaSuccess) return e;
-    }
-    k_div_rhs<<<cell_grid(p.nx, p.ny, (p.nz - 1 + kDivChunk - 1) / kDivChunk), kBlock, 0, s>>>(
-        p, sig_star, b, scale);
+    const March m = march((long)p.nx * p.ny, p.nz - 1);
+    k_div_rhs<<<m.grid, m.threads, 0, s>>>(p, m.chunk, sig_star, b, scale);
     count_launch();
     return cudaGetLastError();
 }
@@ -626,8 +745,9 @@ cudaError_t div_rhs(const StepParams &p, const double *sig_star, double *b, cuda
 cudaError_t stress_correct(const StepParams &p, const double *v, const double *sig_star,
                            double *sig, const double *chi_src, double *chi_dst, cudaStream_t s) {
     const long nc = (long)p.nx * p.ny * p.nz;
-    k_stress_correct<<<cell_grid(p.nx, p.ny, (p.nz + kCellChunk - 1) / kCellChunk), kBlock, 0, s>>>(p, v, sig_star, sig, chi_src,
-                                                                    chi_dst, nc);
+    const March m = march((long)p.nx * p.ny, p.nz);
+    k_stress_correct<<<m.grid, m.threads, 0, s>>>(p, cell_const(p), m.chunk, v, sig_star, sig,
+                                                  chi_src, chi_dst, nc);
     count_launch();
     return cudaGetLastError();
 }
@@ -644,8 +764,9 @@ cudaError_t correct_predict(const StepParams &p, const double *v, double *sig_st
                             const double *chi_src, double *chi_dst, double *dpl, double *sbar,
                             cudaStream_t s) {
     const long nc = (long)p.nx * p.ny * p.nz;
-    k_correct_predict<<<cell_grid(p.nx, p.ny, (p.nz + kCellChunk - 1) / kCellChunk), kBlock, 0,
-                        s>>>(p, stz_const(p), v, sig_star, sig, chi_src, chi_dst, dpl, sbar, nc);
+    const March m = march((long)p.nx * p.ny, p.nz);
+    k_correct_predict<<<m.grid, m.threads, 0, s>>>(p, cell_const(p), stz_const(p), m.chunk, v,
+                                                   sig_star, sig, chi_src, chi_dst, dpl, sbar, nc);
     count_launch();
     return cudaGetLastError();
 }
@@ -847,9 +968,9 @@ __global__ void k_adj_predict(StepParams p, StzConst c, const double *__restrict
                               const double *__restrict__ chib, const double *__restrict__ Db_in,
                               const double *__restrict__ sbb_in, const double *__restrict__ sgb,
                               double *__restrict__ chib_out, double *__restrict__ Lb,
-                              double w_work, long nc) {
+                              double w_work, long nc, int chunk) {
     CellColumn C;
-    if (!cell_column(p.nx, p.ny, p.nz, C)) return;
+    if (!cell_column(p.nx, p.ny, p.nz, chunk, C)) return;
     const double inv4h = 0.25 / p.h, dt = p.dt, mu = p.mu;
     const double rhs_scale = p.h * p.h / (p.mu * dt);  // (h^2/(mu dt)) / (4h) * 4h
     const double work = w_work * 2.0 * dt * p.h * p.h * p.h;
@@ -981,34 +1102,40 @@ __device__ __forceinline__ DivLayer tensor_layer(const Load &ld, long base, long
     DivLayer L;
 #pragma unroll
     for (int a = 0; a < 3; a++) {
-        L.X[a] = (T01[a][0] - T00[a][0]) + (T11[a][0] - T10[a][0]);
-        L.Y[a] = (T10[a][1] - T00[a][1]) + (T11[a][1] - T01[a][1]);
+        L.XY[a] = ((T01[a][0] - T00[a][0]) + (T11[a][0] - T10[a][0])) +
+                  ((T10[a][1] - T00[a][1]) + (T11[a][1] - T01[a][1]));
         L.Z[a] = (T00[a][2] + T01[a][2]) + (T10[a][2] + T11[a][2]);
     }
     return L;
 }
 
-// out = add + scale * corner-div T at the interior corners (wall planes of
-// out are left alone); the transpose of the cell gradient of Eq. (31) is
-// -1/(4h) times this divergence
+// out = add + scale * corner-div T at the interior corners, zero on the wall
+// planes; the transpose of the cell gradient of Eq. (31) is -1/(4h) times this
+// divergence
 template <class Load>
-__global__ void k_corner_div(StepParams p, Load ld, const double *__restrict__ add,
-                             double *__restrict__ out, double scale) {
+__global__ void __launch_bounds__(128)
+    k_corner_div(StepParams p, Load ld, int chunk, const double *__restrict__ add,
+                 double *__restrict__ out, double scale) {
     const int nx = p.nx, ny = p.ny, nz = p.nz;
-    const int i = blockIdx.x * BX + threadIdx.x, j = blockIdx.y * BY + threadIdx.y;
-    if (i >= nx || j >= ny) return;
-    const int k0 = 1 + blockIdx.z * kDivChunk;
-    const int k1 = k0 + kDivChunk < nz ? k0 + kDivChunk : nz;
+    const int m = blockIdx.x * blockDim.x + threadIdx.x, j = m / nx, i = m - j * nx;
+    if (j >= ny) return;
+    const int k0 = 1 + blockIdx.y * chunk;
+    const int k1 = k0 + chunk < nz ? k0 + chunk : nz;
     const int im = i ? i - 1 : nx - 1, jm = j ? j - 1 : ny - 1;
     const long pl = (long)nx * ny, cs = (long)(nz + 1) * pl;
     const long rj0 = (long)jm * nx, rj1 = (long)j * nx;
+#pragma unroll
+    for (int a = 0; a < 3; a++) {
+        if (k0 == 1) out[a * cs + m] = 0.0;
+        if (k1 == nz) out[a * cs + nz * pl + m] = 0.0;
+    }
     DivLayer lo = tensor_layer(ld, (long)(k0 - 1) * pl, rj0, rj1, im, i);
     for (int k = k0; k < k1; k++) {
         const DivLayer hi = tensor_layer(ld, (long)k * pl, rj0, rj1, im, i);
-        const long node = (long)k * pl + (long)j * nx + i;
+        const long node = (long)k * pl + m;
 #pragma unroll
         for (int a = 0; a < 3; a++) {
-            const double d = (lo.X[a] + hi.X[a]) + (lo.Y[a] + hi.Y[a]) + (hi.Z[a] - lo.Z[a]);
+            const double d = (lo.XY[a] + hi.XY[a]) + (hi.Z[a] - lo.Z[a]);
             out[a * cs + node] = (add ? add[a * cs + node] : 0.0) + scale * d;
         }
         lo = hi;
@@ -1036,27 +1163,15 @@ __global__ void __launch_bounds__(kRedThreads)
     }
 }
 
-cudaError_t zero_walls(const StepParams &p, double *x, cudaStream_t s) {
-    const long pl = (long)p.nx * p.ny, cs = (long)(p.nz + 1) * pl;
-    for (int a = 0; a < 3; a++) {
-        cudaError_t e = cudaMemsetAsync(x + a * cs, 0, pl * sizeof(double), s);
-        if (e != cudaSuccess) return e;
-        e = cudaMemsetAsync(x + a * cs + (long)p.nz * pl, 0, pl * sizeof(double), s);
-        if (e != cudaSuccess) return e;
-    }
-    return cudaSuccess;
-}
-
 }  // namespace
 
 cudaError_t adj_correct(const StepParams &p, const double *sb1, const double *vb1,
                         double *rhs_out, cudaStream_t s) {
     const long nc = (long)p.nx * p.ny * p.nz;
-    cudaError_t e = zero_walls(p, rhs_out, s);
-    if (e != cudaSuccess) return e;
     const LoadCSym ld{sb1, nc, p.lam, p.mu};
-    k_corner_div<LoadCSym><<<cell_grid(p.nx, p.ny, (p.nz - 1 + kDivChunk - 1) / kDivChunk),
-                             kBlock, 0, s>>>(p, ld, vb1, rhs_out, -p.dt * 0.25 / p.h);
+    const March m = march((long)p.nx * p.ny, p.nz - 1);
+    k_corner_div<LoadCSym><<<m.grid, m.threads, 0, s>>>(p, ld, m.chunk, vb1, rhs_out,
+                                                        -p.dt * 0.25 / p.h);
     count_launch();
     return cudaGetLastError();
 }
@@ -1076,8 +1191,9 @@ cudaError_t adj_predict(const StepParams &p, const double *v, const double *lam,
                         const double *Db, const double *sbb, const double *sgb, double *chib_out,
                         double *Lb, double w_work, cudaStream_t s) {
     const long nc = (long)p.nx * p.ny * p.nz;
-    k_adj_predict<<<cell_grid(p.nx, p.ny, (p.nz + kCellChunk - 1) / kCellChunk), kBlock, 0, s>>>(
-        p, stz_const(p), v, lam, sig, chi, sb1, chib, Db, sbb, sgb, chib_out, Lb, w_work, nc);
+    const March m = march((long)p.nx * p.ny, p.nz);
+    k_adj_predict<<<m.grid, m.threads, 0, s>>>(p, stz_const(p), v, lam, sig, chi, sb1, chib, Db,
+                                               sbb, sgb, chib_out, Lb, w_work, nc, m.chunk);
     count_launch();
     return cudaGetLastError();
 }
@@ -1085,11 +1201,9 @@ cudaError_t adj_predict(const StepParams &p, const double *v, const double *lam,
 cudaError_t adj_grad_transpose(const StepParams &p, const double *Lb, double *vb,
                                cudaStream_t s) {
     const long nc = (long)p.nx * p.ny * p.nz;
-    cudaError_t e = zero_walls(p, vb, s);
-    if (e != cudaSuccess) return e;
     const LoadFull ld{Lb, nc};
-    k_corner_div<LoadFull><<<cell_grid(p.nx, p.ny, (p.nz - 1 + kDivChunk - 1) / kDivChunk),
-                             kBlock, 0, s>>>(p, ld, nullptr, vb, -0.25 / p.h);
+    const March m = march((long)p.nx * p.ny, p.nz - 1);
+    k_corner_div<LoadFull><<<m.grid, m.threads, 0, s>>>(p, ld, m.chunk, nullptr, vb, -0.25 / p.h);
     count_launch();
     return cudaGetLastError();
 }

@@ -57,23 +57,25 @@ struct CoarseStrip {
     Coarse<double> c;
 };
 
-// numerators of the node at window row jj, columns xm, x0, xp (offsets): the
-// right-hand side minus every off-centre term
-__device__ __forceinline__ void numer(const FineStrip &op, const double *P, const double *D,
+// residual of the node at window row jj, columns xm, x0, xp (offsets),
+// summed so that the centre terms cancel against their neighbours first
+__device__ __forceinline__ void resid(const FineStrip &op, const double *P, const double *D,
                                       const double *R, const double *, const double *, int w,
                                       int jj, int xm, int x0, int xp, double o[3]) {
-    const double lp = op.f.lp, kq = op.f.kq;
+    const double lp = op.f.lp, kq = op.f.kq, d0 = op.f.d0;
     const double *p = P + jj * w, *pm = p - w, *pp = p + w, *d = D + jj * w, *dm = d - w,
                  *dp = d + w, *r = R + jj * w + x0;
     const double m01 = ((pp[xp + 1] - pm[xp + 1]) - (pp[xm + 1] - pm[xm + 1])) +
                        (d[xp + 2] - d[xm + 2]);
     const double m10 = ((pp[xp] - pm[xp]) - (pp[xm] - pm[xm])) + (dp[x0 + 2] - dm[x0 + 2]);
     const double m2 = (d[xp] - d[xm]) + (dp[x0 + 1] - dm[x0 + 1]);
-    o[0] = r[0] + lp * (p[xm] + p[xp]) + (pm[x0] + pp[x0]) + kq * m01;
-    o[1] = r[1] + lp * (pm[x0 + 1] + pp[x0 + 1]) + (p[xm + 1] + p[xp + 1]) + kq * m10;
-    o[2] = r[2] + (p[xm + 2] + p[xp + 2]) + (pm[x0 + 2] + pp[x0 + 2]) + kq * m2;
+    o[0] = ((lp * (p[xm] + p[xp]) - d0 * p[x0]) + (pm[x0] + pp[x0]) + r[0]) + kq * m01;
+    o[1] = ((lp * (pm[x0 + 1] + pp[x0 + 1]) - d0 * p[x0 + 1]) + (p[xm + 1] + p[xp + 1]) + r[1]) +
+           kq * m10;
+    o[2] = ((r[2] - d0 * p[x0 + 2]) + (p[xm + 2] + p[xp + 2]) + (pm[x0 + 2] + pp[x0 + 2])) +
+           kq * m2;
 }
-__device__ __forceinline__ void numer(const CoarseStrip &op, const double *P, const double *,
+__device__ __forceinline__ void resid(const CoarseStrip &op, const double *P, const double *,
                                       const double *R, const double *U, const double *V, int w,
                                       int jj, int xm, int x0, int xp, double o[3]) {
     const int col[3] = {xm, x0, xp};
@@ -82,9 +84,11 @@ __device__ __forceinline__ void numer(const CoarseStrip &op, const double *P, co
     coarse_plane_terms(op.c, u, t);
     const int q = jj * w + x0;
 #pragma unroll
-    for (int a = 0; a < 3; a++) o[a] = R[q + a] - ((U[q - w + a] + V[q + w + a]) + t[a]);
+    for (int a = 0; a < 3; a++)
+        o[a] = R[q + a] - (op.c.cd[a][0] * P[q + a] + ((U[q - w + a] + V[q + w + a]) + t[a]));
 }
-// component a alone: the passes give every component a thread, so that a pass
+// numerator of component a of a node's update (the right-hand side minus every
+// off-centre term): the passes give every component a thread, so that a pass
 // over a few rows occupies all four schedulers (one warp instruction holds its
 // scheduler's FP64 pipe for 64 clocks)
 __device__ __forceinline__ double numer_c(const FineStrip &op, const double *P, const double *D,
@@ -116,8 +120,6 @@ __device__ __forceinline__ double numer_c(const CoarseStrip &op, const double *P
 }
 __device__ __forceinline__ double dinv(const FineStrip &op, int) { return op.f.dinv; }
 __device__ __forceinline__ double dinv(const CoarseStrip &op, int a) { return op.c.dinv[a]; }
-__device__ __forceinline__ double diag(const FineStrip &op, int) { return op.f.d0; }
-__device__ __forceinline__ double diag(const CoarseStrip &op, int a) { return op.c.cd[a][0]; }
 
 // what a node contributes besides S and D: nothing on coarse levels, the
 // right-hand side with the z sums on the finest one
@@ -216,12 +218,12 @@ __global__ void __launch_bounds__(NT, 2)
             if (y >= g.ny) continue;
             const int x0 = scol(i, hx);
             double o[3];
-            numer(op, P, D, R, U, V, w, jj, scol(i ? i - 1 : nx - 1, hx), x0,
+            resid(op, P, D, R, U, V, w, jj, scol(i ? i - 1 : nx - 1, hx), x0,
                   scol(i + 1 < nx ? i + 1 : 0, hx), o);
             const long q = (long)y * nx + i;
 #pragma unroll
             for (int a = 0; a < 3; a++) {
-                out[q + a * g.cs] = o[a] - diag(op, a) * P[jj * w + x0 + a];
+                out[q + a * g.cs] = o[a];
                 if (k == 1) vout[q + a * g.cs] = 0.0;
                 if (k + 1 == g.nz) vout[q + a * g.cs + (long)g.nz * g.ps] = 0.0;
             }
