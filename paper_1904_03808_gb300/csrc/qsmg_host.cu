@@ -1217,22 +1217,26 @@ mg_status qs_explicit_step(mg_ctx *ctx, qs_state *state, double dt, double rho, 
     const Dims &d = ctx->L[0];
     const size_t nc = (size_t)d.nx * d.ny * d.nz, nv = corner_count(d);
     const StepParams p = step_params(ctx, dt);
-    // the new stress, chi and velocity go to the context's step scratch
-    // (sig_star, chi_tmp, rhs), then back into the state
+    // steps alternate between the state's arrays and the context's step
+    // scratch (sig_star, chi_tmp, rhs); an odd count is copied back at the end
+    double *sig[2] = {state->sigma, ctx->sig_star}, *chi[2] = {state->chi, ctx->chi_tmp},
+           *v[2] = {state->v, ctx->rhs};
     for (int n = 0; n < nsteps; n++) {
-        CK(explicit_stress(p, state->v, state->sigma, state->chi, ctx->sig_star, ctx->dpl,
-                           ctx->sbar, ctx->st));
-        CK(chi_update(p, state->sigma, state->chi, ctx->dpl, ctx->sbar, ctx->chi_tmp, ctx->st));
-        CK(explicit_velocity(p, rho, kappa, state->v, state->sigma, ctx->rhs, ctx->st));
+        const int i = n & 1, o = 1 - i;
+        CK(explicit_stress(p, v[i], sig[i], chi[i], sig[o], ctx->dpl, ctx->sbar, ctx->st));
+        CK(chi_update(p, sig[i], chi[i], ctx->dpl, ctx->sbar, chi[o], ctx->st));
+        CK(explicit_velocity(p, rho, kappa, v[i], sig[i], v[o], ctx->st));
+        CK(wall_fill(wall_params(ctx, state->t + dt), v[o], ctx->st));
+        state->t += dt;
+        state->step += 1;
+    }
+    if (nsteps & 1) {
         CK(cudaMemcpyAsync(state->sigma, ctx->sig_star, 6 * nc * sizeof(double),
                            cudaMemcpyDeviceToDevice, ctx->st));
         CK(cudaMemcpyAsync(state->chi, ctx->chi_tmp, nc * sizeof(double),
                            cudaMemcpyDeviceToDevice, ctx->st));
         CK(cudaMemcpyAsync(state->v, ctx->rhs, nv * sizeof(double), cudaMemcpyDeviceToDevice,
                            ctx->st));
-        CK(wall_fill(wall_params(ctx, state->t + dt), state->v, ctx->st));
-        state->t += dt;
-        state->step += 1;
     }
     CK(cudaStreamSynchronize(ctx->st));
     return MG_OK;

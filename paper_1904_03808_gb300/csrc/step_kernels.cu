@@ -179,31 +179,30 @@ __device__ __forceinline__ bool cell_column(int nx, int ny, int nz, int chunk, C
 // constants of the predictor and the corrector: G of a cell enters both only
 // as dt G, so the scale of the gradient carries the time step
 struct CellConst {
-    double dt4h;     // dt / (4 h)
+    double dt4h, dt2h;  // dt / (4 h), dt / (2 h)
     double lam, mu, mu2, mu2dt;
 };
 CellConst cell_const(const StepParams &p) {
-    return CellConst{p.dt * (0.25 / p.h), p.lam, p.mu, 2.0 * p.mu, 2.0 * p.mu * p.dt};
+    return CellConst{p.dt * (0.25 / p.h), p.dt * (0.5 / p.h), p.lam, p.mu, 2.0 * p.mu, 2.0 * p.mu * p.dt};
 }
 
 // Eq. (27) at cell q: sigma* = sigma + dt (L sigma + sigma L^T - tr(L) sigma
 // - 2 mu D^pl sigma0 / sbar) from dt times the cell-centre gradient of v^n (G)
-// and the cell's sigma^n (s6) and chi^n; also stores D^pl and sbar.  With
+// and the cell's sigma^n (s6) and chi^n; also stores D^pl and sbar.  Its
+// increment (objective_increment): with
 // P = 2 mu dt D^pl / sbar and H = dt L - (tr(dt L) + P) / 2 I the update is
 // sigma + (H sigma + sigma H^T + P m I), m the mean stress: 49 instructions
 // where the terms one by one take 68.  The increment is summed before it is
 // added to sigma, which rounds the result once.
-__device__ __forceinline__ void predict_cell(const CellConst &w, const StzConst &c,
-                                             const double (&G)[3][3], const double (&s6)[6],
-                                             double chi_q, long q, long nc,
-                                             double *__restrict__ sig_star,
-                                             double *__restrict__ dpl,
-                                             double *__restrict__ sbar_out) {
+__device__ __forceinline__ void objective_increment(const CellConst &w, const StzConst &c,
+                                                    const double (&G)[3][3],
+                                                    const double (&s6)[6], double chi_q,
+                                                    double (&inc)[6], double &D, double &sb) {
     const double S[3][3] = {{s6[0], s6[5], s6[4]}, {s6[5], s6[1], s6[3]}, {s6[4], s6[3], s6[2]}};
     const double m = (s6[0] + s6[1] + s6[2]) * (1.0 / 3.0);
-    double sb, inv_sb;
+    double inv_sb;
     sbar_inv(j2_of(s6, m), sb, inv_sb);
-    const double D = stz_rate(c, sb, inv_sb, chi_q);
+    D = stz_rate(c, sb, inv_sb, chi_q);
     const double P = w.mu2dt * D * inv_sb;
     const double tr = 0.5 * (G[0][0] + G[1][1] + G[2][2] + P);
     double H[3][3];
@@ -216,7 +215,7 @@ __device__ __forceinline__ void predict_cell(const CellConst &w, const StzConst 
         double t = H[a][0] * S[0][a];
         t = fma(H[a][1], S[1][a], t);
         t = fma(H[a][2], S[2][a], t);
-        sig_star[a * nc + q] = S[a][a] + fma(2.0, t, P * m);
+        inc[a] = fma(2.0, t, P * m);
     }
     const int ia[3] = {1, 0, 0}, ib[3] = {2, 2, 1};
 #pragma unroll
@@ -228,8 +227,19 @@ __device__ __forceinline__ void predict_cell(const CellConst &w, const StzConst 
             if (e > 0) t = fma(H[a][e], S[e][b], t);
             t = fma(S[a][e], H[b][e], t);
         }
-        sig_star[(3 + n) * nc + q] = S[a][b] + t;
+        inc[3 + n] = t;
     }
+}
+__device__ __forceinline__ void predict_cell(const CellConst &w, const StzConst &c,
+                                             const double (&G)[3][3], const double (&s6)[6],
+                                             double chi_q, long q, long nc,
+                                             double *__restrict__ sig_star,
+                                             double *__restrict__ dpl,
+                                             double *__restrict__ sbar_out) {
+    double inc[6], D, sb;
+    objective_increment(w, c, G, s6, chi_q, inc, D, sb);
+#pragma unroll
+    for (int n = 0; n < 6; n++) sig_star[n * nc + q] = s6[n] + inc[n];
     dpl[q] = D;
     sbar_out[q] = sb;
 }
@@ -347,8 +357,11 @@ __device__ __forceinline__ double dif_y(const double (&f)[2][2]) {
     return (f[1][0] - f[0][0]) + (f[1][1] - f[0][1]);
 }
 
-__device__ __forceinline__ DivLayer div_layer(const double *__restrict__ ss, long nc, long base,
-                                              long rj0, long rj1, int im, int i) {
+// the layer's x-y part, and the 2 x 2 cells of the components whose z
+// derivative enters (xz, yz, zz)
+__device__ __forceinline__ void div_parts(const double *__restrict__ ss, long nc, long base,
+                                          long rj0, long rj1, int im, int i, double (&xy)[3],
+                                          double (&fz)[3][2][2]) {
     auto cells = [&](int n, double (&f)[2][2]) {
         const double *g = ss + n * nc + base;
         f[0][0] = g[rj0 + im];
@@ -356,24 +369,28 @@ __device__ __forceinline__ DivLayer div_layer(const double *__restrict__ ss, lon
         f[1][0] = g[rj1 + im];
         f[1][1] = g[rj1 + i];
     };
-    DivLayer L;
     double f[2][2];
     cells(5, f);  // xy: its x- and y-differences from the two diagonals
     const double d1 = f[1][1] - f[0][0], d2 = f[0][1] - f[1][0];
-    L.XY[1] = d1 + d2;
-    L.XY[0] = d1 - d2;
+    xy[1] = d1 + d2;
+    xy[0] = d1 - d2;
     cells(0, f);
-    L.XY[0] += dif_x(f);
+    xy[0] += dif_x(f);
     cells(1, f);
-    L.XY[1] += dif_y(f);
-    cells(4, f);
-    L.XY[2] = dif_x(f);
-    L.Z[0] = sum4(f);
-    cells(3, f);
-    L.XY[2] += dif_y(f);
-    L.Z[1] = sum4(f);
-    cells(2, f);
-    L.Z[2] = sum4(f);
+    xy[1] += dif_y(f);
+    cells(4, fz[0]);
+    cells(3, fz[1]);
+    cells(2, fz[2]);
+    xy[2] = dif_x(fz[0]) + dif_y(fz[1]);
+}
+
+__device__ __forceinline__ DivLayer div_layer(const double *__restrict__ ss, long nc, long base,
+                                              long rj0, long rj1, int im, int i) {
+    DivLayer L;
+    double f[3][2][2];
+    div_parts(ss, nc, base, rj0, rj1, im, i, L.XY, f);
+#pragma unroll
+    for (int a = 0; a < 3; a++) L.Z[a] = sum4(f[a]);
     return L;
 }
 
@@ -497,62 +514,89 @@ __global__ void k_wall_fill(WallParams w, double *__restrict__ v) {
 // ------------------------------------------------------------ explicit method
 // (section 3.2): forward Euler of Eqs. (24)-(26) with ENO advection (Eq. 33)
 
-// ENO first derivative, Eq. (33), from the values at offsets -2..2 along one
-// axis and the velocity component u along it: the one-sided three-point
-// stencil on the upwind side where that side is smoother than the centre,
-// else the centred difference.  The smoothness test compares the magnitudes
-// of the undivided second differences: the curvatures of Eq. (33) are those
-// divided by the same h^2 > 0, which cannot reorder them (the division is
-// monotone), and FP64 division is costly here; inv2h = 1 / (2h).
-__device__ __forceinline__ double eno_d(double fm2, double fm1, double f0, double fp1, double fp2,
-                                        double u, double inv2h) {
-    const double cm = fabs(f0 - 2.0 * fm1 + fm2);
-    const double c0 = fabs(fp1 - 2.0 * f0 + fm1);
-    const double cp = fabs(fp2 - 2.0 * fp1 + f0);
-    if (u < 0.0 && c0 > cp) return (-fp2 + 4.0 * fp1 - 3.0 * f0) * inv2h;
-    if (u > 0.0 && c0 > cm) return (3.0 * f0 - 4.0 * fm1 + fm2) * inv2h;
-    return (fp1 - fm1) * inv2h;
+// ENO first derivative, Eq. (33), times 2 h, from the values at offsets -2..2
+// along one axis and the velocity component u along it: the one-sided
+// three-point stencil on the upwind side where that side is smoother than the
+// centre, else the centred difference.  The smoothness test compares the
+// magnitudes of the undivided second differences: the curvatures of Eq. (33)
+// are those divided by the same h^2 > 0, which cannot reorder them.  With f1
+// the neighbour on the upwind side and c_up the second difference about it the
+// one-sided stencil 3 f0 - 4 f1 + f2 is c_up + 2 (f0 - f1); values are chosen
+// and magnitudes compared with integer instructions, which leaves 7 FP64
+// instructions (they set the pace: 19 clocks of an SM each) of about 20.  c0 returns the centred second
+// difference.
+__device__ __forceinline__ double eno_2h(double fm2, double fm1, double f0, double fp1, double fp2,
+                                         double u, double &c0) {
+    const bool neg = u < 0.0;
+    const double f1 = neg ? fp1 : fm1;
+    // (explicit fma: a doubling would otherwise become an addition of its own)
+    const double cu = fma(-2.0, f1, neg ? fp2 : f0) + (neg ? f0 : fm2);
+    c0 = fma(-2.0, f0, fp1) + fm1;
+    const double one = fma(2.0, f0 - f1, cu), mid = fp1 - fm1;
+    // |c0| > |cu|, false for a NaN on either side
+    const long long m0 = __double_as_longlong(c0) & 0x7fffffffffffffffLL,
+                    mu = __double_as_longlong(cu) & 0x7fffffffffffffffLL;
+    const bool smoother = m0 > mu && m0 <= 0x7ff0000000000000LL;
+    const double side = __longlong_as_double(__double_as_longlong(one) ^
+                                             (neg ? (long long)0x8000000000000000ULL : 0LL));
+    return smoother && (neg || u > 0.0) ? side : mid;
 }
 
-// (u.grad) sigma_n at cell (i, j, k) for the 6 stored components: ENO
+// offsets along an axis of n entries, -2 .. 2 around i, periodic
+__device__ __forceinline__ void around(int i, int n, int (&o)[5]) {
+#pragma unroll
+    for (int m = 0; m < 5; m++) {
+        const int a = i + m - 2;
+        o[m] = a < 0 ? a + n : (a >= n ? a - n : a);
+    }
+}
+
+// 2 h (u.grad) sigma_n at cell (i, j, k) for the 6 stored components: ENO
 // derivatives (Eq. 33) along x and y (wrapping) and z, where cell fields two
 // layers beyond the z boundaries are extrapolated linearly from the two
 // layers next to them; u is the cell's advecting velocity
-__device__ __forceinline__ void stress_advection(const StepParams &p,
-                                                 const double *__restrict__ sig, long nc, int i,
-                                                 int j, int k, const double (&u)[3],
-                                                 double inv2h, double (&adv)[6]) {
-    const int nx = p.nx, ny = p.ny, nz = p.nz;
-    const long pl = (long)nx * ny;
-    int ix[5], jy[5];
-#pragma unroll
-    for (int m = 0; m < 5; m++) {
-        int a = i + m - 2, b = j + m - 2;
-        ix[m] = a < 0 ? a + nx : (a >= nx ? a - nx : a);
-        jy[m] = b < 0 ? b + ny : (b >= ny ? b - ny : b);
-    }
+__device__ __forceinline__ void stress_advection(const double *__restrict__ sig, long nc, int nx,
+                                                 long pl, int nz, int j, int k, long col,
+                                                 const int (&ix)[5], const int (&jy)[5],
+                                                 const double (&u)[3], double (&adv)[6]) {
+    const long rx = k * pl + (long)j * nx, cy = k * pl + (col - (long)j * nx);
+    const bool inner = k >= 2 && k < nz - 2;
 #pragma unroll
     for (int n = 0; n < 6; n++) {
         const double *f = sig + n * nc;
-        double fx[5], fy[5], fz[5];
+        double fx[5], fy[5], fz[5], c0;
 #pragma unroll
         for (int m = 0; m < 5; m++) {
-            fx[m] = f[(long)k * pl + (long)j * nx + ix[m]];
-            fy[m] = f[(long)k * pl + (long)jy[m] * nx + i];
-            const int kk = k + m - 2;
-            const long col = (long)j * nx + i;
-            if (kk < 0)
-                fz[m] = f[col] + kk * (f[pl + col] - f[col]);
-            else if (kk > nz - 1)
-                fz[m] = f[(long)(nz - 1) * pl + col] +
-                        (kk - (nz - 1)) * (f[(long)(nz - 1) * pl + col] - f[(long)(nz - 2) * pl + col]);
-            else
-                fz[m] = f[(long)kk * pl + col];
+            fx[m] = f[rx + ix[m]];
+            fy[m] = f[cy + (long)jy[m] * nx];
         }
-        adv[n] = u[0] * eno_d(fx[0], fx[1], fx[2], fx[3], fx[4], u[0], inv2h) +
-                 u[1] * eno_d(fy[0], fy[1], fy[2], fy[3], fy[4], u[1], inv2h) +
-                 u[2] * eno_d(fz[0], fz[1], fz[2], fz[3], fz[4], u[2], inv2h);
+        if (inner) {
+#pragma unroll
+            for (int m = 0; m < 5; m++) fz[m] = f[(k + m - 2) * pl + col];
+        } else {
+#pragma unroll
+            for (int m = 0; m < 5; m++) {
+                const int kk = k + m - 2;
+                if (kk < 0)
+                    fz[m] = f[col] + kk * (f[pl + col] - f[col]);
+                else if (kk > nz - 1)
+                    fz[m] = f[(nz - 1) * pl + col] +
+                            (kk - (nz - 1)) * (f[(nz - 1) * pl + col] - f[(nz - 2) * pl + col]);
+                else
+                    fz[m] = f[kk * pl + col];
+            }
+        }
+        double t = u[0] * eno_2h(fx[0], fx[1], fx[2], fx[3], fx[4], u[0], c0);
+        t = fma(u[1], eno_2h(fy[0], fy[1], fy[2], fy[3], fy[4], u[1], c0), t);
+        adv[n] = fma(u[2], eno_2h(fz[0], fz[1], fz[2], fz[3], fz[4], u[2], c0), t);
     }
+}
+
+// the mean of a cell's 8 corner velocities, from the plane sums below and above
+__device__ __forceinline__ void mean_velocity(const GradPlane &lo, const GradPlane &hi,
+                                              double (&u)[3]) {
+#pragma unroll
+    for (int a = 0; a < 3; a++) u[a] = 0.125 * (lo.Z[a] + hi.Z[a]);
 }
 
 // Eq. (25) at cell centres: sigma' = sigma + dt (-(u.grad) sigma + L sigma +
@@ -560,152 +604,157 @@ __device__ __forceinline__ void stress_advection(const StepParams &p,
 // gradient of v, u the mean of the cell's 8 corner velocities; the ENO
 // stencils reach two cells out, z ghost cells extrapolate each component
 // linearly from the two layers next to the wall; D^pl and sbar of the state
-// are written for the chi update
-__global__ void k_explicit_stress(StepParams p, StzConst c, const double *__restrict__ v,
-                                  const double *__restrict__ sig, const double *__restrict__ chi,
-                                  double *__restrict__ sig_new, double *__restrict__ dpl,
-                                  double *__restrict__ sbar_out, long nc) {
-    const int nx = p.nx, ny = p.ny, nz = p.nz;
-    int i, j, k;
-    if (!cell_ijk(nx, ny, i, j, k)) return;
-    const long pl = (long)nx * ny, cs = (long)(nz + 1) * pl;
-    const int i1 = i + 1 < nx ? i + 1 : 0, j1 = j + 1 < ny ? j + 1 : 0;
-    const double h = p.h, inv2h = 0.5 / p.h;
-    double G[3][3], u[3];
+// are written for the chi update.  Columns march in z as in the predictor.
+__global__ void __launch_bounds__(128)
+    k_explicit_stress(StepParams p, CellConst w, StzConst c, int chunk,
+                      const double *__restrict__ v, const double *__restrict__ sig,
+                      const double *__restrict__ chi, double *__restrict__ sig_new,
+                      double *__restrict__ dpl, double *__restrict__ sbar_out, long nc) {
+    CellColumn C;
+    if (!cell_column(p.nx, p.ny, p.nz, chunk, C)) return;
+    const long col = C.r0 + C.i;
+    int ix[5], jy[5];
+    around(C.i, p.nx, ix);
+    around(C.j, p.ny, jy);
+    GradPlane lo = grad_plane(v, C.cs, C.k0 * C.pl, C.r0, C.r1, C.i, C.i1);
+    for (int k = C.k0; k < C.k1; k++) {
+        const GradPlane hi = grad_plane(v, C.cs, (k + 1) * C.pl, C.r0, C.r1, C.i, C.i1);
+        const long q = k * C.pl + col;
+        double G[3][3], u[3], adv[6], s6[6], rate[6], D, sb;
+        grad_cell(lo, hi, w.dt4h, G);
+        mean_velocity(lo, hi, u);
+        lo = hi;
+        stress_advection(sig, nc, p.nx, C.pl, p.nz, C.j, k, col, ix, jy, u, adv);
 #pragma unroll
-    for (int a = 0; a < 3; a++) {
-        const double *g = v + a * cs;
-        const long b0 = (long)k * pl, b1 = b0 + pl, r0 = (long)j * nx, r1 = (long)j1 * nx;
-        const double c000 = g[b0 + r0 + i], c001 = g[b0 + r0 + i1], c010 = g[b0 + r1 + i],
-                     c011 = g[b0 + r1 + i1], c100 = g[b1 + r0 + i], c101 = g[b1 + r0 + i1],
-                     c110 = g[b1 + r1 + i], c111 = g[b1 + r1 + i1];
-        G[a][0] = ((c001 - c000) + (c011 - c010) + (c101 - c100) + (c111 - c110)) * (0.25 / h);
-        G[a][1] = ((c010 - c000) + (c011 - c001) + (c110 - c100) + (c111 - c101)) * (0.25 / h);
-        G[a][2] = ((c100 - c000) + (c110 - c010) + (c101 - c001) + (c111 - c011)) * (0.25 / h);
-        u[a] = 0.125 * (((c000 + c001) + (c010 + c011)) + ((c100 + c101) + (c110 + c111)));
+        for (int a = 0; a < 6; a++) s6[a] = sig[a * nc + q];
+        objective_increment(w, c, G, s6, chi[q], rate, D, sb);
+        const double lt = w.lam * (G[0][0] + G[1][1] + G[2][2]);
+#pragma unroll
+        for (int a = 0; a < 3; a++) rate[a] += fma(w.mu2, G[a][a], lt);
+        rate[3] = fma(w.mu, G[1][2] + G[2][1], rate[3]);
+        rate[4] = fma(w.mu, G[0][2] + G[2][0], rate[4]);
+        rate[5] = fma(w.mu, G[0][1] + G[1][0], rate[5]);
+#pragma unroll
+        for (int n = 0; n < 6; n++) sig_new[n * nc + q] = s6[n] + fma(-w.dt2h, adv[n], rate[n]);
+        dpl[q] = D;
+        sbar_out[q] = sb;
     }
-    const long q = (long)k * pl + (long)j * nx + i;
-    double s6[6], adv[6];
-#pragma unroll
-    for (int n = 0; n < 6; n++) s6[n] = sig[n * nc + q];
-    stress_advection(p, sig, nc, i, j, k, u, inv2h, adv);
-    const double S[3][3] = {{s6[0], s6[5], s6[4]}, {s6[5], s6[1], s6[3]}, {s6[4], s6[3], s6[2]}};
-    const double sb = sbar_of(s6);
-    const double inv_sb = sb > 0.0 ? 1.0 / sb : 0.0;
-    const double D = stz_rate(c, sb, inv_sb, chi[q]);
-    const double trL = G[0][0] + G[1][1] + G[2][2];
-    const double m3 = (s6[0] + s6[1] + s6[2]) * (1.0 / 3.0);
-    const double pl_ = (D > 0.0) ? 2.0 * p.mu * D * inv_sb : 0.0;
-    const int ia[6] = {0, 1, 2, 1, 0, 0}, ib[6] = {0, 1, 2, 2, 2, 1};
-#pragma unroll
-    for (int n = 0; n < 6; n++) {
-        const int a = ia[n], b = ib[n];
-        double rate = -adv[n] - trL * S[a][b];
-#pragma unroll
-        for (int e = 0; e < 3; e++) rate += G[a][e] * S[e][b] + S[a][e] * G[b][e];
-        rate += (a == b ? p.lam * trL : 0.0) + p.mu * (G[a][b] + G[b][a]);
-        rate -= pl_ * (S[a][b] - (a == b ? m3 : 0.0));
-        sig_new[n * nc + q] = S[a][b] + p.dt * rate;
-    }
-    dpl[q] = D;
-    sbar_out[q] = sb;
 }
 
 // the stress advection of the general constitutive law (section 2), which
 // Eq. (27) drops, as an option of the quasi-static step: sigma* -= dt (u.grad)
 // sigma^n, u the mean of the cell's 8 corner velocities of v^n (the
 // explicit method's advection, Eq. 33 and its ghosts)
-__global__ void k_stress_advect(StepParams p, const double *__restrict__ v,
-                                const double *__restrict__ sig, double *__restrict__ sig_star,
-                                long nc) {
-    const int nx = p.nx, ny = p.ny, nz = p.nz;
-    int i, j, k;
-    if (!cell_ijk(nx, ny, i, j, k)) return;
-    const long pl = (long)nx * ny, cs = (long)(nz + 1) * pl;
-    const int i1 = i + 1 < nx ? i + 1 : 0, j1 = j + 1 < ny ? j + 1 : 0;
-    double u[3];
+__global__ void __launch_bounds__(128)
+    k_stress_advect(StepParams p, CellConst w, int chunk, const double *__restrict__ v,
+                    const double *__restrict__ sig, double *__restrict__ sig_star, long nc) {
+    CellColumn C;
+    if (!cell_column(p.nx, p.ny, p.nz, chunk, C)) return;
+    const long col = C.r0 + C.i;
+    int ix[5], jy[5];
+    around(C.i, p.nx, ix);
+    around(C.j, p.ny, jy);
+    auto corner_sum = [&](int k, double (&z)[3]) {
 #pragma unroll
-    for (int a = 0; a < 3; a++) {
-        const double *g = v + a * cs;
-        const long b0 = (long)k * pl, b1 = b0 + pl, r0 = (long)j * nx, r1 = (long)j1 * nx;
-        u[a] = 0.125 * (((g[b0 + r0 + i] + g[b0 + r0 + i1]) + (g[b0 + r1 + i] + g[b0 + r1 + i1])) +
-                        ((g[b1 + r0 + i] + g[b1 + r0 + i1]) + (g[b1 + r1 + i] + g[b1 + r1 + i1])));
+        for (int a = 0; a < 3; a++) {
+            const double *g = v + a * C.cs + k * C.pl;
+            z[a] = (g[C.r0 + C.i] + g[C.r0 + C.i1]) + (g[C.r1 + C.i] + g[C.r1 + C.i1]);
+        }
+    };
+    double lo[3], hi[3];
+    corner_sum(C.k0, lo);
+    for (int k = C.k0; k < C.k1; k++) {
+        corner_sum(k + 1, hi);
+        double u[3], adv[6], ss[6];
+#pragma unroll
+        for (int a = 0; a < 3; a++) {
+            u[a] = 0.125 * (lo[a] + hi[a]);
+            lo[a] = hi[a];
+        }
+        stress_advection(sig, nc, p.nx, C.pl, p.nz, C.j, k, col, ix, jy, u, adv);
+        const long q = k * C.pl + col;
+#pragma unroll
+        for (int n = 0; n < 6; n++) ss[n] = sig_star[n * nc + q];
+#pragma unroll
+        for (int n = 0; n < 6; n++) sig_star[n * nc + q] = fma(-w.dt2h, adv[n], ss[n]);
     }
-    double adv[6], ss[6];
-    stress_advection(p, sig, nc, i, j, k, u, 0.5 / p.h, adv);
-    const long q = (long)k * pl + (long)j * nx + i;
-#pragma unroll
-    for (int n = 0; n < 6; n++) ss[n] = sig_star[n * nc + q];
-#pragma unroll
-    for (int n = 0; n < 6; n++) sig_star[n * nc + q] = ss[n] - p.dt * adv[n];
 }
 
 // Eq. (24) at interior corners (k = 1 .. nz-1):
 //   v' = v + dt (-(v.grad) v + div sigma / rho + kappa lap v),
 // the divergence the corner version of Eq. (31) over the 8 cells around the
-// corner, the Laplacian Eq. (32) along each axis, ENO advection with the
-// corner's own velocity; corners up to two planes beyond a wall reflect v
-// through the wall value, v(-m) = 2 v(0) - v(m)
-__global__ void k_explicit_velocity(StepParams p, double inv_rho, double kappa,
-                                    const double *__restrict__ v, const double *__restrict__ sig,
-                                    double *__restrict__ v_new, long nc) {
+// corner, the Laplacian Eq. (32) along each axis (the second differences the
+// ENO test forms anyway), ENO advection with the corner's own velocity;
+// corners up to two planes beyond a wall reflect v through the wall value,
+// v(-m) = 2 v(0) - v(m)
+struct VelConst {
+    double div, lap, adv;  // dt / (4 h rho);  dt kappa / h^2;  dt / (2 h)
+};
+__global__ void __launch_bounds__(128)
+    k_explicit_velocity(StepParams p, VelConst w, int chunk, const double *__restrict__ v,
+                        const double *__restrict__ sig, double *__restrict__ v_new, long nc) {
     const int nx = p.nx, ny = p.ny, nz = p.nz;
-    const int i = blockIdx.x * BX + threadIdx.x, j = blockIdx.y * BY + threadIdx.y;
-    const int k = blockIdx.z + 1;
-    if (i >= nx || j >= ny) return;
+    const int col = blockIdx.x * blockDim.x + threadIdx.x, j = col / nx, i = col - j * nx;
+    if (j >= ny) return;
+    const int k0 = 1 + blockIdx.y * chunk;
+    const int k1 = k0 + chunk < nz ? k0 + chunk : nz;
     const long pl = (long)nx * ny, cs = (long)(nz + 1) * pl;
-    const double h = p.h, inv_h2 = 1.0 / (p.h * p.h), inv2h = 0.5 / p.h;
     const int im = i ? i - 1 : nx - 1, jm = j ? j - 1 : ny - 1;
-    const int ip = i + 1 < nx ? i + 1 : 0, jp = j + 1 < ny ? j + 1 : 0;
-    const long node = (long)k * pl + (long)j * nx + i;
+    const long rj0 = (long)jm * nx, rj1 = (long)j * nx;
     int ix[5], jy[5];
+    around(i, nx, ix);
+    around(j, ny, jy);
+    // the z differences are taken column by column (the layer sums of the
+    // right-hand side would cost 9 instructions less and 3% more rounding)
+    double flo[3][2][2], fhi[3][2][2], xlo[3], xhi[3];
+    div_parts(sig, nc, (long)(k0 - 1) * pl, rj0, rj1, im, i, xlo, flo);
+    for (int k = k0; k < k1; k++) {
+        div_parts(sig, nc, (long)k * pl, rj0, rj1, im, i, xhi, fhi);
+        const long node = (long)k * pl + col;
+        const double u[3] = {v[node], v[cs + node], v[2 * cs + node]};
+        const bool inner = k >= 2 && k <= nz - 2;
 #pragma unroll
-    for (int m = 0; m < 5; m++) {
-        int a = i + m - 2, b = j + m - 2;
-        ix[m] = a < 0 ? a + nx : (a >= nx ? a - nx : a);
-        jy[m] = b < 0 ? b + ny : (b >= ny ? b - ny : b);
-    }
-    const double u[3] = {v[node], v[cs + node], v[2 * cs + node]};
-    const int comp[3][3] = {{0, 5, 4}, {5, 1, 3}, {4, 3, 2}};
-    const long c0 = (long)(k - 1) * pl, c1 = (long)k * pl;
-    const long rm = (long)jm * nx, r0 = (long)j * nx;
+        for (int a = 0; a < 3; a++) {
+            const double *g = v + a * cs;
+            double fx[5], fy[5], fz[5], cx, cy, cz;
 #pragma unroll
-    for (int a = 0; a < 3; a++) {
-        const double *fx = sig + comp[a][0] * nc, *fy = sig + comp[a][1] * nc,
-                     *fz = sig + comp[a][2] * nc;
-        const double div =
-            (((fx[c0 + rm + i] - fx[c0 + rm + im]) + (fx[c0 + r0 + i] - fx[c0 + r0 + im])) +
-             ((fx[c1 + rm + i] - fx[c1 + rm + im]) + (fx[c1 + r0 + i] - fx[c1 + r0 + im])) +
-             ((fy[c0 + r0 + im] - fy[c0 + rm + im]) + (fy[c0 + r0 + i] - fy[c0 + rm + i])) +
-             ((fy[c1 + r0 + im] - fy[c1 + rm + im]) + (fy[c1 + r0 + i] - fy[c1 + rm + i])) +
-             ((fz[c1 + rm + im] - fz[c0 + rm + im]) + (fz[c1 + rm + i] - fz[c0 + rm + i])) +
-             ((fz[c1 + r0 + im] - fz[c0 + r0 + im]) + (fz[c1 + r0 + i] - fz[c0 + r0 + i]))) *
-            (0.25 / h);
-        const double *g = v + a * cs;
-        const double w0 = g[node];
-        const double lap = ((g[node - i + ip] - 2.0 * w0 + g[node - i + im]) +
-                            (g[node - (long)j * nx + (long)jp * nx] - 2.0 * w0 +
-                             g[node - (long)j * nx + (long)jm * nx]) +
-                            (g[node + pl] - 2.0 * w0 + g[node - pl])) *
-                           inv_h2;
-        double fxl[5], fyl[5], fzl[5];
+            for (int m = 0; m < 5; m++) {
+                fx[m] = g[k * pl + rj1 + ix[m]];
+                fy[m] = g[k * pl + (long)jy[m] * nx + i];
+            }
+            if (inner) {
 #pragma unroll
-        for (int m = 0; m < 5; m++) {
-            fxl[m] = g[(long)k * pl + (long)j * nx + ix[m]];
-            fyl[m] = g[(long)k * pl + (long)jy[m] * nx + i];
-            const int kk = k + m - 2;
-            const long col = (long)j * nx + i;
-            if (kk < 0)
-                fzl[m] = 2.0 * g[col] - g[(long)(-kk) * pl + col];
-            else if (kk > nz)
-                fzl[m] = 2.0 * g[(long)nz * pl + col] - g[(long)(2 * nz - kk) * pl + col];
-            else
-                fzl[m] = g[(long)kk * pl + col];
+                for (int m = 0; m < 5; m++) fz[m] = g[(k + m - 2) * pl + col];
+            } else {
+#pragma unroll
+                for (int m = 0; m < 5; m++) {
+                    const int kk = k + m - 2;
+                    if (kk < 0)
+                        fz[m] = 2.0 * g[col] - g[-kk * pl + col];
+                    else if (kk > nz)
+                        fz[m] = 2.0 * g[nz * pl + col] - g[(2 * nz - kk) * pl + col];
+                    else
+                        fz[m] = g[kk * pl + col];
+                }
+            }
+            double t = u[0] * eno_2h(fx[0], fx[1], fx[2], fx[3], fx[4], u[0], cx);
+            t = fma(u[1], eno_2h(fy[0], fy[1], fy[2], fy[3], fy[4], u[1], cy), t);
+            t = fma(u[2], eno_2h(fz[0], fz[1], fz[2], fz[3], fz[4], u[2], cz), t);
+            const double div = (xlo[a] + xhi[a]) +
+                               (((fhi[a][0][0] - flo[a][0][0]) + (fhi[a][0][1] - flo[a][0][1])) +
+                                ((fhi[a][1][0] - flo[a][1][0]) + (fhi[a][1][1] - flo[a][1][1])));
+            const double lap = (cx + cy) + cz;
+            v_new[a * cs + node] =
+                fx[2] + fma(w.lap, lap, fma(w.div, div, -w.adv * t));
         }
-        const double adv = u[0] * eno_d(fxl[0], fxl[1], fxl[2], fxl[3], fxl[4], u[0], inv2h) +
-                           u[1] * eno_d(fyl[0], fyl[1], fyl[2], fyl[3], fyl[4], u[1], inv2h) +
-                           u[2] * eno_d(fzl[0], fzl[1], fzl[2], fzl[3], fzl[4], u[2], inv2h);
-        v_new[a * cs + node] = w0 + p.dt * (-adv + div * inv_rho + kappa * lap);
+#pragma unroll
+        for (int a = 0; a < 3; a++) {
+            xlo[a] = xhi[a];
+#pragma unroll
+            for (int y = 0; y < 2; y++)
+#pragma unroll
+                for (int e = 0; e < 2; e++) flo[a][y][e] = fhi[a][y][e];
+        }
     }
 }
 
@@ -755,7 +804,8 @@ cudaError_t stress_correct(const StepParams &p, const double *v, const double *s
 cudaError_t stress_advect(const StepParams &p, const double *v, const double *sig,
                           double *sig_star, cudaStream_t s) {
     const long nc = (long)p.nx * p.ny * p.nz;
-    k_stress_advect<<<cell_grid(p.nx, p.ny, p.nz), kBlock, 0, s>>>(p, v, sig, sig_star, nc);
+    const March m = march((long)p.nx * p.ny, p.nz);
+    k_stress_advect<<<m.grid, m.threads, 0, s>>>(p, cell_const(p), m.chunk, v, sig, sig_star, nc);
     count_launch();
     return cudaGetLastError();
 }
@@ -781,8 +831,9 @@ cudaError_t explicit_stress(const StepParams &p, const double *v, const double *
                             const double *chi, double *sig_new, double *dpl, double *sbar,
                             cudaStream_t s) {
     const long nc = (long)p.nx * p.ny * p.nz;
-    k_explicit_stress<<<cell_grid(p.nx, p.ny, p.nz), kBlock, 0, s>>>(p, stz_const(p), v, sig, chi,
-                                                                     sig_new, dpl, sbar, nc);
+    const March m = march((long)p.nx * p.ny, p.nz);
+    k_explicit_stress<<<m.grid, m.threads, 0, s>>>(p, cell_const(p), stz_const(p), m.chunk, v, sig,
+                                                   chi, sig_new, dpl, sbar, nc);
     count_launch();
     return cudaGetLastError();
 }
@@ -791,8 +842,9 @@ cudaError_t explicit_velocity(const StepParams &p, double rho, double kappa, con
                               const double *sig, double *v_new, cudaStream_t s) {
     const long nc = (long)p.nx * p.ny * p.nz;
     if (p.nz < 2) return cudaSuccess;
-    k_explicit_velocity<<<cell_grid(p.nx, p.ny, p.nz - 1), kBlock, 0, s>>>(p, 1.0 / rho, kappa, v,
-                                                                          sig, v_new, nc);
+    const March m = march((long)p.nx * p.ny, p.nz - 1);
+    const VelConst w{p.dt * (0.25 / p.h) / rho, p.dt * kappa / (p.h * p.h), p.dt * (0.5 / p.h)};
+    k_explicit_velocity<<<m.grid, m.threads, 0, s>>>(p, w, m.chunk, v, sig, v_new, nc);
     count_launch();
     return cudaGetLastError();
 }
