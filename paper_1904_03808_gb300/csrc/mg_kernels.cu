@@ -43,20 +43,13 @@ __device__ __forceinline__ int colmap(int i, int nx, int split) {
     return split ? ((i & 1) * (nx >> 1) + (i >> 1)) : i;
 }
 
-// value of x at plane kk; with WO ("walls only") interior planes read as zero
-template <typename T, bool WO>
-__device__ __forceinline__ T ldx(const T *x, long idx, int kk, int nz) {
-    if (WO && kk > 0 && kk < nz) return T(0);
-    return x[idx];
-}
-
 // o_a = sum over the 18 non-centre offsets of S_d[a][b] x_b(p + d)
 //   = -( lp x_a(+-e_a) + x_a(+-e_b, b != a) + kq sum_{b!=a} M_ab[x_b] ),
 // M_ab[g] = g(+a,+b) - g(+a,-b) - g(-a,+b) + g(-a,-b)  (4-point mixed difference)
-template <typename T, bool WO>
+template <typename T>
 __device__ __forceinline__ void fine_off(const T *x, const Dims &d, int i0, int j, int k, T lp,
                                          T kq, T o[3], int split = 0) {
-    const int nx = d.nx, ny = d.ny, nz = d.nz;
+    const int nx = d.nx, ny = d.ny;
     const long ps = (long)nx * ny;
     const int im = colmap(i0 ? i0 - 1 : nx - 1, nx, split),
               ip = colmap((i0 + 1 < nx) ? i0 + 1 : 0, nx, split);
@@ -65,9 +58,9 @@ __device__ __forceinline__ void fine_off(const T *x, const Dims &d, int i0, int 
     const long pc = (long)k * ps, pm = pc - ps, pp = pc + ps;
     const long r0 = (long)j * nx, rm = (long)jm * nx, rp = (long)jp * nx;
     const T *x0 = x, *x1 = x + d.cs, *x2 = x + 2 * d.cs;
-#define XC(g, r, c) ldx<T, WO>(g, pc + (r) + (c), k, nz)
-#define XM(g, r, c) ldx<T, WO>(g, pm + (r) + (c), k - 1, nz)
-#define XP(g, r, c) ldx<T, WO>(g, pp + (r) + (c), k + 1, nz)
+#define XC(g, r, c) (g)[pc + (r) + (c)]
+#define XM(g, r, c) (g)[pm + (r) + (c)]
+#define XP(g, r, c) (g)[pp + (r) + (c)]
     const T a0 = lp * (XC(x0, r0, im) + XC(x0, r0, ip)) + (XC(x0, rm, i) + XC(x0, rp, i)) +
                  (XM(x0, r0, i) + XP(x0, r0, i));
     const T a1 = lp * (XC(x1, rm, i) + XC(x1, rp, i)) + (XC(x1, r0, im) + XC(x1, r0, ip)) +
@@ -143,7 +136,7 @@ __global__ void k_gs_fine(Dims d, Fine<T> f, const T *__restrict__ b, T *x, int 
     int i, j, k;
     if (!colour_node(colour, hx, hy, i, j, k)) return;
     T o[3];
-    fine_off<T, false>(x, d, i, j, k, f.lp, f.kq, o);
+    fine_off<T>(x, d, i, j, k, f.lp, f.kq, o);
     const long p = ((long)k * d.ny + j) * d.nx + i;
     const T u0 = (b[p] - o[0]) * f.dinv;
     const T u1 = (b[p + d.cs] - o[1]) * f.dinv;
@@ -171,7 +164,7 @@ __global__ void k_res_fine(Dims d, Fine<T> f, const T *__restrict__ b, const T *
     int i, j, k;
     if (!node_ijk(d, i, j, k)) return;
     T o[3];
-    fine_off<T, false>(x, d, i, j, k, f.lp, f.kq, o, split);
+    fine_off<T>(x, d, i, j, k, f.lp, f.kq, o, split);
     const long p = ((long)k * d.ny + j) * d.nx + colmap(i, d.nx, split);
 #pragma unroll
     for (int a = 0; a < 3; a++) r[p + a * d.cs] = b[p + a * d.cs] - (f.d0 * x[p + a * d.cs] + o[a]);
@@ -208,62 +201,6 @@ __device__ double block_sum(double v) {
     v = (threadIdx.x < (unsigned)nw) ? sh[threadIdx.x] : 0.0;
     if (w == 0) v = warp_sum(v);
     return v;
-}
-
-template <bool WO>
-__global__ void __launch_bounds__(kRedThreads)
-    k_res_norm_fine64(Dims d, Fine<double> f, const double *__restrict__ b,
-                      const double *__restrict__ x, float *__restrict__ r32, double out_scale,
-                      double *__restrict__ partials, int split32) {
-    // rows (j, k) are dealt to blocks in a fixed order, columns to threads,
-    // so the partial sums do not depend on timing
-    double acc = 0.0;
-    const int nrows = d.ny * (d.nz - 1);
-    for (int row = blockIdx.x; row < nrows; row += gridDim.x) {
-        const int k = row / d.ny + 1, j = row - (k - 1) * d.ny;
-        if (WO && k != 1 && k != d.nz - 1) {
-            // away from the walls the lifted right-hand side is b itself
-            const long p0 = ((long)k * d.ny + j) * d.nx;
-            for (int i = threadIdx.x; i < d.nx; i += blockDim.x)
-#pragma unroll
-                for (int a = 0; a < 3; a++) {
-                    const double r = b[p0 + i + a * d.cs];
-                    acc += r * r;
-                }
-            continue;
-        }
-        for (int i = threadIdx.x; i < d.nx; i += blockDim.x) {
-            double o[3];
-            fine_off<double, WO>(x, d, i, j, k, f.lp, f.kq, o);
-            const long p = ((long)k * d.ny + j) * d.nx + i;
-#pragma unroll
-            for (int a = 0; a < 3; a++) {
-                const double xc = WO ? 0.0 : x[p + a * d.cs];
-                const double r = b[p + a * d.cs] - (f.d0 * xc + o[a]);
-                acc += r * r;
-                if (r32) r32[p - i + colmap(i, d.nx, split32) + a * d.cs] = (float)(r * out_scale);
-            }
-        }
-    }
-    const double s = block_sum(acc);
-    if (threadIdx.x == 0) partials[blockIdx.x] = s;
-}
-
-__global__ void __launch_bounds__(kRedThreads)
-    k_sumsq(Dims d, const double *__restrict__ r, double *__restrict__ partials) {
-    double acc = 0.0;
-    const int nrows = d.ny * (d.nz - 1);
-    for (int row = blockIdx.x; row < nrows; row += gridDim.x) {
-        const long p0 = (long)(row + d.ny) * d.nx;  // interior rows start at plane 1
-        for (int i = threadIdx.x; i < d.nx; i += blockDim.x)
-#pragma unroll
-            for (int a = 0; a < 3; a++) {
-                const double v = r[p0 + i + a * d.cs];
-                acc += v * v;
-            }
-    }
-    const double s = block_sum(acc);
-    if (threadIdx.x == 0) partials[blockIdx.x] = s;
 }
 
 __global__ void __launch_bounds__(1024) k_sum_partials(const double *__restrict__ partials,
@@ -590,10 +527,6 @@ static cudaError_t res_coarse_t(const Dims &d, const Coarse<T> &c, const T *b, c
     return cudaSuccess;
 }
 
-cudaError_t residual_fine(const Dims &d, const Fine<double> &f, const double *b, const double *x,
-                          double *r, cudaStream_t s) {
-    return res_fine_t(d, f, b, x, r, s, 0);
-}
 cudaError_t residual_fine(const Dims &d, const Fine<float> &f, const float *b, const float *x,
                           float *r, cudaStream_t s, int split) {
     // whole-row strips where the rows fit (smoother_rows.cu), else one
@@ -617,25 +550,6 @@ cudaError_t residual_coarse(const Dims &d, const Coarse<double> &c, const double
 cudaError_t residual_coarse(const Dims &d, const Coarse<float> &c, const float *b, const float *x,
                             float *r, cudaStream_t s) {
     return res_coarse_t(d, c, b, x, r, s);
-}
-
-cudaError_t residual_norm_fine64(const Dims &d, const Fine<double> &f, const double *b,
-                                 const double *x, bool wall_only, float *r32, double out_scale,
-                                 double *partials, cudaStream_t s, int split32) {
-    if (wall_only)
-        k_res_norm_fine64<true><<<kRedBlocks, kRedThreads, 0, s>>>(d, f, b, x, r32, out_scale,
-                                                                   partials, split32);
-    else
-        k_res_norm_fine64<false><<<kRedBlocks, kRedThreads, 0, s>>>(d, f, b, x, r32, out_scale,
-                                                                    partials, split32);
-    count_launch();
-    return cudaGetLastError();
-}
-
-cudaError_t sumsq(const Dims &d, const double *r, double *partials, cudaStream_t s) {
-    k_sumsq<<<kRedBlocks, kRedThreads, 0, s>>>(d, r, partials);
-    count_launch();
-    return cudaGetLastError();
 }
 
 cudaError_t sum_partials(const double *partials, double *out, cudaStream_t s) {

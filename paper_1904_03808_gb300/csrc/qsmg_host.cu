@@ -85,7 +85,8 @@ struct mg_ctx {
     SmallPlan<double> s64;
     SmallPlan<float> s32;
     int top64, top32;
-    double *partials, *dsum, *hsum;
+    double *partials, *dsum, *hsum;  // dsum, hsum: lifted norm, residual norm (squared)
+    NormBuf norms;
     // cross-CTA state of the fused finest-level sweep (when it applies)
     SweepSync sync;
     bool has_sync;
@@ -353,26 +354,29 @@ mg_status sync_error(mg_ctx *ctx) {
     return MG_ERR_CUDA;
 }
 
-mg_status read_sum(mg_ctx *ctx, double *out) {
-    CK(sum_partials(ctx->partials, ctx->dsum, ctx->st));
-    CK(cudaMemcpyAsync(ctx->hsum, ctx->dsum, sizeof(double), cudaMemcpyDeviceToHost, ctx->st));
+// dsum to the host, with the fused sweep's error word
+mg_status read_sums(mg_ctx *ctx) {
+    CK(cudaMemcpyAsync(ctx->hsum, ctx->dsum, 2 * sizeof(double), cudaMemcpyDeviceToHost, ctx->st));
     if (ctx->has_sync)
         CK(cudaMemcpyAsync(ctx->herr, ctx->sync.err, sizeof(int), cudaMemcpyDeviceToHost, ctx->st));
     CK(cudaStreamSynchronize(ctx->st));
-    *out = ctx->hsum[0];
     CKS(sync_error(ctx));
     return prof_drain(ctx);
 }
 
-// ||b - A v||_2 on the finest level (FP64), optionally writing
-// float(r * out_scale) into r32; wall_only gives ||b_lifted||_2
-mg_status fine_resnorm(mg_ctx *ctx, const double *b, const double *v, bool wall_only, float *r32,
-                       double out_scale, double *norm, int split32 = 0) {
-    CK(residual_norm_fine64(ctx->L[0], ctx->f64, b, v, wall_only, r32, out_scale, ctx->partials,
-                            ctx->st, split32));
-    double s2;
-    CKS(read_sum(ctx, &s2));
-    *norm = sqrt(s2);
+// ||b - A v||_2 on the finest level (FP64), squared into slot 1 - from of the
+// sums; r32 (optional) receives the residual scaled by the exponent of the norm
+// in slot `from`.  With lifted, ||b_lifted||_2 goes to slot `from` first, in
+// the same round trip to the host.
+mg_status fine_resnorm(mg_ctx *ctx, const double *b, const double *v, float *r32, int from,
+                       double *norm, double *lifted = nullptr) {
+    double *const s = ctx->dsum;
+    if (lifted) CK(lifted_norm(ctx->L[0], ctx->f64, b, v, ctx->norms, s + from, ctx->st));
+    CK(residual_norm(ctx->L[0], ctx->f64, b, v, r32, ctx->split0, s + from, ctx->norms,
+                     s + 1 - from, ctx->st));
+    CKS(read_sums(ctx));
+    if (lifted) *lifted = sqrt(ctx->hsum[from]);
+    *norm = sqrt(ctx->hsum[1 - from]);
     return MG_OK;
 }
 
@@ -556,10 +560,9 @@ template <typename T>
 mg_status residual_level(mg_ctx *ctx, int l, const T *b, const T *x, T *r) {
     const Dims &d = ctx->L[l];
     // the coarsest level may have odd sizes, and is never smoothed
-    const bool strip = l + 1 < ctx->nlev && strip_fits(d, l == 0);
+    const bool strip = l + 1 < ctx->nlev && strip_fits(d, false);
     if (l == 0)
-        CK(strip ? residual_strip(d, ctx->f64, b, x, r, ctx->st)
-                 : residual_fine(d, Bufs<T>::fine(ctx), b, x, r, ctx->st));
+        CK(residual_march(d, ctx->f64, b, x, r, ctx->st));
     else
         CK(strip ? residual_strip(d, ctx->c64[l], b, x, r, ctx->st)
                  : residual_coarse(d, Bufs<T>::coarse(ctx, l), b, x, r, ctx->st));
@@ -725,7 +728,7 @@ mg_status check_ctx(mg_ctx *ctx) {
 
 mg_status solve_fp64(mg_ctx *ctx, const double *b, double *v, double tol, mg_stats *st) {
     double bn, rn;
-    CKS(fine_resnorm(ctx, b, v, true, nullptr, 0.0, &bn));
+    CKS(fine_resnorm(ctx, b, v, nullptr, 0, &rn, &bn));
     st->bnorm = bn;
     if (bn == 0.0) {
         CK(zero_interior(ctx->L[0], v, ctx->st));
@@ -733,7 +736,6 @@ mg_status solve_fp64(mg_ctx *ctx, const double *b, double *v, double tol, mg_sta
         st->resid_hist[0] = 0.0;
         return MG_OK;
     }
-    CKS(fine_resnorm(ctx, b, v, false, nullptr, 0.0, &rn));
     double rel = rn / bn;
     st->resid_hist[0] = rel;
     int it = 0;
@@ -754,15 +756,16 @@ mg_status solve_fp64(mg_ctx *ctx, const double *b, double *v, double tol, mg_sta
         }
         CKS(vcycle<double>(ctx, 0, b, v));
         it++;
-        CKS(fine_resnorm(ctx, b, v, false, nullptr, 0.0, &rn));
+        CKS(fine_resnorm(ctx, b, v, nullptr, 0, &rn));
         rel = rn / bn;
         if (it < MG_HIST) st->resid_hist[it] = rel;
     }
 }
 
 // FP32 V-cycles on the correction equation inside FP64 iterative refinement:
-//   r = b - A v (FP64, stored as float(r / s)), e ~ A^{-1} r by FP32 V-cycles
-//   from e = 0, v += s e.
+//   r = b - A v (FP64, stored as float(r / s), s the power of two below the
+//   norm of the previous residual), e ~ A^{-1} r by FP32 V-cycles from e = 0,
+//   v += s e.
 // With opts.inner_cycles > 0 every refinement step runs that many cycles.
 // With 0 the count is chosen per step: enough cycles to bring the FP64
 // residual to tol at the contraction factor observed so far (initially 0.4),
@@ -817,7 +820,8 @@ mg_status inner_cycles(mg_ctx *ctx, int n) {
 
 mg_status solve_mixed(mg_ctx *ctx, const double *b, double *v, double tol, mg_stats *st) {
     double bn, rn;
-    CKS(fine_resnorm(ctx, b, v, true, nullptr, 0.0, &bn));
+    int from = 0;  // the sum whose exponent scales the next FP32 residual
+    CKS(fine_resnorm(ctx, b, v, ctx->b32[0], from, &rn, &bn));
     st->bnorm = bn;
     if (bn == 0.0) {
         CK(zero_interior(ctx->L[0], v, ctx->st));
@@ -825,8 +829,7 @@ mg_status solve_mixed(mg_ctx *ctx, const double *b, double *v, double tol, mg_st
         st->resid_hist[0] = 0.0;
         return MG_OK;
     }
-    double scale = bn;
-    CKS(fine_resnorm(ctx, b, v, false, ctx->b32[0], 1.0 / scale, &rn, ctx->split0));
+    double scale = ldexp(1.0, norm_exponent(ctx->hsum[from]));
     double rel = rn / bn;
     st->resid_hist[0] = rel;
     int outer = 0, cycles = 0;
@@ -853,8 +856,9 @@ mg_status solve_mixed(mg_ctx *ctx, const double *b, double *v, double tol, mg_st
         CK(axpy_f32(ctx->L[0], scale, ctx->x32[0], v, ctx->st, ctx->split0));
         outer++;
         cycles += n;
-        scale = rn;
-        CKS(fine_resnorm(ctx, b, v, false, ctx->b32[0], 1.0 / scale, &rn, ctx->split0));
+        from = 1 - from;
+        scale = ldexp(1.0, norm_exponent(ctx->hsum[from]));
+        CKS(fine_resnorm(ctx, b, v, ctx->b32[0], from, &rn));
         const double rel_new = rn / bn;
         if (rel_new > 0.0 && rel_new < rel) {
             const double k = pow(rel_new / rel, 1.0 / n);
@@ -1080,8 +1084,13 @@ mg_status mg_setup(const mg_grid *grid, const mg_moduli *moduli, const mg_bc *bc
         ALLOC(ctx->xs32[l], n);
     }
     ALLOC(ctx->Ainv, Ainv.size());
-    ALLOC(ctx->partials, (size_t)kRedBlocks);
-    ALLOC(ctx->dsum, (size_t)1);
+    {
+        const long nb = norm_blocks(ctx->L[0]);
+        ALLOC(ctx->partials, (size_t)(nb > kRedBlocks ? nb : kRedBlocks));
+        ALLOC(ctx->norms.count, (size_t)1);
+        ctx->norms.partials = ctx->partials;
+    }
+    ALLOC(ctx->dsum, (size_t)2);
     {
         const size_t nc = (size_t)nx * ny * nz;
         ALLOC(ctx->sig_star, 6 * nc);
@@ -1114,7 +1123,7 @@ mg_status mg_setup(const mg_grid *grid, const mg_moduli *moduli, const mg_bc *bc
         s = MG_ERR_CUDA;
         goto fail;
     }
-    if (cudaMallocHost((void **)&ctx->hsum, sizeof(double)) != cudaSuccess) {
+    if (cudaMallocHost((void **)&ctx->hsum, 2 * sizeof(double)) != cudaSuccess) {
         set_err("cudaMallocHost failed");
         s = MG_ERR_OOM;
         goto fail;

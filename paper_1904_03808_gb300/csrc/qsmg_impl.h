@@ -126,7 +126,7 @@ cudaError_t gs_colour_coarse(const Dims &d, const Coarse<double> &c, const doubl
 cudaError_t gs_colour_coarse(const Dims &d, const Coarse<float> &c, const float *b, float *x,
                              int colour, cudaStream_t s);
 
-// FP64 sweeps and residuals on row strips (strip64.cu).  strip_fits: whether a
+// FP64 sweeps and coarse residuals on row strips (strip64.cu).  strip_fits: whether a
 // level of these dimensions takes them (finest: the 19-point operator).
 // One 8-colour sweep vin -> vout, interior planes only; wall: an array that
 // holds the wall planes.  The longest rows: on 128-wide fine rows the repeated
@@ -143,9 +143,7 @@ cudaError_t gs_sweep_strip(const Dims &d, const Fine<double> &f, const double *b
 cudaError_t gs_sweep_strip(const Dims &d, const Coarse<double> &c, const double *b,
                            const double *vin, const double *wall, double *vout, bool descending,
                            cudaStream_t s);
-// r = b - A x (interior), r walls zero
-cudaError_t residual_strip(const Dims &d, const Fine<double> &f, const double *b,
-                           const double *x, double *r, cudaStream_t s);
+// coarse levels: r = b - A x (interior), r walls zero
 cudaError_t residual_strip(const Dims &d, const Coarse<double> &c, const double *b,
                            const double *x, double *r, cudaStream_t s);
 
@@ -219,8 +217,6 @@ cudaError_t gs_sweep_coarse_tiled(const Dims &d, const Coarse<float> &c, const f
                                   const float *vin, float *vout, bool descending, cudaStream_t s);
 
 // r = b - A x (interior), r walls zero
-cudaError_t residual_fine(const Dims &d, const Fine<double> &f, const double *b, const double *x,
-                          double *r, cudaStream_t s);
 cudaError_t residual_fine(const Dims &d, const Fine<float> &f, const float *b, const float *x,
                           float *r, cudaStream_t s, int split = 0);
 cudaError_t residual_coarse(const Dims &d, const Coarse<double> &c, const double *b,
@@ -228,15 +224,37 @@ cudaError_t residual_coarse(const Dims &d, const Coarse<double> &c, const double
 cudaError_t residual_coarse(const Dims &d, const Coarse<float> &c, const float *b, const float *x,
                             float *r, cudaStream_t s);
 
-// FP64 fine residual with the sum of squares into partials[kRedBlocks];
-// wall_only treats interior x as zero (lifted right-hand side);
-// r32 (optional) receives float(r * out_scale), in parity-split column order
-// if split32
-cudaError_t residual_norm_fine64(const Dims &d, const Fine<double> &f, const double *b,
-                                 const double *x, bool wall_only, float *r32, double out_scale,
-                                 double *partials, cudaStream_t s, int split32 = 0);
-// sum of squares of a level vector's interior into partials
-cudaError_t sumsq(const Dims &d, const double *r, double *partials, cudaStream_t s);
+// FP64 finest-level residual and norms (residual64.cu).  A norm kernel's last
+// block adds the partial sums of all blocks in a fixed order into *sum;
+// partials has norm_blocks(d) entries, count starts at zero.
+struct NormBuf {
+    double *partials;
+    unsigned *count;
+};
+// exponent e of the power of two 2^e <= sqrt(s2) < 2^(e+1) up to rounding, by
+// which a residual of squared norm s2 is scaled for FP32; 0 if s2 is zero,
+// subnormal or not finite
+__host__ __device__ inline int norm_exponent(double s2) {
+    union {
+        double d;
+        long long i;
+    } u;
+    u.d = s2;
+    const int ex = (int)((u.i >> 52) & 0x7ff);
+    return ex == 0 || ex == 0x7ff ? 0 : (ex - 1023) >> 1;
+}
+long norm_blocks(const Dims &d);
+// r = b - A x (interior), r walls zero
+cudaError_t residual_march(const Dims &d, const Fine<double> &f, const double *b, const double *x,
+                           double *r, cudaStream_t s);
+// *sum = |b - A x|^2; r32 (optional) receives float(r 2^-norm_exponent(*scale2))
+// (scale2: device), in parity-split column order if split
+cudaError_t residual_norm(const Dims &d, const Fine<double> &f, const double *b, const double *x,
+                          float *r32, int split, const double *scale2, const NormBuf &nb,
+                          double *sum, cudaStream_t s);
+// *sum = |b - A (x on the walls, zero inside)|^2, the lifted right-hand side
+cudaError_t lifted_norm(const Dims &d, const Fine<double> &f, const double *b, const double *x,
+                        const NormBuf &nb, double *sum, cudaStream_t s);
 // out[0] = sum of partials[0..kRedBlocks)
 cudaError_t sum_partials(const double *partials, double *out, cudaStream_t s);
 

@@ -66,7 +66,7 @@ extern "C" mg_status mg_residual_restrict_static(const mg_grid *grid, const mg_m
     cudaStream_t st = (cudaStream_t)stream;
     // the residual kernel writes every interior value of r and zeroes its wall
     // planes, so nothing of the previous call's contents is read
-    e = residual_fine(d, f, b, x, r, st);
+    e = residual_march(d, f, b, x, r, st);
     if (e == cudaSuccess) e = cudaMemsetAsync(bc, 0, 3 * (size_t)dc.cs * sizeof(double), st);
     if (e == cudaSuccess) e = restrict_fw(d, r, bc, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);

@@ -1,5 +1,5 @@
-// strip64.cu -- FP64 Gauss-Seidel sweeps and residuals on row strips of one
-// plane, for levels whose rows are short enough for shared memory.
+// strip64.cu -- FP64 Gauss-Seidel sweeps (and coarse residuals) on row strips of
+// one plane, for levels whose rows are short enough for shared memory.
 //
 // The FP64 pipe takes a warp instruction every 16 clocks of an SM and every 64
 // clocks of one scheduler, however many lanes are active, so an FP64 sweep is
@@ -57,24 +57,7 @@ struct CoarseStrip {
     Coarse<double> c;
 };
 
-// residual of the node at window row jj, columns xm, x0, xp (offsets),
-// summed so that the centre terms cancel against their neighbours first
-__device__ __forceinline__ void resid(const FineStrip &op, const double *P, const double *D,
-                                      const double *R, const double *, const double *, int w,
-                                      int jj, int xm, int x0, int xp, double o[3]) {
-    const double lp = op.f.lp, kq = op.f.kq, d0 = op.f.d0;
-    const double *p = P + jj * w, *pm = p - w, *pp = p + w, *d = D + jj * w, *dm = d - w,
-                 *dp = d + w, *r = R + jj * w + x0;
-    const double m01 = ((pp[xp + 1] - pm[xp + 1]) - (pp[xm + 1] - pm[xm + 1])) +
-                       (d[xp + 2] - d[xm + 2]);
-    const double m10 = ((pp[xp] - pm[xp]) - (pp[xm] - pm[xm])) + (dp[x0 + 2] - dm[x0 + 2]);
-    const double m2 = (d[xp] - d[xm]) + (dp[x0 + 1] - dm[x0 + 1]);
-    o[0] = ((lp * (p[xm] + p[xp]) - d0 * p[x0]) + (pm[x0] + pp[x0]) + r[0]) + kq * m01;
-    o[1] = ((lp * (pm[x0 + 1] + pp[x0 + 1]) - d0 * p[x0 + 1]) + (p[xm + 1] + p[xp + 1]) + r[1]) +
-           kq * m10;
-    o[2] = ((r[2] - d0 * p[x0 + 2]) + (p[xm + 2] + p[xp + 2]) + (pm[x0 + 2] + pp[x0 + 2])) +
-           kq * m2;
-}
+// residual of the node at window row jj, columns xm, x0, xp (offsets)
 __device__ __forceinline__ void resid(const CoarseStrip &op, const double *P, const double *,
                                       const double *R, const double *U, const double *V, int w,
                                       int jj, int xm, int x0, int xp, double o[3]) {
@@ -211,7 +194,7 @@ __global__ void __launch_bounds__(NT, 2)
         }
         __syncthreads();
     }
-    if (RES) {
+    if constexpr (RES) {
         double *out = vout + k * g.ps;
         for (int e = tid; e < TY * nx; e += NT) {
             const int jt = fdiv(e, g.mnx), i = e - jt * nx, jj = 1 + jt, y = y0 + jt;
@@ -306,24 +289,19 @@ cudaError_t sweep(const Dims &d, const OP &op, const double *b, const double *vi
     return launch<OP, 1, false>(d, op, b, vin, vout, wall, vout, 2, ne, s);
 }
 
-template <class OP>
-cudaError_t attrs() {
-    cudaError_t e = cudaFuncSetAttribute(k_gs_strip<OP, 0, false>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, kStripSmem);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_gs_strip<OP, 1, false>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, kStripSmem);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_gs_strip<OP, 0, true>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, kStripSmem);
-    return e;
+template <class K>
+cudaError_t allow(K kernel) {
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kStripSmem);
 }
 
 }  // namespace
 
 cudaError_t strip_init() {
-    const cudaError_t e = attrs<FineStrip>();
-    return e == cudaSuccess ? attrs<CoarseStrip>() : e;
+    cudaError_t e = allow(k_gs_strip<FineStrip, 0, false>);
+    if (e == cudaSuccess) e = allow(k_gs_strip<FineStrip, 1, false>);
+    if (e == cudaSuccess) e = allow(k_gs_strip<CoarseStrip, 0, false>);
+    if (e == cudaSuccess) e = allow(k_gs_strip<CoarseStrip, 1, false>);
+    return e == cudaSuccess ? allow(k_gs_strip<CoarseStrip, 0, true>) : e;
 }
 
 bool strip_fits(const Dims &d, bool finest) {
@@ -345,9 +323,4 @@ cudaError_t residual_strip(const Dims &d, const Coarse<double> &c, const double 
                            const double *x, double *r, cudaStream_t s) {
     return launch<CoarseStrip, 0, true>(d, CoarseStrip{c}, b, x, x, x, r, 1, d.nz - 1, s);
 }
-cudaError_t residual_strip(const Dims &d, const Fine<double> &f, const double *b,
-                           const double *x, double *r, cudaStream_t s) {
-    return launch<FineStrip, 0, true>(d, FineStrip{f}, b, x, x, x, r, 1, d.nz - 1, s);
-}
-
 }  // namespace qsmg
