@@ -462,11 +462,11 @@ mg_status sweeps_colour(mg_ctx *ctx, int l, const T *b, T *x, int sweeps, bool d
 template <typename T>
 mg_status sweeps(mg_ctx *ctx, int l, const T *b, T *x, int n, bool descending) {
     const Dims &d = ctx->L[l];
-    if (!strip_fits(d, l == 0)) return sweeps_colour<T>(ctx, l, b, x, n, descending);
+    if (!strip_fits<T>(d, l == 0)) return sweeps_colour<T>(ctx, l, b, x, n, descending);
     T *a = x, *o = ctx->r64[l];
     for (int s = 0; s < n; s++) {
         if (l == 0)
-            CK(gs_sweep_strip(d, ctx->f64, b, a, x, o, descending, ctx->st));
+            CK(gs_sweep_strip(d, ctx->f64, b, a, x, o, descending, ctx->st, 0));
         else
             CK(gs_sweep_strip(d, ctx->c64[l], b, a, x, o, descending, ctx->st));
         T *t = a;
@@ -560,7 +560,7 @@ template <typename T>
 mg_status residual_level(mg_ctx *ctx, int l, const T *b, const T *x, T *r) {
     const Dims &d = ctx->L[l];
     // the coarsest level may have odd sizes, and is never smoothed
-    const bool strip = l + 1 < ctx->nlev && strip_fits(d, false);
+    const bool strip = l + 1 < ctx->nlev && strip_fits<T>(d, false);
     if (l == 0)
         CK(residual_march(d, ctx->f64, b, x, r, ctx->st));
     else
@@ -573,6 +573,8 @@ template <>
 mg_status residual_level<float>(mg_ctx *ctx, int l, const float *b, const float *x, float *r) {
     if (l == 0)
         CK(residual_fine(ctx->L[0], ctx->f32, b, x, r, ctx->st, ctx->split0));
+    else if (l + 1 < ctx->nlev && strip_fits<float>(ctx->L[l], false))
+        CK(residual_strip(ctx->L[l], ctx->c32[l], b, x, r, ctx->st));
     else
         CK(residual_coarse(ctx->L[l], ctx->c32[l], b, x, r, ctx->st));
     return MG_OK;

@@ -126,26 +126,31 @@ cudaError_t gs_colour_coarse(const Dims &d, const Coarse<double> &c, const doubl
 cudaError_t gs_colour_coarse(const Dims &d, const Coarse<float> &c, const float *b, float *x,
                              int colour, cudaStream_t s);
 
-// FP64 sweeps and coarse residuals on row strips (strip64.cu).  strip_fits: whether a
+// Sweeps and coarse residuals on row strips (strip.cu).  strip_fits: whether a
 // level of these dimensions takes them (finest: the 19-point operator).
 // One 8-colour sweep vin -> vout, interior planes only; wall: an array that
-// holds the wall planes.  The longest rows: on 128-wide fine rows the repeated
-// work of a strip outweighs its fewer, longer launches (226 us a sweep at
-// 128^3 against 218 us for eight colour launches; at 64^3 38 against 60 us);
-// 64-wide coarse rows fill half an SM's shared memory (75 against 115 us a
-// 64^3 sweep).
+// holds the wall planes.  The longest rows, FP64: on 128-wide fine rows the
+// repeated work of a strip outweighs its fewer, longer launches (226 us a sweep
+// at 128^3 against 218 us for eight colour launches; at 64^3 38 against 60 us);
+// 64-wide coarse rows fill half an SM's shared memory (75 against 115 us a 64^3
+// sweep).  FP32, us a phase launch: coarse 64^3 7.8, 80x40x40 7.4, 48^3 6.0
+// (tile kernel 13.4-13.8); fine 64^3 6.4, 96^3 10.6, 160x80x80 13.0 (row
+// kernels of smoother_rows.cu 6.8, 15.4, 16.0).
 constexpr int kStripFineNx = 96, kStripCoarseNx = 64;
+constexpr int kStripFineNx32 = 160, kStripCoarseNx32 = 96;
 cudaError_t strip_init();
+template <typename T>
 bool strip_fits(const Dims &d, bool finest);
-cudaError_t gs_sweep_strip(const Dims &d, const Fine<double> &f, const double *b,
-                           const double *vin, const double *wall, double *vout, bool descending,
-                           cudaStream_t s);
-cudaError_t gs_sweep_strip(const Dims &d, const Coarse<double> &c, const double *b,
-                           const double *vin, const double *wall, double *vout, bool descending,
-                           cudaStream_t s);
+template <typename T>
+cudaError_t gs_sweep_strip(const Dims &d, const Fine<T> &f, const T *b, const T *vin,
+                           const T *wall, T *vout, bool descending, cudaStream_t s, int split);
+template <typename T>
+cudaError_t gs_sweep_strip(const Dims &d, const Coarse<T> &c, const T *b, const T *vin,
+                           const T *wall, T *vout, bool descending, cudaStream_t s);
 // coarse levels: r = b - A x (interior), r walls zero
-cudaError_t residual_strip(const Dims &d, const Coarse<double> &c, const double *b,
-                           const double *x, double *r, cudaStream_t s);
+template <typename T>
+cudaError_t residual_strip(const Dims &d, const Coarse<T> &c, const T *b, const T *x, T *r,
+                           cudaStream_t s);
 
 // V-cycle of the small levels in one launch (small_cycle.cu).  Offsets are
 // in elements of the CTA's shared memory; m* are division multipliers.

@@ -448,6 +448,8 @@ cudaError_t plane_init() {
 cudaError_t gs_sweep_fine_tiled(const Dims &d, const Fine<float> &f, const float *b,
                                 const float *vin, float *vout, bool descending, cudaStream_t s,
                                 int split, const SweepSync *sync) {
+    if (!sync && strip_fits<float>(d, true))
+        return gs_sweep_strip(d, f, b, vin, vin, vout, descending, s, split);
     // whole rows per CTA where the rows are short enough (smoother_rows.cu)
     const cudaError_t e = gs_sweep_fine_rows(d, f, b, vin, vout, descending, s, split, sync);
     if (e != cudaErrorNotSupported) return e;
@@ -457,6 +459,8 @@ cudaError_t gs_sweep_fine_tiled(const Dims &d, const Fine<float> &f, const float
 
 cudaError_t gs_sweep_coarse_tiled(const Dims &d, const Coarse<float> &c, const float *b,
                                   const float *vin, float *vout, bool descending, cudaStream_t s) {
+    if (strip_fits<float>(d, false))
+        return gs_sweep_strip(d, c, b, vin, vin, vout, descending, s);
     if ((long)d.nx * d.ny <= kPlaneMax) {
         // whole planes in shared memory
         cudaError_t e;
