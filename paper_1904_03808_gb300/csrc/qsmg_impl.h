@@ -166,6 +166,7 @@ struct SmallPlan {
     int nlev, nu1, nu2, ncoarse;
     int plmax, scratch;  // the largest plane; offset of the scratch
     int threads, nodes;  // threads of a CTA, nodes of a plane a thread may own
+    const void *kernel;
     size_t smem;
     const double *Ainv;
     SmallLevel lev[kSmallLevels];

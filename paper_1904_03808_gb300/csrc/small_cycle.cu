@@ -26,8 +26,8 @@
 // What bounds it: latency.  At 16^3 a phase is about 2.5 k clocks -- 600 for
 // the folded rows, 4 x 250 for the passes, 900 for the barrier and the copies
 // before it -- and at 32^3 the shared-memory loads add to that.  One FP32
-// V-cycle from 32^3 (32^3, 16^3, 8^3 and the 4^3 solve) takes 81 us against
-// about 250 us as 40 launches in a CUDA graph, one from 16^3 29 against
+// V-cycle from 32^3 (32^3, 16^3, 8^3 and the 4^3 solve) takes 78 us against
+// about 250 us as 40 launches in a CUDA graph, one from 16^3 31 against
 // 150 us.  FP64 is bound by the pipe besides (kSmallNodes64): the cycle from
 // 16^3 takes 127 us (176 with three components a thread) against 780 us.  Slower forms measured on the way, per cycle
 // from 32^3: neighbour planes read remotely at the start of a phase 89 us,
@@ -40,6 +40,8 @@
 // row and 2 w from row to row, fall into 32 different banks.
 #include <cooperative_groups.h>
 
+#include <vector>
+
 #include "qsmg_impl.h"
 
 namespace qsmg {
@@ -48,12 +50,6 @@ namespace {
 namespace cg = cooperative_groups;
 
 constexpr int kCta = 16;          // CTAs of the cluster
-// most threads of a CTA when each owns up to `nodes` nodes of a plane: the
-// register file divided by what a thread needs
-template <typename T>
-constexpr int small_threads(int nodes) {
-    return sizeof(T) == 8 ? (nodes == 1 ? 768 : 512) : nodes == 1 ? 1024 : 640;
-}
 constexpr int kMaxNodes = 4;
 constexpr size_t kSmallSmem = 220 * 1024;
 
@@ -482,8 +478,8 @@ struct Walker {
     }
 };
 
-template <typename T, int NODES>
-__global__ void __launch_bounds__(small_threads<T>(NODES), 1)
+template <typename T, int NODES, int MAXT>
+__global__ void __launch_bounds__(MAXT, 1)
     k_small_cycle(const __grid_constant__ SmallPlan<T> g, const T *__restrict__ b, T *x,
                   int from_zero, int cycles) {
     extern __shared__ __align__(16) unsigned char smem_small[];
@@ -545,6 +541,42 @@ void configure(const SmallPlan<T> &g, cudaLaunchConfig_t &cfg, cudaLaunchAttribu
     attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
+}
+
+// The kernel's instantiations, smallest planes first: `most` is the largest
+// plane (FP32: nodes, FP64: node components) and `nodes` of them go to a
+// thread.  Few threads leave each more registers, which hold a level's
+// constants and node offsets across its phases (16^3 step: 796 us with 128 of
+// them against 870 with 64); on 32 x 32 planes 512 threads with two nodes
+// each also pass barriers sooner (64^3 solve 2.83 against 2.92 ms), on planes
+// of 576 and 800 nodes one node a thread stays faster (5.07 against 5.15 ms,
+// 10.41 against 10.53 ms).
+template <typename T>
+using SmallFn = void (*)(SmallPlan<T>, const T *, T *, int, int);
+template <typename T>
+struct SmallKernel {
+    SmallFn<T> f;
+    int most, nodes;
+};
+template <typename T>
+const std::vector<SmallKernel<T>> &small_kernels();
+template <>
+const std::vector<SmallKernel<float>> &small_kernels() {
+    static const std::vector<SmallKernel<float>> k = {
+        {k_small_cycle<float, 1, 256>, 256, 1},
+        {k_small_cycle<float, 1, 512>, 512, 1},
+        {k_small_cycle<float, 1, 1024>, 960, 1},
+        {k_small_cycle<float, 2, 512>, 1024, 2},
+        {k_small_cycle<float, kMaxNodes, 640>, 640 * kMaxNodes, kMaxNodes}};
+    return k;
+}
+template <>
+const std::vector<SmallKernel<double>> &small_kernels() {
+    static const std::vector<SmallKernel<double>> k = {
+        {k_small_cycle<double, 1, 256>, 256, 1},
+        {k_small_cycle<double, 1, 768>, 768, 1},
+        {k_small_cycle<double, kMaxNodes, 512>, 512 * kMaxNodes, kMaxNodes}};
+    return k;
 }
 
 // shared-memory layout of the plan; false if it does not fit
@@ -621,19 +653,22 @@ bool small_plan(const Dims *d, const Coarse<T> *op, int nlev, int ncoarse, const
     g.Ainv = Ainv;
     // with the bank-conflict-free row pitch if that fits, else packed rows
     if (!small_layout(d, op, nlev, true, g) && !small_layout(d, op, nlev, false, g)) return false;
-    // one thread a node where the CTA can be that large, else up to kMaxNodes
     const int np = g.lev[0].np * (sizeof(T) == 8 ? 3 : 1);  // FP64: a thread a component
-    g.nodes = np <= small_threads<T>(1) ? 1 : kMaxNodes;
-    const int per = (np + g.nodes - 1) / g.nodes;
-    g.threads = per < 128 ? 128 : (per + 31) / 32 * 32;
-    if (g.threads > small_threads<T>(g.nodes)) return false;
+    g.nodes = 0;
+    for (const SmallKernel<T> &k : small_kernels<T>()) {
+        if (np > k.most) continue;
+        g.kernel = (const void *)k.f;
+        g.nodes = k.nodes;
+        const int per = (np + k.nodes - 1) / k.nodes;
+        g.threads = per < 128 ? 128 : (per + 31) / 32 * 32;
+        break;
+    }
+    if (!g.nodes) return false;
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute attr[1];
     configure(g, cfg, attr, nullptr);
     int nc = 0;
-    const cudaError_t e =
-        g.nodes == 1 ? cudaOccupancyMaxActiveClusters(&nc, k_small_cycle<T, 1>, &cfg)
-                     : cudaOccupancyMaxActiveClusters(&nc, k_small_cycle<T, kMaxNodes>, &cfg);
+    const cudaError_t e = cudaOccupancyMaxActiveClusters(&nc, (SmallFn<T>)g.kernel, &cfg);
     if (e != cudaSuccess) {
         cudaGetLastError();
         return false;
@@ -648,10 +683,7 @@ cudaError_t small_cycle(const SmallPlan<T> &g, const T *b, T *x, bool from_zero,
     cudaLaunchAttribute attr[1];
     configure(g, cfg, attr, s);
     const cudaError_t e =
-        g.nodes == 1
-            ? cudaLaunchKernelEx(&cfg, k_small_cycle<T, 1>, g, b, x, from_zero ? 1 : 0, cycles)
-            : cudaLaunchKernelEx(&cfg, k_small_cycle<T, kMaxNodes>, g, b, x, from_zero ? 1 : 0,
-                                 cycles);
+        cudaLaunchKernelEx(&cfg, (SmallFn<T>)g.kernel, g, b, x, from_zero ? 1 : 0, cycles);
     count_launch();
     return e;
 }
@@ -665,20 +697,22 @@ template cudaError_t small_cycle<float>(const SmallPlan<float> &, const float *,
 template cudaError_t small_cycle<double>(const SmallPlan<double> &, const double *, double *, bool,
                                          int, cudaStream_t);
 
-template <typename T, int NODES>
+template <typename T>
 static cudaError_t small_attrs() {
-    cudaError_t e = cudaFuncSetAttribute(k_small_cycle<T, NODES>,
-                                         cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    if (e != cudaSuccess) return e;
-    return cudaFuncSetAttribute(k_small_cycle<T, NODES>,
-                                cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmallSmem);
+    for (const SmallKernel<T> &k : small_kernels<T>()) {
+        cudaError_t e =
+            cudaFuncSetAttribute(k.f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(k.f, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)kSmallSmem);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
 }
 
 cudaError_t small_init() {
-    cudaError_t e = small_attrs<float, 1>();
-    if (e == cudaSuccess) e = small_attrs<float, kMaxNodes>();
-    if (e == cudaSuccess) e = small_attrs<double, 1>();
-    return e == cudaSuccess ? small_attrs<double, kMaxNodes>() : e;
+    const cudaError_t e = small_attrs<float>();
+    return e == cudaSuccess ? small_attrs<double>() : e;
 }
 
 }  // namespace qsmg
