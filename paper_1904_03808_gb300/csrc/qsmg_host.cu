@@ -605,15 +605,21 @@ mg_status residual_restrict_level(mg_ctx *ctx, int l, const T *b, const T *x, T 
     return MG_OK;
 }
 
-// FP32 finest level: residual and restriction fused where the row-strip
-// kernel takes the grid (the residual is never stored; r receives the
-// per-plane partial sums), else the two passes
+// FP32: residual and restriction fused where the row-strip kernel takes the
+// level (the residual is never stored; r receives the per-plane partial sums),
+// else the two passes
 template <>
 mg_status residual_restrict_level<float>(mg_ctx *ctx, int l, const float *b, const float *x,
                                          float *r, float *bc) {
     if (l == 0 && !(ctx->opts.flags & MG_FLAG_UNFUSED_TRANSFERS)) {
         const cudaError_t e =
             residual_restrict_fine_rows(ctx->L[0], ctx->f32, b, x, r, bc, ctx->st, ctx->split0);
+        if (e == cudaSuccess) return MG_OK;
+        if (e != cudaErrorNotSupported) CK(e);
+    }
+    if (l > 0) {
+        const cudaError_t e =
+            residual_restrict_coarse_rows(ctx->L[l], ctx->c32[l], b, x, r, bc, ctx->st);
         if (e == cudaSuccess) return MG_OK;
         if (e != cudaErrorNotSupported) CK(e);
     }
@@ -1057,7 +1063,6 @@ mg_status mg_setup(const mg_grid *grid, const mg_moduli *moduli, const mg_bc *bc
     }
     {
         cudaError_t e = smoother_init();
-        if (e == cudaSuccess) e = plane_init();
         if (e == cudaSuccess) e = small_init();
         if (e == cudaSuccess) e = strip_init();
         if (e != cudaSuccess) {

@@ -134,10 +134,12 @@ cudaError_t gs_colour_coarse(const Dims &d, const Coarse<float> &c, const float 
 // at 128^3 against 218 us for eight colour launches; at 64^3 38 against 60 us);
 // 64-wide coarse rows fill half an SM's shared memory (75 against 115 us a 64^3
 // sweep).  FP32, us a phase launch: coarse 64^3 7.8, 80x40x40 7.4, 48^3 6.0
-// (tile kernel 13.4-13.8); fine 64^3 6.4, 96^3 10.6, 160x80x80 13.0 (row
-// kernels of smoother_rows.cu 6.8, 15.4, 16.0).
+// (tile kernel 13.4-13.8); fine 64^3 6.4, 96^3 10.6 (row kernels of
+// smoother_rows.cu 6.8, 15.4).
 constexpr int kStripFineNx = 96, kStripCoarseNx = 64;
-constexpr int kStripFineNx32 = 160, kStripCoarseNx32 = 96;
+// From 128 nodes a row on the persistent strips are faster (160x80x80 step 9.75
+// against 10.03 ms).
+constexpr int kStripFineNx32 = 126, kStripCoarseNx32 = 126;
 cudaError_t strip_init();
 template <typename T>
 bool strip_fits(const Dims &d, bool finest);
@@ -182,10 +184,9 @@ template <typename T>
 cudaError_t small_cycle(const SmallPlan<T> &g, const T *b, T *x, bool from_zero, int cycles,
                         cudaStream_t s);
 
-// one-time kernel attribute set-up of the sweeps (call before any capture):
-// smoother_init for the row-strip kernels, plane_init for the whole-plane one
+// one-time kernel attribute set-up of the row-strip kernels (call before any
+// capture)
 cudaError_t smoother_init();
-cudaError_t plane_init();
 // FP32 finest-level residual with the persistent row-strip kernel;
 // cudaErrorNotSupported when the grid or the arrays do not suit it
 cudaError_t residual_fine_rows(const Dims &d, const Fine<float> &f, const float *b,
@@ -196,6 +197,10 @@ cudaError_t residual_fine_rows(const Dims &d, const Fine<float> &f, const float 
 bool coarse_rows_fit(const Dims &d);
 cudaError_t gs_sweep_coarse_rows(const Dims &d, const Coarse<float> &c, const float *b,
                                  const float *vin, float *vout, bool descending, cudaStream_t s);
+// coarse FP32 residual and restriction without storing the residual (part:
+// 3 (nz+1) ny/2 nx/2 floats), or cudaErrorNotSupported
+cudaError_t residual_restrict_coarse_rows(const Dims &d, const Coarse<float> &c, const float *b,
+                                          const float *x, float *part, float *bc, cudaStream_t s);
 // Cross-CTA state of the fused finest-level sweep (device memory, zeroed at
 // allocation, owned by the context): per-tile ready flags that hold the
 // launch count + 1 once the tile is stored, the launch count, the CTAs done

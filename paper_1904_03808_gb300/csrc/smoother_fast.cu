@@ -345,104 +345,7 @@ cudaError_t sweep(const Dims &d, const Op &op, const T *b, const T *vin, T *vout
 }
 
 
-// ------------------------------------------------------------------------
-// Whole-plane phase kernel for small coarse levels (planes of at most
-// kPlaneMax nodes): one CTA per plane of the phase's parity holds the plane,
-// its two z-neighbour planes and its right-hand side in shared memory
-// ([component][ny][nx] each, 48 KB at 32 x 32), folds the z-neighbour terms
-// into the right-hand side once, and runs the 4 in-plane colour passes on
-// shared memory only, with periodic x, y indexing (no halo: the plane is
-// whole).  The tile kernel, whose 72 x 20 window wraps several times around
-// such small planes, spends ~15-17 us a launch on latency at these sizes;
-// this kernel takes 10.7 us at 32 x 32 (one thread per node) and 6.4-6.7 us
-// at 16 x 16 and 8 x 8 (measured on GB300).  At 64 x 64 it loses to the tile
-// kernel (27.7 against 18 us: one CTA per plane leaves most SMs idle).
-constexpr int kPlaneMax = 1024;
-constexpr int kPlaneThreads = 1024;  // at most; one per node of the plane
-
-template <int F>
-__global__ void __launch_bounds__(kPlaneThreads)
-    k_gs_plane(Dims d, Coarse<float> c, const float *__restrict__ b, const float *__restrict__ vin,
-               const float *__restrict__ zsrc, float *__restrict__ vout, int kbase) {
-    extern __shared__ __align__(16) float smp[];
-    const int nx = d.nx, ny = d.ny, np = nx * ny;
-    const long ps = (long)np, cs = d.cs;
-    float *P = smp, *Lz = smp + 3 * np, *Hz = smp + 6 * np, *Rr = smp + 9 * np;
-    const int k = 2 * blockIdx.x + kbase;
-    for (int e = threadIdx.x; e < 3 * np; e += blockDim.x) {
-        const int a = e / np, m = e - a * np;
-        P[e] = vin[a * cs + k * ps + m];
-        Lz[e] = zsrc[a * cs + (k - 1) * ps + m];
-        Hz[e] = zsrc[a * cs + (k + 1) * ps + m];
-        Rr[e] = b[a * cs + k * ps + m];
-    }
-    __syncthreads();
-    // fold the z-neighbour blocks (dz = -1, +1) into the right-hand side
-    for (int m = threadIdx.x; m < np; m += blockDim.x) {
-        const int j = m / nx, i = m - j * nx;
-        const int col[3] = {i ? i - 1 : nx - 1, i, i + 1 < nx ? i + 1 : 0};
-        const int row[3] = {(j ? j - 1 : ny - 1) * nx, j * nx, (j + 1 < ny ? j + 1 : 0) * nx};
-        auto sd = [&](int b, int dx, int dy, float &S, float &D) {
-            const int q = b * np + row[dy + 1] + col[dx + 1];
-            S = Hz[q] + Lz[q];
-            D = Hz[q] - Lz[q];
-        };
-        float o[3] = {0.f, 0.f, 0.f};
-        coarse_z_terms(c, sd, o);
-        Rr[m] -= o[0];
-        Rr[np + m] -= o[1];
-        Rr[2 * np + m] -= o[2];
-    }
-    __syncthreads();
-    // colours (F,F), (1-F,F), (F,1-F), (1-F,1-F) in (x, y) parity
-    const int hx = nx >> 1, nh = np >> 2;
-#pragma unroll 1
-    for (int pass = 0; pass < 4; pass++) {
-        const int pi = (pass & 1) ? 1 - F : F, pj = (pass & 2) ? 1 - F : F;
-        for (int t = threadIdx.x; t < nh; t += blockDim.x) {
-            const int jh = t / hx, i = 2 * (t - jh * hx) + pi, j = 2 * jh + pj;
-            const int col[3] = {i ? i - 1 : nx - 1, i, i + 1 < nx ? i + 1 : 0};
-            const int row[3] = {(j ? j - 1 : ny - 1) * nx, j * nx, (j + 1 < ny ? j + 1 : 0) * nx};
-            auto u = [&](int b, int dx, int dy) -> float {
-                return P[b * np + row[dy + 1] + col[dx + 1]];
-            };
-            float o[3];
-            coarse_plane_terms(c, u, o);
-            const int m = j * nx + i;
-#pragma unroll
-            for (int a = 0; a < 3; a++) P[a * np + m] = c.dinv[a] * (Rr[a * np + m] - o[a]);
-        }
-        __syncthreads();
-    }
-    for (int e = threadIdx.x; e < 3 * np; e += blockDim.x) {
-        const int a = e / np, m = e - a * np;
-        vout[a * cs + k * ps + m] = P[e];
-    }
-}
-
-template <int F>
-cudaError_t launch_plane(const Dims &d, const Coarse<float> &c, const float *b, const float *vin,
-                         const float *zsrc, float *vout, int par, cudaStream_t s) {
-    const int kbase = par ? 1 : 2;
-    const int nplanes = par ? d.nz / 2 : d.nz / 2 - 1;
-    if (nplanes <= 0) return cudaSuccess;
-    const size_t smem = 12 * (size_t)d.nx * d.ny * sizeof(float);
-    const int np = d.nx * d.ny;
-    const int threads = np < kPlaneThreads ? ((np + 31) / 32) * 32 : kPlaneThreads;
-    k_gs_plane<F><<<nplanes, threads, smem, s>>>(d, c, b, vin, zsrc, vout, kbase);
-    count_launch();
-    return cudaGetLastError();
-}
-
 }  // namespace
-
-cudaError_t plane_init() {
-    const int smem = (int)(12 * (size_t)kPlaneMax * sizeof(float));
-    cudaError_t e = cudaFuncSetAttribute(k_gs_plane<0>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         smem);
-    if (e != cudaSuccess) return e;
-    return cudaFuncSetAttribute(k_gs_plane<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-}
 
 // one 8-colour sweep vin -> vout (vout's wall planes must hold the walls)
 cudaError_t gs_sweep_fine_tiled(const Dims &d, const Fine<float> &f, const float *b,
@@ -461,18 +364,6 @@ cudaError_t gs_sweep_coarse_tiled(const Dims &d, const Coarse<float> &c, const f
                                   const float *vin, float *vout, bool descending, cudaStream_t s) {
     if (strip_fits<float>(d, false))
         return gs_sweep_strip(d, c, b, vin, vin, vout, descending, s);
-    if ((long)d.nx * d.ny <= kPlaneMax) {
-        // whole planes in shared memory
-        cudaError_t e;
-        if (!descending) {
-            e = launch_plane<0>(d, c, b, vin, vin, vout, 0, s);
-            if (e != cudaSuccess) return e;
-            return launch_plane<0>(d, c, b, vin, vout, vout, 1, s);
-        }
-        e = launch_plane<1>(d, c, b, vin, vin, vout, 1, s);
-        if (e != cudaSuccess) return e;
-        return launch_plane<1>(d, c, b, vin, vout, vout, 0, s);
-    }
     // whole-row strips where the rows fit (smoother_rows.cu)
     const cudaError_t e = gs_sweep_coarse_rows(d, c, b, vin, vout, descending, s);
     if (e != cudaErrorNotSupported) return e;

@@ -1,23 +1,20 @@
-// smoother_rows.cu -- row-strip Gauss-Seidel sweep phases (FP32) for the
-// finest level (structured 19-point operator of the scaled Eq. 30) and for
+// smoother_rows.cu -- persistent row-strip Gauss-Seidel sweep phases (FP32) for
+// the finest level (structured 19-point operator of the scaled Eq. 30) and for
 // coarse levels of rows >= 128 nodes (27-point block stencil, Eq. 36), and
-// the finest-level residual.
+// the residuals of those levels.
 //
 // One 8-colour sweep runs as two phase launches, as in smoother_fast.cu:
 // the planes of one k-parity (4 in-plane colours each, reading the old
 // z-neighbour planes), then the planes of the other parity (reading the
-// first phase's output).  Here a CTA owns whole rows of a plane, so the
-// periodic x direction needs no halo.  Two kernels:
-//   k_gs_rows_p  persistent, for rows of 64, 128, 192 or 256 nodes (a
-//                multiple of 64, at least 9 rows): the rows of
-//                each tile are copied into shared memory with cp.async while
-//                the other CTAs on the SM compute; templated on the operator
-//                (FineRowsOp, CoarseRowsOp) and, with RES, computing the
-//                residual b - A x instead of a sweep phase (with RR as well,
-//                restricting it in x and y on the fly instead of storing it);
-//   k_gs_rows    one CTA per tile, operands loaded straight into registers,
-//                for the other finest rows of up to 512 nodes.
-// Both compute every node from the same neighbour values as the sequential
+// first phase's output).  A CTA owns whole rows of a plane where they have at
+// most 512 nodes, so the periodic x direction needs no halo, and tiles of
+// longer rows with 8 halo columns a side.  k_gs_rows_p copies the rows of
+// each tile into shared memory with cp.async while the other CTAs on the SM
+// compute; it is templated on the operator (FineRowsOp, CoarseRowsOp) and, with
+// RES, computes the residual b - A x instead of a sweep phase (with RR as well,
+// restricting it in x and y on the fly instead of storing it).  Rows have a
+// multiple of 4 nodes (of 8 beyond 256) and planes at least 9 of them.
+// Every node is computed from the same neighbour values as in the sequential
 // colour order (tested against the eight colour launches).
 #include <stdint.h>
 
@@ -26,13 +23,8 @@
 namespace qsmg {
 namespace {
 
-__device__ __forceinline__ int wrap_mod(int a, int n) {
-    a %= n;
-    return a < 0 ? a + n : a;
-}
-
 // ------------------------------------------------------------------------
-// Tile geometry shared by both kernels.  A CTA owns TY whole rows of one plane; thread t owns the node pair
+// Tile geometry.  A CTA owns TY rows of one plane; thread t owns the node pair
 // x = 2t ("E") and x = 2t+1 ("O") in every row of the strip's window and
 // keeps their values in registers, so of a node's eight in-plane neighbours
 // only the three on the far x side (the neighbouring thread's column) come
@@ -56,8 +48,6 @@ __device__ __forceinline__ int wrap_mod(int a, int n) {
 //   z_1 = (L1+H1) + kq (D2(y+1) - D2(y-1)),
 //   z_2 = lp (L2+H2) + kq ((D0(x+1) - D0(x-1)) + (D1(y+1) - D1(y-1))),
 // with D = H - L, streamed row by row so each plane value is loaded once.
-constexpr int kRowsMaxThreads = 256;  // rows up to 512 nodes
-
 // numerators of the node of x-parity E at window row jj: the folded
 // right-hand side r plus the in-plane neighbour terms, from the own column
 // values P and the far-side neighbour column X[c * sc + row * sr + xn]
@@ -90,200 +80,6 @@ __device__ __forceinline__ void rows_numer(const float (&P)[3][2][R], float r0, 
              kq * (p[0][2] - p[0][0] - m[0][2] + m[0][0]);
     num[2] = r2 + (m[2][1] + p[2][1]) + (P[2][E][jj - 1] + P[2][E][jj + 1]);
 }
-
-// Gauss-Seidel update of the node of x-parity E at window row jj
-template <int E, int R>
-__device__ __forceinline__ void rows_update(float (&P)[3][2][R], float r0, float r1, float r2,
-                                            const float *X, int sc, int sr, int xn, int jj,
-                                            const Fine<float> &f) {
-    float num[3];
-    rows_numer<E, R>(P, r0, r1, r2, X, sc, sr, xn, jj, f, num);
-#pragma unroll
-    for (int c = 0; c < 3; c++) P[c][E][jj] = num[c] * f.dinv;
-}
-
-template <int TY, int F, bool SPLIT>
-__global__ void __launch_bounds__(kRowsMaxThreads, 2)
-    k_gs_rows(Dims d, Fine<float> f, const float *__restrict__ b, const float *__restrict__ vin,
-              const float *__restrict__ zsrc, float *__restrict__ vout, int kbase) {
-    constexpr int R = TY + 3;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int nt = blockDim.x;
-    float *XE = reinterpret_cast<float *>(smem_raw);  // [3][R][nt] E values by column
-    float *XO = XE + 3 * R * nt;                       // [3][R][nt] O values by column
-    float *RS = XO + 3 * R * nt;                       // [3][2][R][nt] folded right-hand sides
-    const int nx = d.nx, ny = d.ny, hn = nx >> 1;
-    const long ps = (long)nx * ny, cs = d.cs;
-    const int t = threadIdx.x;
-    const bool act = t < hn;
-    const int tc = act ? t : hn - 1;  // spare lanes mirror the last column, store nothing
-    const int tm = tc == 0 ? hn - 1 : tc - 1, tp = tc + 1 == hn ? 0 : tc + 1;
-    const int cE = SPLIT ? tc : 2 * tc, cO = SPLIT ? hn + tc : 2 * tc + 1;
-    const int cOm = SPLIT ? hn + tm : 2 * tm + 1;  // x - 1 of the E node
-    const int cEp = SPLIT ? tp : 2 * tp;           // x + 1 of the O node
-    const int k = 2 * blockIdx.y + kbase;
-    const int y0 = blockIdx.x * TY;
-    const float lp = f.lp, kq = f.kq;
-
-    // right-hand side with the z-neighbour terms folded in, for rows 1 .. R-2,
-    // streamed row by row (row jj's plane values complete row jj-1)
-    const float *Lz = zsrc + (long)(k - 1) * ps, *Hz = zsrc + (long)(k + 1) * ps;
-    const float *Bk = b + (long)k * ps;
-    float S1[3][2], D1[3][2];  // row jj-1: L+H and H-L of the own columns
-    float D2y[2][2];           // row jj-2: H-L of components 1, 2
-    float dm0 = 0.f, dm2 = 0.f, dp0 = 0.f, dp2 = 0.f;  // row jj-1: far-side H-L
-#pragma unroll 2
-    for (int jj = 0; jj < R; jj++) {
-        const int o = wrap_mod(y0 - 1 - F + jj, ny) * nx;
-        float S0[3][2], D0[3][2];
-#pragma unroll
-        for (int c = 0; c < 3; c++) {
-            const float lE = __ldg(Lz + c * cs + o + cE), hE = __ldg(Hz + c * cs + o + cE);
-            const float lO = __ldg(Lz + c * cs + o + cO), hO = __ldg(Hz + c * cs + o + cO);
-            S0[c][0] = lE + hE;
-            S0[c][1] = lO + hO;
-            D0[c][0] = hE - lE;
-            D0[c][1] = hO - lO;
-        }
-        const float nm0 = __ldg(Hz + o + cOm) - __ldg(Lz + o + cOm);
-        const float nm2 = __ldg(Hz + 2 * cs + o + cOm) - __ldg(Lz + 2 * cs + o + cOm);
-        const float np0 = __ldg(Hz + o + cEp) - __ldg(Lz + o + cEp);
-        const float np2 = __ldg(Hz + 2 * cs + o + cEp) - __ldg(Lz + 2 * cs + o + cEp);
-        if (jj >= 2) {
-            const int ob = wrap_mod(y0 - 2 - F + jj, ny) * nx;
-            const int w = jj - 1;
-#define RSW(c, e) RS[(((c) * 2 + (e)) * R + w) * nt + t]
-            // E node: x-1 is the neighbour's O column, x+1 the own O column
-            RSW(0, 0) = __ldg(Bk + ob + cE) + (S1[0][0] + kq * (D1[2][1] - dm2));
-            RSW(1, 0) = __ldg(Bk + cs + ob + cE) + (S1[1][0] + kq * (D0[2][0] - D2y[1][0]));
-            RSW(2, 0) = __ldg(Bk + 2 * cs + ob + cE) +
-                        (lp * S1[2][0] + kq * ((D1[0][1] - dm0) + (D0[1][0] - D2y[0][0])));
-            // O node: x-1 is the own E column, x+1 the neighbour's E column
-            RSW(0, 1) = __ldg(Bk + ob + cO) + (S1[0][1] + kq * (dp2 - D1[2][0]));
-            RSW(1, 1) = __ldg(Bk + cs + ob + cO) + (S1[1][1] + kq * (D0[2][1] - D2y[1][1]));
-            RSW(2, 1) = __ldg(Bk + 2 * cs + ob + cO) +
-                        (lp * S1[2][1] + kq * ((dp0 - D1[0][0]) + (D0[1][1] - D2y[0][1])));
-#undef RSW
-        }
-#pragma unroll
-        for (int e = 0; e < 2; e++) {
-            D2y[0][e] = D1[1][e];
-            D2y[1][e] = D1[2][e];
-#pragma unroll
-            for (int c = 0; c < 3; c++) {
-                S1[c][e] = S0[c][e];
-                D1[c][e] = D0[c][e];
-            }
-        }
-        dm0 = nm0;
-        dm2 = nm2;
-        dp0 = np0;
-        dp2 = np2;
-    }
-
-    // own columns of this plane
-    int roff[R];
-#pragma unroll
-    for (int jj = 0; jj < R; jj++) roff[jj] = wrap_mod(y0 - 1 - F + jj, ny) * nx;
-    const float *Pk = vin + (long)k * ps;
-    float P[3][2][R];
-#pragma unroll
-    for (int c = 0; c < 3; c++)
-#pragma unroll
-        for (int jj = 0; jj < R; jj++) {
-            P[c][0][jj] = __ldg(Pk + c * cs + roff[jj] + cE);
-            P[c][1][jj] = __ldg(Pk + c * cs + roff[jj] + cO);
-        }
-
-    // publish the own columns for the neighbours
-#pragma unroll
-    for (int c = 0; c < 3; c++)
-#pragma unroll
-        for (int jj = 0; jj < R; jj++) {
-            XE[(c * R + jj) * nt + t] = P[c][0][jj];
-            XO[(c * R + jj) * nt + t] = P[c][1][jj];
-        }
-    __syncthreads();
-    // an E node's far side is column t-1's O, an O node's is column t+1's E
-    constexpr int EF = F, EG = 1 - F;
-    float *XF = EF == 0 ? XE : XO, *XG = EG == 0 ? XE : XO;
-    const float *NF = EF == 0 ? XO : XE, *NG = EG == 0 ? XO : XE;
-    const int tnF = EF == 0 ? tm : tp, tnG = EG == 0 ? tm : tp;
-    // pass 1: x-parity F on the odd rows
-#pragma unroll
-    for (int jj = 1; jj < R - 1; jj += 2) {
-        rows_update<EF, R>(P, RS[((0 * 2 + EF) * R + jj) * nt + t], RS[((1 * 2 + EF) * R + jj) * nt + t],
-                               RS[((2 * 2 + EF) * R + jj) * nt + t], NF, R * nt, nt, tnF, jj, f);
-#pragma unroll
-        for (int c = 0; c < 3; c++) XF[(c * R + jj) * nt + t] = P[c][EF][jj];
-    }
-    __syncthreads();
-    // pass 2: x-parity 1-F on the odd rows
-#pragma unroll
-    for (int jj = 1; jj < R - 1; jj += 2) {
-        rows_update<EG, R>(P, RS[((0 * 2 + EG) * R + jj) * nt + t], RS[((1 * 2 + EG) * R + jj) * nt + t],
-                               RS[((2 * 2 + EG) * R + jj) * nt + t], NG, R * nt, nt, tnG, jj, f);
-#pragma unroll
-        for (int c = 0; c < 3; c++) XG[(c * R + jj) * nt + t] = P[c][EG][jj];
-    }
-    __syncthreads();
-    // pass 3: x-parity F on the even rows
-#pragma unroll
-    for (int jj = 2; jj < R - 2; jj += 2) {
-        rows_update<EF, R>(P, RS[((0 * 2 + EF) * R + jj) * nt + t], RS[((1 * 2 + EF) * R + jj) * nt + t],
-                               RS[((2 * 2 + EF) * R + jj) * nt + t], NF, R * nt, nt, tnF, jj, f);
-#pragma unroll
-        for (int c = 0; c < 3; c++) XF[(c * R + jj) * nt + t] = P[c][EF][jj];
-    }
-    __syncthreads();
-    // pass 4: x-parity 1-F on the even rows
-#pragma unroll
-    for (int jj = 2; jj < R - 2; jj += 2) rows_update<EG, R>(P, RS[((0 * 2 + EG) * R + jj) * nt + t], RS[((1 * 2 + EG) * R + jj) * nt + t],
-                               RS[((2 * 2 + EG) * R + jj) * nt + t], NG, R * nt, nt, tnG, jj, f);
-
-    // store the tile rows
-    if (!act) return;
-    float *Ok = vout + (long)k * ps;
-#pragma unroll
-    for (int jj = 1 + F; jj < TY + 1 + F; jj++) {
-        const int y = y0 - 1 - F + jj;
-        if (y < ny) {
-#pragma unroll
-            for (int c = 0; c < 3; c++) {
-                Ok[c * cs + roff[jj] + cE] = P[c][0][jj];
-                Ok[c * cs + roff[jj] + cO] = P[c][1][jj];
-            }
-        }
-    }
-}
-
-constexpr int kRowsTY = 6;  // tile rows: 128 registers without spills
-
-// shared memory of one row-strip CTA: exchange columns (2 x 3 x R) and the
-// folded right-hand sides (3 x 2 x R), nt columns each
-inline size_t rows_smem(int nt) { return 12 * (size_t)(kRowsTY + 3) * nt * sizeof(float); }
-
-template <int F, bool SPLIT>
-cudaError_t launch_rows(const Dims &d, const Fine<float> &f, const float *b, const float *vin,
-                        const float *zsrc, float *vout, int par, cudaStream_t s) {
-    const int kbase = par ? 1 : 2;
-    const int nplanes = par ? d.nz / 2 : d.nz / 2 - 1;
-    if (nplanes <= 0) return cudaSuccess;
-    const int nt = ((d.nx / 2 + 31) / 32) * 32;
-    const size_t smem = rows_smem(nt);
-    dim3 grid((d.ny + kRowsTY - 1) / kRowsTY, nplanes);
-    k_gs_rows<kRowsTY, F, SPLIT><<<grid, nt, smem, s>>>(d, f, b, vin, zsrc, vout, kbase);
-    count_launch();
-    return cudaGetLastError();
-}
-
-template <int F>
-cudaError_t rows_phase(const Dims &d, const Fine<float> &f, const float *b, const float *vin,
-                       const float *zsrc, float *vout, int par, cudaStream_t s, int split) {
-    return split ? launch_rows<F, true>(d, f, b, vin, zsrc, vout, par, s)
-                 : launch_rows<F, false>(d, f, b, vin, zsrc, vout, par, s);
-}
-
 
 // ------------------------------------------------------------------------
 // Persistent kernel.  Two CTAs per SM at nx = 256 (128 threads each; four at
@@ -318,7 +114,18 @@ cudaError_t rows_phase(const Dims &d, const Fine<float> &f, const float *b, cons
 constexpr int kPersTY = 6;
 constexpr int kPersR = kPersTY + 3;
 constexpr int kPersMinBlocks = 2;  // resident CTAs per SM at nx = 256 (more for shorter rows)
-constexpr int kPersMaxNx = 256;
+constexpr int kPersMaxNx = 256;    // longest whole rows; longer ones are cut into tiles
+constexpr int kPersHalo = 8;       // halo columns a side of a tile (aligned 16-byte copies)
+constexpr int kPersMaxW = kPersMaxNx + 2 * kPersHalo;
+constexpr int kPersMaxWide = 512;  // longest whole rows with one CTA an SM
+// How a row is dealt to CTAs: whole rows of up to 256 nodes (two CTAs an SM or
+// more), whole rows of up to 512 (one CTA of 256 threads: what the other CTA
+// would overlap, the larger copies in flight make up for), tiles of longer
+// ones.  512 x 512 x 256, us a phase: whole rows 363; tiles of 256 in windows of
+// 272, two CTAs an SM, 482 (five warps leave 168 registers a thread and one of
+// them is nearly empty); tiles of 176 in windows of 192 with 255 registers 564;
+// one CTA a tile without the persistent loop 588.
+enum { kRows = 0, kWide = 1, kTiles = 2 };
 constexpr int kPersPB = 16;  // planes per block of the tile order
 
 __host__ __device__ constexpr long pers_floats(int nx) {
@@ -421,39 +228,66 @@ struct CoarseRowsOp {
                                                   int comp, int x2) {
         return *reinterpret_cast<const float2 *>(&A[q.at(row, comp, x2)]);
     }
+    // row by row: row y contributes A to its own right-hand side, U to the row
+    // above it and V to the row below, each formed from four columns of that
+    // row only (z_row in small_cycle.cu has the algebra), so a row's z sums and
+    // differences are loaded and formed once instead of for three rows
     template <int R>
     __device__ __forceinline__ void fold(float (&r)[3][2][R], const float *Ls, const float *Hs,
                                          const float *Bs, const RowCols &q) const {
         const int xl = q.xom - 1, xr = q.xep;  // first columns of the left / right pairs
 #pragma unroll
-        for (int jj = 1; jj < R - 1; jj++) {
+        for (int jj = 1; jj < R - 1; jj++)
+#pragma unroll
+            for (int a = 0; a < 3; a++) {
+                const float2 b2 = pair(Bs, q, jj - 1, a, q.xe);
+                r[a][0][jj] = b2.x;
+                r[a][1][jj] = b2.y;
+            }
+#pragma unroll
+        for (int jj = 0; jj < R; jj++) {
             // z sums and differences at columns x_E - 1, x_E, x_O, x_O + 1
-            float S[3][3][4], D[3][3][4];  // [component][dy + 1][column]
+            float S[3][4], D[3][4];
 #pragma unroll
-            for (int b = 0; b < 3; b++)
+            for (int b = 0; b < 3; b++) {
+                const float2 ll = pair(Ls, q, jj, b, xl), lo = pair(Ls, q, jj, b, q.xe),
+                             lr = pair(Ls, q, jj, b, xr);
+                const float2 hl = pair(Hs, q, jj, b, xl), ho = pair(Hs, q, jj, b, q.xe),
+                             hr = pair(Hs, q, jj, b, xr);
+                const float L4[4] = {ll.y, lo.x, lo.y, lr.x}, H4[4] = {hl.y, ho.x, ho.y, hr.x};
 #pragma unroll
-                for (int dy = -1; dy <= 1; dy++) {
-                    const float2 ll = pair(Ls, q, jj + dy, b, xl), lo = pair(Ls, q, jj + dy, b, q.xe),
-                                 lr = pair(Ls, q, jj + dy, b, xr);
-                    const float2 hl = pair(Hs, q, jj + dy, b, xl), ho = pair(Hs, q, jj + dy, b, q.xe),
-                                 hr = pair(Hs, q, jj + dy, b, xr);
-                    const float L4[4] = {ll.y, lo.x, lo.y, lr.x}, H4[4] = {hl.y, ho.x, ho.y, hr.x};
-#pragma unroll
-                    for (int m = 0; m < 4; m++) {
-                        S[b][dy + 1][m] = H4[m] + L4[m];
-                        D[b][dy + 1][m] = H4[m] - L4[m];
-                    }
+                for (int m = 0; m < 4; m++) {
+                    S[b][m] = H4[m] + L4[m];
+                    D[b][m] = H4[m] - L4[m];
                 }
+            }
 #pragma unroll
             for (int e = 0; e < 2; e++) {
-                auto sd = [&](int b, int dx, int dy, float &s_, float &d_) {
-                    s_ = S[b][dy + 1][e + dx + 1];
-                    d_ = D[b][dy + 1][e + dx + 1];
-                };
-                float o[3] = {0.f, 0.f, 0.f};
-                coarse_z_terms(c, sd, o);
+                const int m = e, o = e + 1, p = e + 2;  // columns x - 1, x, x + 1
+                const float d0 = D[0][p] - D[0][m], d2 = D[2][p] - D[2][m];
+                float B[3], G[3], sx[3];
 #pragma unroll
-                for (int a = 0; a < 3; a++) r[a][e][jj] = Bs[q.at(jj - 1, a, e ? q.xo : q.xe)] - o[a];
+                for (int a = 0; a < 3; a++) {
+                    sx[a] = S[a][m] + S[a][p];
+                    B[a] = c.cd[a][6] * S[a][o] + c.cd[a][7] * sx[a];
+                }
+                B[0] += c.g[1][1] * d2;
+                B[2] += c.g[1][1] * d0;
+                G[0] = c.g[2][1] * (S[1][p] - S[1][m]);
+                G[1] = c.g[2][1] * (S[0][p] - S[0][m]) +
+                       (c.g[0][0] * D[2][o] + c.g[0][1] * (D[2][m] + D[2][p]));
+                G[2] = c.g[0][0] * D[1][o] + c.g[0][1] * (D[1][m] + D[1][p]);
+#pragma unroll
+                for (int a = 0; a < 3; a++) {
+                    if (jj >= 1 && jj < R - 1) {
+                        float A = c.cd[a][4] * S[a][o] + c.cd[a][5] * sx[a];
+                        if (a == 0) A += c.g[1][0] * d2;
+                        if (a == 2) A += c.g[1][0] * d0;
+                        r[a][e][jj] -= A;
+                    }
+                    if (jj + 1 < R - 1) r[a][e][jj + 1] -= B[a] - G[a];
+                    if (jj >= 2) r[a][e][jj - 1] -= B[a] + G[a];
+                }
             }
         }
     }
@@ -510,15 +344,25 @@ __device__ __forceinline__ void pers_update(const OP &op, float (&P)[3][2][R],
 // x and y parts of the restriction to it and vout receives, per fine plane,
 // the coarse-grid partial sums [c][k][J][I] (c stride (nz+1) ny/2 nx/2) that
 // k_restrict_z combines along z.
-template <class OP, int F, bool SPLIT, bool RES, bool RR = false>
-__global__ void __launch_bounds__(kPersMaxNx / 2, kPersMinBlocks)
+// kTiles: a tile is XT columns of longer rows with kPersHalo columns around them
+// (the window is what a row is otherwise; its outermost columns see a false
+// neighbour, which reaches one column further in each pass and never the tile).
+template <class OP, int F, bool SPLIT, int MODE, bool RES, bool RR = false>
+__global__ void __launch_bounds__(MODE == kRows    ? kPersMaxNx / 2
+                                  : MODE == kWide ? kPersMaxWide / 2
+                                                  : kPersMaxW / 2,
+                                  MODE == kWide ? 1 : kPersMinBlocks)
     k_gs_rows_p(Dims d, OP op, const float *__restrict__ b, const float *__restrict__ vin,
                 const float *__restrict__ zsrc, float *__restrict__ vout, int kbase, int kstep,
-                int nplanes, int nstrips) {
+                int nplanes, int nstrips, int xt) {
     constexpr int TY = kPersTY, R = kPersR;
+    constexpr bool WIN = MODE == kTiles;
     extern __shared__ __align__(16) float sm[];
-    const int nx = d.nx, ny = d.ny, hn = nx >> 1, cpr = nx >> 2;
-    const long ps = (long)nx * ny, cs = d.cs;
+    const int gnx = d.nx, ny = d.ny, ghn = gnx >> 1;
+    const int nx = WIN ? xt + 2 * kPersHalo : gnx;  // columns of the window
+    const int ntx = WIN ? (gnx + xt - 1) / xt : 1;  // (nstrips counts x tiles too)
+    const int hn = nx >> 1, cpr = nx >> 2;
+    const long ps = (long)gnx * ny, cs = d.cs;
     const int plane_f = 3 * R * nx, bst_f = 3 * (R - 2) * nx;
     float *const Ps = sm, *const Bs = sm + plane_f, *const Zs0 = Bs + bst_f;
     const int t = threadIdx.x;
@@ -534,13 +378,29 @@ __global__ void __launch_bounds__(kPersMaxNx / 2, kPersMinBlocks)
     const long n0 = blockIdx.x * ntiles / gridDim.x, n1 = (blockIdx.x + 1) * ntiles / gridDim.x;
     if (n0 >= n1) return;
 
+    // first row and first column (before the halo) of strip s
+    auto row0 = [&](int s) { return WIN ? s / ntx * TY : s * TY; };
+    auto col0 = [&](int s) { return WIN ? s % ntx * xt : 0; };
+    // position of this thread's copy chunk in a global row, window at column x0
+    auto chunk_col = [&](int x0) {
+        if (!WIN) return q4;
+        if (SPLIT) {
+            const int half = q4 >= hn, c = q4 - half * hn;  // hn is a multiple of 4
+            int p = ((x0 - kPersHalo) >> 1) + c;
+            p = p < 0 ? p + ghn : p;
+            return half * ghn + p % ghn;
+        }
+        int p = x0 - kPersHalo + q4;
+        p = p < 0 ? p + gnx : p;
+        return p % gnx;
+    };
     // window rows [jlo, jhi) of plane qq of src into dst (rows from jlo)
-    auto copy_rows = [&](float *dst, const float *src, int qq, int y0, int jlo, int jhi) {
-        const float *base = src + (long)qq * ps + q4;
+    auto copy_rows = [&](float *dst, const float *src, int qq, int y0, int gc, int jlo, int jhi) {
+        const float *base = src + (long)qq * ps + gc;
         for (int jj = jlo + g; jj < jhi; jj += 2) {
             int y = y0 - 1 - F + jj;  // ny >= R: at most one wrap
             y = y < 0 ? y + ny : (y >= ny ? y - ny : y);
-            const float *srow = base + (long)y * nx;
+            const float *srow = base + (long)y * gnx;
             float *drow = dst + (jj - jlo) * 3 * nx + q4;
             cp_async16(drow, srow);
             cp_async16(drow + nx, srow + cs);
@@ -562,8 +422,8 @@ __global__ void __launch_bounds__(kPersMaxNx / 2, kPersMinBlocks)
     auto issue_bz = [&](long n, int &sL, int &sH) {
         int s, k;
         tile_of(n, s, k);
-        const int y0 = s * TY;
-        copy_rows(Bs, b, k, y0, 1, R - 1);
+        const int y0 = row0(s), gc = chunk_col(col0(s));
+        copy_rows(Bs, b, k, y0, gc, 1, R - 1);
         const int keyL = s * (d.nz + 1) + k - 1, keyH = keyL + 2;
         sL = tag0 == keyL ? 0 : (tag1 == keyL ? 1 : -1);
         sH = tag0 == keyH ? 0 : (tag1 == keyH ? 1 : -1);
@@ -573,7 +433,7 @@ __global__ void __launch_bounds__(kPersMaxNx / 2, kPersMinBlocks)
                 tag0 = keyL;
             else
                 tag1 = keyL;
-            copy_rows(Zs0 + sL * plane_f, zsrc, k - 1, y0, 0, R);
+            copy_rows(Zs0 + sL * plane_f, zsrc, k - 1, y0, gc, 0, R);
         }
         if (sH < 0) {
             sH = 1 - sL;
@@ -581,7 +441,7 @@ __global__ void __launch_bounds__(kPersMaxNx / 2, kPersMinBlocks)
                 tag0 = keyH;
             else
                 tag1 = keyH;
-            copy_rows(Zs0 + sH * plane_f, zsrc, k + 1, y0, 0, R);
+            copy_rows(Zs0 + sH * plane_f, zsrc, k + 1, y0, gc, 0, R);
         }
         cp_async_commit();
     };
@@ -589,7 +449,7 @@ __global__ void __launch_bounds__(kPersMaxNx / 2, kPersMinBlocks)
     auto issue_p = [&](long n) {
         int s, k;
         tile_of(n, s, k);
-        copy_rows(Ps, vin, k, s * TY, 0, R);
+        copy_rows(Ps, vin, k, row0(s), chunk_col(col0(s)), 0, R);
         cp_async_commit();
     };
 
@@ -601,7 +461,10 @@ __global__ void __launch_bounds__(kPersMaxNx / 2, kPersMinBlocks)
         __syncthreads();
         int s, k;
         tile_of(n, s, k);
-        const int y0 = s * TY;
+        const int y0 = row0(s);
+        // this thread's columns in the grid; its pair is stored if in the tile
+        const int gx = col0(s) - (WIN ? kPersHalo : 0) + 2 * t;
+        const bool mine = !WIN || (t >= kPersHalo / 2 && t < hn - kPersHalo / 2 && gx < gnx);
         // right-hand side with the z-neighbour terms folded in
         float r[3][2][R];
         op.template fold<R>(r, Zs0 + sL * plane_f, Zs0 + sH * plane_f, Bs, q);
@@ -643,8 +506,8 @@ __global__ void __launch_bounds__(kPersMaxNx / 2, kPersMinBlocks)
             }
             if (RR) {
                 // full weighting R = T^T (weight 1 at offset 0, 1/2 at +-1 per
-                // axis), x and y parts: coarse column I = t takes fine
-                // x = 2t - 1 (the O node of thread t - 1), 2t, 2t + 1; coarse
+                // axis), x and y parts: coarse column I = gx / 2 takes
+                // fine x = gx - 1 (the O node of thread t - 1), gx, gx + 1; coarse
                 // row J = y0/2 + jc takes fine rows 2J - 1 .. 2J + 1, window
                 // rows 2 jc + 1 .. 2 jc + 3.  The O residuals go through the
                 // (now dead) plane rows in shared memory.
@@ -656,7 +519,7 @@ __global__ void __launch_bounds__(kPersMaxNx / 2, kPersMinBlocks)
                     for (int jj = 1; jj < NR; jj++) Xo[(c * NR + jj) * hn + t] = res[c][1][jj];
                 __syncthreads();
                 const int hny = ny >> 1;
-                const long pcs = (long)(d.nz + 1) * hny * hn;
+                const long pcs = (long)(d.nz + 1) * hny * ghn;
 #pragma unroll
                 for (int c = 0; c < 3; c++) {
                     float rx[NR];
@@ -667,8 +530,8 @@ __global__ void __launch_bounds__(kPersMaxNx / 2, kPersMinBlocks)
 #pragma unroll
                     for (int jc = 0; jc < TY / 2; jc++) {
                         const int J = (y0 >> 1) + jc;
-                        if (J < hny)
-                            vout[c * pcs + ((long)k * hny + J) * hn + t] =
+                        if (J < hny && mine)
+                            vout[c * pcs + ((long)k * hny + J) * ghn + (gx >> 1)] =
                                 (0.5f * rx[2 * jc + 1] + rx[2 * jc + 2]) + 0.5f * rx[2 * jc + 3];
                     }
                 }
@@ -717,11 +580,12 @@ __global__ void __launch_bounds__(kPersMaxNx / 2, kPersMinBlocks)
 #pragma unroll
         for (int jj = 1 + F; jj < TY + 1 + F; jj++) {
             const int y = y0 - 1 - F + jj;
-            if (!RR && y < ny) {
+            if (!RR && y < ny && mine) {
+                const int ge = SPLIT ? gx >> 1 : gx, go = SPLIT ? ghn + ge : gx + 1;
 #pragma unroll
                 for (int c = 0; c < 3; c++) {
-                    Ok[c * cs + (long)y * nx + q.xe] = P[c][0][jj];
-                    Ok[c * cs + (long)y * nx + q.xo] = P[c][1][jj];
+                    Ok[c * cs + (long)y * gnx + ge] = P[c][0][jj];
+                    Ok[c * cs + (long)y * gnx + go] = P[c][1][jj];
                 }
             }
         }
@@ -736,10 +600,15 @@ __global__ void __launch_bounds__(kPersMaxNx / 2, kPersMinBlocks)
 
 int g_sms[64];  // SM count per device, set by smoother_init
 
-// resident CTAs of the persistent kernel per SM: shared memory and registers
-// scale with the row length (two CTAs at nx = 256, four at 128, eight at 64)
-inline long pers_slots(int nx, int sms) {
-    return (long)sms * kPersMinBlocks * (kPersMaxNx / nx);
+// resident CTAs of the persistent kernel on the device with windows of W
+// columns: two an SM at 256, more of shorter rows (shared memory, 255 registers
+// a thread)
+inline long pers_slots(int W, int sms) {
+    const int threads = (W / 2 + 31) / 32 * 32;
+    const long smem = 227 * 1024 / (pers_floats(W) * (long)sizeof(float) + 1024);
+    const long regs = 65536 / (256 * threads);
+    const long n = smem < regs ? smem : regs;
+    return sms * (n < kPersMinBlocks ? kPersMinBlocks : n);
 }
 
 template <class OP, int F, bool SPLIT, bool RES, bool RR = false>
@@ -747,12 +616,20 @@ cudaError_t launch_rows_p(const Dims &d, const OP &op, const float *b, const flo
                           const float *zsrc, float *vout, int kbase, int kstep, int nplanes,
                           cudaStream_t s, int sms) {
     if (nplanes <= 0) return cudaSuccess;
-    const int nstrips = (d.ny + kPersTY - 1) / kPersTY;
+    // tiles: equal ones of a multiple of 8 columns
+    const bool win = d.nx > kPersMaxWide;
+    const int want = (d.nx + kPersMaxNx - 1) / kPersMaxNx;
+    const int xt = win ? ((d.nx + want - 1) / want + 7) / 8 * 8 : d.nx;
+    const int W = win ? xt + 2 * kPersHalo : d.nx;
+    const int nstrips = (d.ny + kPersTY - 1) / kPersTY * (win ? (d.nx + xt - 1) / xt : 1);
     const long ntiles = (long)nstrips * nplanes;
-    const long slots = pers_slots(d.nx, sms);
+    const long slots = !win && W > kPersMaxNx ? sms : pers_slots(W, sms);
     const int grid = (int)(ntiles < slots ? ntiles : slots);
-    k_gs_rows_p<OP, F, SPLIT, RES, RR><<<grid, d.nx / 2, pers_floats(d.nx) * sizeof(float), s>>>(
-        d, op, b, vin, zsrc, vout, kbase, kstep, nplanes, nstrips);
+    const size_t smem = pers_floats(W) * sizeof(float);
+    auto *kernel = win                ? k_gs_rows_p<OP, F, SPLIT, kTiles, RES, RR>
+                   : W > kPersMaxNx ? k_gs_rows_p<OP, F, SPLIT, kWide, RES, RR>
+                                      : k_gs_rows_p<OP, F, SPLIT, kRows, RES, RR>;
+    kernel<<<grid, W / 2, smem, s>>>(d, op, b, vin, zsrc, vout, kbase, kstep, nplanes, nstrips, xt);
     count_launch();
     return cudaGetLastError();
 }
@@ -1129,7 +1006,11 @@ bool rows_p_shape(const Dims &d, int &sms) {
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return false;
     sms = (dev >= 0 && dev < 64) ? g_sms[dev] : 0;
-    return sms > 0 && d.nx % 64 == 0 && d.nx <= kPersMaxNx && d.ny >= kPersR;
+    return sms > 0 && d.nx % (d.nx > kPersMaxNx ? 8 : 4) == 0 && d.nx >= 16 && d.ny >= kPersR;
+}
+// ... and the fused sweep (rows of 64, 128, 192 or 256 nodes)
+bool rows_f_shape(const Dims &d, int &sms) {
+    return rows_p_shape(d, sms) && d.nx % 64 == 0 && d.nx <= kPersMaxNx;
 }
 // ... and these arrays (16-byte aligned for the copies)
 bool rows_p_ok(const Dims &d, const void *a, const void *b, const void *c, int &sms) {
@@ -1147,26 +1028,29 @@ cudaError_t smoother_init() {
         e = cudaDeviceGetAttribute(&g_sms[dev], cudaDevAttrMultiProcessorCount, dev);
         if (e != cudaSuccess) return e;
     }
-    const int smem = (int)rows_smem(kRowsMaxThreads);
     const int smem_p = (int)(pers_floats(kPersMaxNx) * sizeof(float));
 #define SET(kern, bytes)                                                                   \
     if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes)) != \
         cudaSuccess)                                                                       \
         return e;
-    SET((k_gs_rows<kRowsTY, 0, false>), smem)
-    SET((k_gs_rows<kRowsTY, 0, true>), smem)
-    SET((k_gs_rows<kRowsTY, 1, false>), smem)
-    SET((k_gs_rows<kRowsTY, 1, true>), smem)
-    SET((k_gs_rows_p<FineRowsOp, 0, false, false>), smem_p)
-    SET((k_gs_rows_p<FineRowsOp, 0, true, false>), smem_p)
-    SET((k_gs_rows_p<FineRowsOp, 1, false, false>), smem_p)
-    SET((k_gs_rows_p<FineRowsOp, 1, true, false>), smem_p)
-    SET((k_gs_rows_p<FineRowsOp, 0, false, true>), smem_p)
-    SET((k_gs_rows_p<FineRowsOp, 0, true, true>), smem_p)
-    SET((k_gs_rows_p<FineRowsOp, 1, false, true, true>), smem_p)
-    SET((k_gs_rows_p<FineRowsOp, 1, true, true, true>), smem_p)
-    SET((k_gs_rows_p<CoarseRowsOp, 0, false, false>), smem_p)
-    SET((k_gs_rows_p<CoarseRowsOp, 1, false, false>), smem_p)
+    const int smem_w = (int)(pers_floats(kPersMaxW) * sizeof(float));
+    const int smem_l = (int)(pers_floats(kPersMaxWide) * sizeof(float));
+#define SET_P(OP, F, SPLIT, RES, RR)                                 \
+    SET((k_gs_rows_p<OP, F, SPLIT, kRows, RES, RR>), smem_p)         \
+    SET((k_gs_rows_p<OP, F, SPLIT, kWide, RES, RR>), smem_l)         \
+    SET((k_gs_rows_p<OP, F, SPLIT, kTiles, RES, RR>), smem_w)
+    SET_P(FineRowsOp, 0, false, false, false)
+    SET_P(FineRowsOp, 0, true, false, false)
+    SET_P(FineRowsOp, 1, false, false, false)
+    SET_P(FineRowsOp, 1, true, false, false)
+    SET_P(FineRowsOp, 0, false, true, false)
+    SET_P(FineRowsOp, 0, true, true, false)
+    SET_P(FineRowsOp, 1, false, true, true)
+    SET_P(FineRowsOp, 1, true, true, true)
+    SET_P(CoarseRowsOp, 0, false, false, false)
+    SET_P(CoarseRowsOp, 1, false, false, false)
+    SET_P(CoarseRowsOp, 1, false, true, true)
+#undef SET_P
     const int smem_f = smem_p;
     SET((k_gs_rows_f<0, false>), smem_f)
     SET((k_gs_rows_f<0, true>), smem_f)
@@ -1196,7 +1080,7 @@ cudaError_t smoother_init() {
 
 bool fused_sweep_sizes(const Dims &d, long &naflag) {
     int sms = 0, dev = 0;
-    if (!rows_p_shape(d, sms) || cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64)
+    if (!rows_f_shape(d, sms) || cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64)
         return false;
     if (fused_k(d, g_fused_slots[dev][d.nx / 64 - 1]) < 1) return false;
     naflag = (long)fused_nstrips(d) * (d.nz / 2 + 1);
@@ -1212,7 +1096,7 @@ cudaError_t gs_sweep_fine_rows(const Dims &d, const Fine<float> &f, const float 
     if (rows_p_ok(d, b, vin, vout, sms)) {
         const FineRowsOp op{f};
         int dev = 0;
-        const int kz = sync && cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < 64
+        const int kz = sync && rows_f_shape(d, sms) && cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < 64
                            ? fused_k(d, g_fused_slots[dev][d.nx / 64 - 1])
                            : 0;
         if (kz > 0) {
@@ -1227,16 +1111,7 @@ cudaError_t gs_sweep_fine_rows(const Dims &d, const Fine<float> &f, const float 
         return split ? rows_p_sweep<FineRowsOp, true>(d, op, b, vin, vout, descending, s, sms)
                      : rows_p_sweep<FineRowsOp, false>(d, op, b, vin, vout, descending, s, sms);
     }
-    if (d.nx / 2 > kRowsMaxThreads) return cudaErrorNotSupported;
-    cudaError_t e;
-    if (!descending) {
-        e = rows_phase<0>(d, f, b, vin, vin, vout, 0, s, split);
-        if (e != cudaSuccess) return e;
-        return rows_phase<0>(d, f, b, vin, vout, vout, 1, s, split);
-    }
-    e = rows_phase<1>(d, f, b, vin, vin, vout, 1, s, split);
-    if (e != cudaSuccess) return e;
-    return rows_phase<1>(d, f, b, vin, vout, vout, 0, s, split);
+    return cudaErrorNotSupported;
 }
 
 // FP32 finest-level residual r = b - A x (interior planes) with the
@@ -1274,11 +1149,22 @@ cudaError_t residual_restrict_fine_rows(const Dims &d, const Fine<float> &f, con
     return restrict_z(d, part, bc, s);
 }
 
-// Coarse levels take the row strips only where they win (measured on GB300,
-// 27-point stencil, FMA-issue bound in every form): rows of 128 nodes and up
-// (128^3 level: 98 us a sweep against 103 us for eight colour launches); at
-// 64^3 the tile kernel is faster (35 against 49 us), and the coarse residual
-// stays one thread per node (55 against 59 us at 128^3).
+// the same on a coarse level (its sizes even, natural column order)
+cudaError_t residual_restrict_coarse_rows(const Dims &d, const Coarse<float> &c, const float *b,
+                                          const float *x, float *part, float *bc,
+                                          cudaStream_t s) {
+    int sms = 0;
+    if (!coarse_rows_fit(d) || (d.ny & 1) || d.nz < 4 || (d.nz & 1) ||
+        !rows_p_ok(d, b, x, part, sms))
+        return cudaErrorNotSupported;
+    const CoarseRowsOp op{c};
+    const cudaError_t e = launch_rows_p<CoarseRowsOp, 1, false, true, true>(
+        d, op, b, x, x, part, 1, 1, d.nz - 1, s, sms);
+    return e == cudaSuccess ? restrict_z(d, part, bc, s) : e;
+}
+
+// Coarse levels take these strips at rows of 128 nodes and up; below, the
+// strips of strip.cu are faster.
 bool coarse_rows_fit(const Dims &d) {
     int sms = 0;
     return d.nx >= 128 && rows_p_shape(d, sms);
