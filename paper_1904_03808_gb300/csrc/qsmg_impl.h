@@ -160,7 +160,7 @@ constexpr int kSmallLevels = 6, kSmallCoarse = 768;
 struct SmallLevel {
     int nx, ny, nz, np, ppc;  // np = nx ny; ppc: interior planes per CTA
     int hx, w, pl;            // nx / 2 (0: coarsest), row pitch, plane size
-    unsigned mnx, mnp, mhx, mnh, mppc, mpl;
+    unsigned mnx, mnp, mhx, mnh, mppc, mn3;
     int x, b, p;  // x, right-hand side, x-y restricted residual
 };
 template <typename T>

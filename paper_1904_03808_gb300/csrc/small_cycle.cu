@@ -9,8 +9,8 @@
 //     their x and b in shared memory for the whole launch, with copies (halos)
 //     of the plane below and the plane above them; only the top level's
 //     arrays are read from and written to global memory;
-//   - an updated plane is copied through distributed shared memory to the
-//     halos that mirror it, and a cluster barrier (0.2 us measured, against
+//   - an update is stored (FP64: an updated plane is copied) through distributed
+//     shared memory to the halos that mirror it too, and a cluster barrier (0.2 us measured, against
 //     1.2 us for a grid-wide one) takes the place of a launch boundary;
 //   - a sweep is the two phases of smoother_fast.cu, planes of one k-parity
 //     and then of the other: the dz = +-1 part of the 27-point operator is
@@ -26,18 +26,18 @@
 // What bounds it: latency.  At 16^3 a phase is about 2.5 k clocks -- 600 for
 // the folded rows, 4 x 250 for the passes, 900 for the barrier and the copies
 // before it -- and at 32^3 the shared-memory loads add to that.  One FP32
-// V-cycle from 32^3 (32^3, 16^3, 8^3 and the 4^3 solve) takes 78 us against
-// about 250 us as 40 launches in a CUDA graph, one from 16^3 31 against
+// V-cycle from 32^3 (32^3, 16^3, 8^3 and the 4^3 solve) takes 75 us against
+// about 250 us as 40 launches in a CUDA graph, one from 16^3 28 against
 // 150 us.  FP64 is bound by the pipe besides (kSmallNodes64): the cycle from
 // 16^3 takes 127 us (176 with three components a thread) against 780 us.  Slower forms measured on the way, per cycle
-// from 32^3: neighbour planes read remotely at the start of a phase 89 us,
+// from 32^3: three words a node instead of one 16-byte access 78 us,
+// neighbour planes read remotely at the start of a phase 89 us,
 // one thread per component with the 116-operation form of the fold 123 us,
 // halos written by the single updates 92 us.
 //
 // Shared planes are [row][column][component] with the columns in parity-split
-// order and a row pitch w with 2 w = 3 nx/2 (mod 32 banks): threads own nodes
-// in colour-major order, so the 32 nodes of a warp, 3 words apart along a
-// row and 2 w from row to row, fall into 32 different banks.
+// order and a row pitch by which the nodes of a warp, which threads own in
+// colour-major order, fall into different banks.
 #include <cooperative_groups.h>
 
 #include <vector>
@@ -58,6 +58,30 @@ __device__ __forceinline__ int fdiv(int t, unsigned m) {
     return m ? (int)__umulhi((unsigned)t, m) : t;
 }
 
+// Elements of a node in a shared plane: in FP32 its three components and one
+// more, so that a node is one 16-byte load or store (8 loads of a node's
+// neighbours instead of 24, 6 instead of 18 for the fold)
+template <typename T>
+constexpr int kNode = sizeof(T) == 4 ? 4 : 3;
+
+__device__ __forceinline__ void load3(const float *p, float (&v)[3]) {
+    const float4 q = *reinterpret_cast<const float4 *>(p);
+    v[0] = q.x;
+    v[1] = q.y;
+    v[2] = q.z;
+}
+__device__ __forceinline__ void load3(const double *p, double (&v)[3]) {
+#pragma unroll
+    for (int a = 0; a < 3; a++) v[a] = p[a];
+}
+__device__ __forceinline__ void store3(float *p, const float (&v)[3]) {
+    *reinterpret_cast<float4 *>(p) = make_float4(v[0], v[1], v[2], 0.f);
+}
+__device__ __forceinline__ void store3(double *p, const double (&v)[3]) {
+#pragma unroll
+    for (int a = 0; a < 3; a++) p[a] = v[a];
+}
+
 // A node of a plane, in the colour-major order in which threads own nodes
 // (colour, then row, then column of the colour's quarter of the plane: a warp
 // works on one colour), with the element offsets of its columns and rows at
@@ -68,8 +92,9 @@ struct Node {
 };
 
 // offset of column i in a row of level L (parity-split where it is smoothed)
+template <typename T>
 __device__ __forceinline__ int col_of(const SmallLevel &L, int i) {
-    return 3 * (L.hx ? (i & 1) * L.hx + (i >> 1) : i);
+    return kNode<T> * (L.hx ? (i & 1) * L.hx + (i >> 1) : i);
 }
 
 // The dz = +-1 part of the 27-point operator (coarse_z_terms) is separable
@@ -82,14 +107,16 @@ __device__ __forceinline__ void z_row(const Coarse<T> &c, const T *lo, const T *
                                       T A[3], T U[3], T V[3]) {
     T S[3][3], D[3][3];  // [column][component]
 #pragma unroll
-    for (int x = 0; x < 3; x++)
+    for (int x = 0; x < 3; x++) {
+        T l[3], h[3];
+        load3(lo + n.r[1] + n.c[x], l);
+        load3(hi + n.r[1] + n.c[x], h);
 #pragma unroll
         for (int a = 0; a < 3; a++) {
-            const int q = n.r[1] + n.c[x] + a;
-            const T l = lo[q], h = hi[q];
-            S[x][a] = h + l;
-            D[x][a] = h - l;
+            S[x][a] = h[a] + l[a];
+            D[x][a] = h[a] - l[a];
         }
+    }
     T B[3], G[3];
 #pragma unroll
     for (int a = 0; a < 3; a++) {
@@ -116,7 +143,13 @@ __device__ __forceinline__ void z_row(const Coarse<T> &c, const T *lo, const T *
 // sum over the 8 in-plane offsets at node n of plane P
 template <typename T>
 __device__ __forceinline__ void plane_at(const Coarse<T> &c, const T *P, const Node &n, T o[3]) {
-    auto u = [&](int b, int dx, int dy) -> T { return P[n.r[dy + 1] + n.c[dx + 1] + b]; };
+    T v[3][3][3];  // [row][column][component]
+#pragma unroll
+    for (int y = 0; y < 3; y++)
+#pragma unroll
+        for (int x = 0; x < 3; x++)
+            if (x != 1 || y != 1) load3(P + n.r[y] + n.c[x], v[y][x]);
+    auto u = [&](int b, int dx, int dy) -> T { return v[dy + 1][dx + 1][b]; };
     coarse_plane_terms(c, u, o);
 }
 
@@ -223,9 +256,9 @@ struct Walker {
             const int i = 2 * ih + (q & 1), j = 2 * jh + (q >> 1);
             Node &n = node[u];
             n.colour = t < own ? q : -1;
-            n.c[0] = col_of(L, i ? i - 1 : L.nx - 1);
-            n.c[1] = col_of(L, i);
-            n.c[2] = col_of(L, i + 1 < L.nx ? i + 1 : 0);
+            n.c[0] = col_of<T>(L, i ? i - 1 : L.nx - 1);
+            n.c[1] = col_of<T>(L, i);
+            n.c[2] = col_of<T>(L, i + 1 < L.nx ? i + 1 : 0);
             n.r[0] = L.w * (j ? j - 1 : L.ny - 1);
             n.r[1] = L.w * j;
             n.r[2] = L.w * (j + 1 < L.ny ? j + 1 : 0);
@@ -239,18 +272,17 @@ struct Walker {
 #pragma unroll
         for (int u = 0; u < NODES; u++) {
             if (node[u].colour < 0) continue;
-            T up[NC], vp[NC];
+            T up[NC], vp[NC], bp[NC];
+            const int o = node[u].r[1] + node[u].c[1] + comp[u];
             if constexpr (COMP)
                 z_row_c(c, lo, hi, node[u], comp[u], r[u][0], up[0], vp[0]);
             else
                 z_row(c, lo, hi, node[u], r[u], up, vp);
-            const int o = node[u].r[1] + node[u].c[1] + comp[u];
+            put(U + o, up);
+            put(V + o, vp);
+            get(b + o, bp);
 #pragma unroll
-            for (int a = 0; a < NC; a++) {
-                U[o + a] = up[a];
-                V[o + a] = vp[a];
-                r[u][a] = b[o + a] - r[u][a];
-            }
+            for (int a = 0; a < NC; a++) r[u][a] = bp[a] - r[u][a];
         }
         sync_act();
 #pragma unroll
@@ -258,9 +290,25 @@ struct Walker {
             if (node[u].colour < 0) continue;
             const int om = node[u].r[0] + node[u].c[1] + comp[u],
                       op = node[u].r[2] + node[u].c[1] + comp[u];
+            T up[NC], vp[NC];
+            get(U + om, up);
+            get(V + op, vp);
 #pragma unroll
-            for (int a = 0; a < NC; a++) r[u][a] -= U[om + a] + V[op + a];
+            for (int a = 0; a < NC; a++) r[u][a] -= up[a] + vp[a];
         }
+    }
+    // the owned components of a node
+    __device__ __forceinline__ static void get(const T *p, T (&v)[NC]) {
+        if constexpr (COMP)
+            v[0] = p[0];
+        else
+            load3(p, v);
+    }
+    __device__ __forceinline__ static void put(T *p, const T (&v)[NC]) {
+        if constexpr (COMP)
+            p[0] = v[0];
+        else
+            store3(p, v);
     }
     // the in-plane terms at own node u
     __device__ __forceinline__ void in_plane(const Coarse<T> &c, const T *P, int u,
@@ -291,11 +339,8 @@ struct Walker {
                     if (zero && s == 0) {
 #pragma unroll
                         for (int u = 0; u < NODES; u++)
-#pragma unroll
-                            for (int a = 0; a < NC; a++)
-                                r[u][a] = node[u].colour < 0
-                                              ? T(0)
-                                              : b[node[u].r[1] + node[u].c[1] + comp[u] + a];
+                            if (node[u].colour >= 0)
+                                get(b + node[u].r[1] + node[u].c[1] + comp[u], r[u]);
                     } else {
                         fold(c, b, P - pl, P + pl, r);
                     }
@@ -312,12 +357,17 @@ struct Walker {
                             const int e = node[u].r[1] + node[u].c[1] + comp[u];
 #pragma unroll
                             for (int a = 0; a < NC; a++)
-                                P[e + a] = c.dinv[comp[u] + a] * (r[u][a] - o[a]);
+                                o[a] = c.dinv[comp[u] + a] * (r[u][a] - o[a]);
+                            put(P + e, o);
+                            if constexpr (!COMP) {
+                                if (h0) put(h0 + e, o);
+                                if (h1) put(h1 + e, o);
+                            }
                         }
                     }
-                    // 16 bytes at a time: the scattered stores of the single
-                    // updates cost more than this pass over the plane
-                    if (h0 || h1) {
+                    // FP64: 16 bytes at a time after the passes, which takes less
+                    // than scattered stores of the single components
+                    if (COMP && (h0 || h1)) {
                         sync_act();
                         const float4 *src = reinterpret_cast<const float4 *>(P);
                         for (int e = tid; e < pl * (int)sizeof(T) / 16; e += act) {
@@ -352,9 +402,12 @@ struct Walker {
                     T o[NC];
                     in_plane(c, P, u, o);
                     const int q = node[u].r[1] + node[u].c[1] + comp[u];
+                    T x[NC];
+                    get(P + q, x);
 #pragma unroll
                     for (int a = 0; a < NC; a++)
-                        R[q + a] = r[u][a] - (o[a] + c.cd[comp[u] + a][0] * P[q + a]);
+                        o[a] = r[u][a] - (o[a] + c.cd[comp[u] + a][0] * x[a]);
+                    put(R + q, o);
                 }
                 sync_act();
                 // x and y parts of the full weighting
@@ -362,14 +415,15 @@ struct Walker {
                 for (int e = tid; e < nc3; e += act) {
                     const int m = e / 3, a = e - 3 * m;
                     const int J = fdiv(m, C.mnx), I = m - J * C.nx;
-                    const int im = 3 * (L.hx + (I ? I - 1 : L.hx - 1)) + a, i0 = 3 * I + a,
-                              ip = i0 + 3 * L.hx;
+                    constexpr int N = kNode<T>;
+                    const int im = N * (L.hx + (I ? I - 1 : L.hx - 1)) + a, i0 = N * I + a,
+                              ip = i0 + N * L.hx;
                     const T *r0 = R + 2 * J * L.w, *rm = R + (J ? 2 * J - 1 : L.ny - 1) * L.w,
                             *rp = r0 + L.w;
                     const T tm = (T(0.5) * rm[im] + rm[i0]) + T(0.5) * rm[ip];
                     const T t0 = (T(0.5) * r0[im] + r0[i0]) + T(0.5) * r0[ip];
                     const T tp = (T(0.5) * rp[im] + rp[i0]) + T(0.5) * rp[ip];
-                    p[J * C.w + col_of(C, I) + a] = (T(0.5) * tm + t0) + T(0.5) * tp;
+                    p[J * C.w + col_of<T>(C, I) + a] = (T(0.5) * tm + t0) + T(0.5) * tp;
                 }
                 sync_act();
             }
@@ -397,7 +451,6 @@ struct Walker {
     // x of level l += T x of level l+1
     __device__ __forceinline__ void prolong(int l) {
         const SmallLevel &L = g.lev[l], &C = g.lev[l + 1];
-        const int n3 = 3 * L.np;
         const int k0 = first(l), k1 = last(l);
         T *Z = sm + g.scratch;  // the coarse planes averaged to each own plane's z
         for (int k = k0; k < k1; k++) {
@@ -408,24 +461,29 @@ struct Walker {
                 Z[(k - k0) * C.pl + e] = T(0.5) * ((lo ? lo[e] : T(0)) + (hi ? hi[e] : T(0)));
         }
         __syncthreads();
-        for (int k = k0; k < k1; k++) {
-            T *X = own(l, L.x, k);
-            T *h0 = k == k0 ? halo(l, 0) : nullptr;
-            T *h1 = k - k0 == L.ppc - 1 ? halo(l, 1) : nullptr;
-            const T *z = Z + (k - k0) * C.pl;
-            for (int e = tid; e < n3; e += nt) {
-                const int m = e / 3, a = e - 3 * m;
-                const int j = fdiv(m, L.mnx), i = m - j * L.nx;
-                const int I = i >> 1, J = j >> 1;
-                const int c0 = col_of(C, I), c1 = (i & 1) ? col_of(C, I + 1 < C.nx ? I + 1 : 0) : c0;
-                const T *z0 = z + J * C.w + a,
-                        *z1 = (j & 1) ? z + (J + 1 < C.ny ? J + 1 : 0) * C.w + a : z0;
-                const int q = j * L.w + col_of(L, i) + a;
-                const T v = X[q] + T(0.25) * ((z0[c0] + z0[c1]) + (z1[c0] + z1[c1]));
-                X[q] = v;
-                if (h0) h0[q] = v;
-                if (h1) h1[q] = v;
-            }
+        T *const below = halo(l, 0), *const above = halo(l, 1);
+        for (int e = tid; e < (k1 - k0) * L.np; e += nt) {
+            const int p = fdiv(e, L.mnp), m = e - p * L.np;
+            const int j = fdiv(m, L.mnx), i = m - j * L.nx;
+            const int I = i >> 1, J = j >> 1;
+            const int c0 = col_of<T>(C, I),
+                      c1 = (i & 1) ? col_of<T>(C, I + 1 < C.nx ? I + 1 : 0) : c0;
+            const T *z0 = Z + p * C.pl + J * C.w,
+                    *z1 = (j & 1) ? Z + p * C.pl + (J + 1 < C.ny ? J + 1 : 0) * C.w : z0;
+            const int q = j * L.w + col_of<T>(L, i);
+            T *X = sm + L.x + p * L.pl + q;
+            T v[3], z00[3], z01[3], z10[3], z11[3];
+            load3(X, v);
+            load3(z0 + c0, z00);
+            load3(z0 + c1, z01);
+            load3(z1 + c0, z10);
+            load3(z1 + c1, z11);
+#pragma unroll
+            for (int a = 0; a < 3; a++)
+                v[a] += T(0.25) * ((z00[a] + z01[a]) + (z10[a] + z11[a]));
+            store3(X, v);
+            if (below && p == 0) store3(below + q, v);
+            if (above && p == L.ppc - 1) store3(above + q, v);
         }
         cl.sync();
         clear(l + 1);  // for the next cycle
@@ -433,11 +491,12 @@ struct Walker {
 
     // x = Ainv b on the coarsest level (x = 0 before): every CTA gathers b
     // and takes every 16th row, 16 lanes a row, FP64 sums in a fixed order.
-    // The unknowns are ordered as the arrays are: plane, node, component.
+    // The unknowns are ordered plane, node, component.
     __device__ __forceinline__ void coarsest() {
         const int l = g.nlev - 1;
         const SmallLevel &L = g.lev[l];
-        const int n3 = L.pl, lane = tid & 15, ng = nt >> 4, n = g.ncoarse;
+        const int n3 = 3 * L.np, lane = tid & 15, ng = nt >> 4, n = g.ncoarse;
+        auto at = [](int m3) { return kNode<T> == 3 ? m3 : m3 + m3 / 3; };  // place in a plane
         double *v = reinterpret_cast<double *>(sm + g.scratch);
         // the first row's leading entries, loaded while b is on its way
         constexpr int PRE = 9;
@@ -450,8 +509,8 @@ struct Walker {
         }
         cl.sync();
         for (int e = tid; e < n; e += nt) {
-            const int K1 = fdiv(e, L.mpl);
-            v[e] = (double)plane(l, L.b, K1 + 1, n3)[e - K1 * n3];
+            const int K1 = fdiv(e, L.mn3);
+            v[e] = (double)plane(l, L.b, K1 + 1, L.pl)[at(e - K1 * n3)];
         }
         __syncthreads();
         for (int t0 = 0; t0 < n; t0 += kCta * ng) {  // uniform: the shuffles need whole warps
@@ -470,8 +529,8 @@ struct Walker {
 #pragma unroll
             for (int o = 8; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o, 16);
             if (lane == 0 && u < n) {
-                const int K1 = fdiv(u, L.mpl);
-                plane(l, L.x, K1 + 1, n3)[u - K1 * n3] = (T)acc;
+                const int K1 = fdiv(u, L.mn3);
+                plane(l, L.x, K1 + 1, L.pl)[at(u - K1 * n3)] = (T)acc;
             }
         }
         cl.sync();
@@ -493,7 +552,7 @@ __global__ void __launch_bounds__(MAXT, 1)
     for (int e = w.tid; e < (k1 > k0 ? k1 - k0 + 2 : 0) * n3; e += w.nt) {
         const int t = fdiv(e, L.mnp), m = e - t * L.np, q = t / 3, a = t - 3 * q;
         const int j = fdiv(m, L.mnx), i = m - j * L.nx, k = k0 - 1 + q;
-        const int s = j * L.w + col_of(L, i) + a;
+        const int s = j * L.w + col_of<T>(L, i) + a;
         const long gq = a * cs + k * ps + m;
         w.own(0, L.x, k)[s] = from_zero ? T(0) : x[gq];
         if (k >= k0 && k < k1) w.own(0, L.b, k)[s] = b[gq];
@@ -520,7 +579,7 @@ __global__ void __launch_bounds__(MAXT, 1)
     for (int e = w.tid; e < (k1 - k0) * n3; e += w.nt) {
         const int t = fdiv(e, L.mnp), m = e - t * L.np, q = t / 3, a = t - 3 * q;
         const int j = fdiv(m, L.mnx), i = m - j * L.nx;
-        x[a * cs + (k0 + q) * ps + m] = w.own(0, L.x, k0 + q)[j * L.w + col_of(L, i) + a];
+        x[a * cs + (k0 + q) * ps + m] = w.own(0, L.x, k0 + q)[j * L.w + col_of<T>(L, i) + a];
     }
     // no CTA leaves while another may still store into its shared memory
     w.cl.sync();
@@ -547,10 +606,11 @@ void configure(const SmallPlan<T> &g, cudaLaunchConfig_t &cfg, cudaLaunchAttribu
 // plane (FP32: nodes, FP64: node components) and `nodes` of them go to a
 // thread.  Few threads leave each more registers, which hold a level's
 // constants and node offsets across its phases (16^3 step: 796 us with 128 of
-// them against 870 with 64); on 32 x 32 planes 512 threads with two nodes
-// each also pass barriers sooner (64^3 solve 2.83 against 2.92 ms), on planes
-// of 576 and 800 nodes one node a thread stays faster (5.07 against 5.15 ms,
-// 10.41 against 10.53 ms).
+// them against 870 with 64; 80 x 40 x 40 and 48^3 levels' planes of 800 and 576
+// nodes gain 1 and 2% of a step from bounds of 832 and 640 instead of 1024); on
+// 32 x 32 planes 512 threads with two nodes each also pass barriers sooner
+// (64^3 solve 2.83 against 2.92 ms), on the smaller ones one node a thread
+// stays faster.
 template <typename T>
 using SmallFn = void (*)(SmallPlan<T>, const T *, T *, int, int);
 template <typename T>
@@ -565,7 +625,8 @@ const std::vector<SmallKernel<float>> &small_kernels() {
     static const std::vector<SmallKernel<float>> k = {
         {k_small_cycle<float, 1, 256>, 256, 1},
         {k_small_cycle<float, 1, 512>, 512, 1},
-        {k_small_cycle<float, 1, 1024>, 960, 1},
+        {k_small_cycle<float, 1, 640>, 640, 1},
+        {k_small_cycle<float, 1, 832>, 832, 1},
         {k_small_cycle<float, 2, 512>, 1024, 2},
         {k_small_cycle<float, kMaxNodes, 640>, 640 * kMaxNodes, kMaxNodes}};
     return k;
@@ -583,7 +644,10 @@ const std::vector<SmallKernel<double>> &small_kernels() {
 template <typename T>
 bool small_layout(const Dims *d, const Coarse<T> *op, int nlev, bool pad, SmallPlan<T> &g) {
     long off = 0;
-    const int banks = 128 / sizeof(T);  // elements a shared-memory wavefront serves
+    constexpr int N = kNode<T>;
+    // nodes a shared-memory wavefront serves: eight of 16 bytes in FP32, the
+    // banks of 16 elements three apart in FP64
+    const int unit = N == 4 ? 8 : 16;
     for (int l = 0; l < nlev; l++) {
         SmallLevel &L = g.lev[l];
         g.op[l] = op[l];
@@ -595,16 +659,20 @@ bool small_layout(const Dims *d, const Coarse<T> *op, int nlev, bool pad, SmallP
         L.mnx = magic(L.nx);
         L.mnp = magic(L.np);
         L.mppc = magic(L.ppc);
-        L.w = 3 * L.nx;
+        L.mn3 = magic(3 * L.np);
+        L.w = N * L.nx;
         if (l + 1 < nlev) {
             L.hx = L.nx / 2;
             L.mhx = magic(L.hx);
             L.mnh = magic(L.np / 4);
-            while (pad && (2 * L.w - 3 * L.hx) % banks > 1) L.w++;
+            // two rows of a colour apart, as if its lanes went on in one row
+            if (N == 4)
+                while (pad && (2 * (L.w / N) - L.hx) % unit > 1) L.w += N;
+            else
+                while (pad && (2 * L.w - N * L.hx) % unit > 1) L.w++;
         }
         L.pl = L.ny * L.w;
         if (l + 1 < nlev) L.pl = (L.pl + 3) & ~3;  // planes are copied 16 bytes at a time
-        L.mpl = magic(L.pl);
     }
     for (int l = 0; l < nlev; l++) {
         SmallLevel &L = g.lev[l];
