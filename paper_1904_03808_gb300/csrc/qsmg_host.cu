@@ -482,15 +482,20 @@ mg_status sweeps(mg_ctx *ctx, int l, const T *b, T *x, int n, bool descending) {
     return MG_OK;
 }
 
-// FP32: the two-phase kernels (row strips where the rows fit, else tiles),
-// except on large coarse levels without row strips, where the 27-point tile
-// kernel (128 registers, 2 CTAs per SM) loses to colour launches (measured on
-// GB300 at 128^2 planes: 71 us per phase launch against 4 x 13 us)
+// FP32: the two-phase kernels (strips, persistent row strips, tiles), except
+//  - on large coarse levels without row strips, where the 27-point tile kernel
+//    (128 registers, 2 CTAs per SM) loses to colour launches (71 us per phase
+//    launch against 4 x 13 us at 128^2 planes);
+//  - on arrays that are not 16-byte aligned (a caller's, through mg_smooth),
+//    unless the strips take the level: they and the colour launches read
+//    single words, the row strips copy 16 bytes and the tiles pairs.
 template <>
 mg_status sweeps<float>(mg_ctx *ctx, int l, const float *b, float *x, int n, bool descending) {
     const Dims &d = ctx->L[l];
+    const bool odd = (((uintptr_t)b | (uintptr_t)x) & 15) != 0;
     const bool colour = (ctx->opts.flags & MG_FLAG_COLOUR_PASSES) ||
-                        (l > 0 && (long)d.nx * d.ny >= 128L * 128L && !coarse_rows_fit(d));
+                        (l > 0 && (long)d.nx * d.ny >= 128L * 128L && !coarse_rows_fit(d)) ||
+                        (odd && !(strip_fits<float>(d, l == 0) && !(l == 0 && ctx->has_sync)));
     if (!colour) return sweeps_tiled(ctx, l, b, x, n, descending);
     return sweeps_colour<float>(ctx, l, b, x, n, descending);
 }

@@ -57,3 +57,24 @@ def test_tiles_match_oracle(shape):
             assert np.array_equal(got[:, [0, nz]], x[:, [0, nz]])
             assert rel(got, y) <= 2e-6, (l, descending)
     ctx.close()
+
+
+@pytest.mark.parametrize("shape,level", [((320, 256, 64), 1), ((144, 48, 32), 0),
+                                         ((64, 64, 16), 1)])
+def test_arrays_at_odd_words(shape, level):
+    """Caller's arrays that start on any word are taken, with the result of
+    aligned ones (up to the rounding of another kernel, 1e-6 as between the
+    other pairs of kernels)."""
+    rng = np.random.default_rng(9)
+    ctx = Context(*shape, 2e-2 / shape[0], K, MU, precision=MG_MIXED)
+    nx, ny, nz = ctx.level_dims(level)
+    n = 3 * (nz + 1) * ny * nx
+    b, x = (torch.from_numpy(rng.uniform(-1, 1, n).astype(np.float32)).cuda() for _ in range(2))
+    b1, x1 = torch.empty(n + 1, device="cuda"), torch.empty(n + 1, device="cuda")
+    b1[1:] = b
+    x1[1:] = x
+    sh = (3, nz + 1, ny, nx)
+    ctx.smooth(level, b.view(sh), x.view(sh), 2, False)
+    ctx.smooth(level, b1[1:].view(sh), x1[1:].view(sh), 2, False)
+    assert rel(x1[1:].cpu().numpy(), x.cpu().numpy()) <= 1e-6
+    ctx.close()
