@@ -256,7 +256,9 @@ __device__ __forceinline__ void correct_cell(const CellConst &w, const double (&
     s6[5] = fma(w.mu, G[0][1] + G[1][0], ss[5]);
 }
 
-// Eq. (27) over a column chunk of cells
+// Eq. (27) over a column chunk of cells.  FP64 instructions bound it (its 144
+// bytes a cell take 0.36 ms at 256^3): 4.16 ms there, 5.94 with the gradient
+// unshifted, both exponentials in FP64 and 32 x 8 thread blocks.
 __global__ void __launch_bounds__(128)
     k_stress_predict(StepParams p, CellConst w, StzConst c, int chunk, const double *__restrict__ v,
                      const double *__restrict__ sig, const double *__restrict__ chi,
@@ -284,7 +286,7 @@ __global__ void __launch_bounds__(128)
 // the STZ rate of those extrapolated values
 // A thread marches a column in z: a z face's flux serves the cells below and
 // above it.  The products of constants are formed on the host -- three FP64
-// divisions a cell were half of this kernel.
+// divisions a cell were half of this kernel: 0.68 ms at 256^3, 1.73 before.
 struct ChiConst {
     double grow, diff;  // 2 dt / (c0 s_Y);  dt l^2 / (2 c0 h^2)
     double chi_inf;
@@ -341,7 +343,8 @@ __global__ void __launch_bounds__(128)
 // contributions -- the x-differences of sigma_a0 plus the y-differences of
 // sigma_a1, and the layer sum of sigma_a2 over the 2 x 2 cells around the
 // column -- are formed once and shared by the corners below and above the
-// layer (FP64 is add-bound here: 40 instructions a corner instead of 72)
+// layer (FP64 is add-bound here: 40 instructions a corner instead of 72);
+// 1.33 ms at 256^3, 1.49 with one z chunk length and 32 x 8 blocks
 struct DivLayer {
     double XY[3], Z[3];
 };
@@ -604,7 +607,9 @@ __device__ __forceinline__ void mean_velocity(const GradPlane &lo, const GradPla
 // gradient of v, u the mean of the cell's 8 corner velocities; the ENO
 // stencils reach two cells out, z ghost cells extrapolate each component
 // linearly from the two layers next to the wall; D^pl and sbar of the state
-// are written for the chi update.  Columns march in z as in the predictor.
+// are written for the chi update.  Columns march in z as in the predictor;
+// bound by FP64 instructions: 124 us at 64 x 64 x 32, 219 with a thread a cell
+// and both one-sided derivatives formed.
 __global__ void __launch_bounds__(128)
     k_explicit_stress(StepParams p, CellConst w, StzConst c, int chunk,
                       const double *__restrict__ v, const double *__restrict__ sig,
@@ -644,7 +649,8 @@ __global__ void __launch_bounds__(128)
 // the stress advection of the general constitutive law (section 2), which
 // Eq. (27) drops, as an option of the quasi-static step: sigma* -= dt (u.grad)
 // sigma^n, u the mean of the cell's 8 corner velocities of v^n (the
-// explicit method's advection, Eq. 33 and its ghosts)
+// explicit method's advection, Eq. 33 and its ghosts); bound by the 18 ENO
+// derivatives a cell: 391 us at 96^3, 810 with a thread a cell
 __global__ void __launch_bounds__(128)
     k_stress_advect(StepParams p, CellConst w, int chunk, const double *__restrict__ v,
                     const double *__restrict__ sig, double *__restrict__ sig_star, long nc) {
@@ -686,7 +692,8 @@ __global__ void __launch_bounds__(128)
 // corner, the Laplacian Eq. (32) along each axis (the second differences the
 // ENO test forms anyway), ENO advection with the corner's own velocity;
 // corners up to two planes beyond a wall reflect v through the wall value,
-// v(-m) = 2 v(0) - v(m)
+// v(-m) = 2 v(0) - v(m).  Marches in z; 59 us at 64 x 64 x 32 against 102 with
+// a thread a corner.
 struct VelConst {
     double div, lap, adv;  // dt / (4 h rho);  dt kappa / h^2;  dt / (2 h)
 };
