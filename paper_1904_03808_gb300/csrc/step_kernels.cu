@@ -257,7 +257,7 @@ __device__ __forceinline__ void correct_cell(const CellConst &w, const double (&
 }
 
 // Eq. (27) over a column chunk of cells.  FP64 instructions bound it (its 144
-// bytes a cell take 0.36 ms at 256^3): 4.16 ms there, 5.94 with the gradient
+// bytes a cell take 0.36 ms at 256^3): 4.36 ms there, 5.94 with the gradient
 // unshifted, both exponentials in FP64 and 32 x 8 thread blocks.
 __global__ void __launch_bounds__(128)
     k_stress_predict(StepParams p, CellConst w, StzConst c, int chunk, const double *__restrict__ v,
@@ -286,7 +286,7 @@ __global__ void __launch_bounds__(128)
 // the STZ rate of those extrapolated values
 // A thread marches a column in z: a z face's flux serves the cells below and
 // above it.  The products of constants are formed on the host -- three FP64
-// divisions a cell were half of this kernel: 0.68 ms at 256^3, 1.73 before.
+// divisions a cell were half of this kernel: 0.72 ms at 256^3, 1.73 before.
 struct ChiConst {
     double grow, diff;  // 2 dt / (c0 s_Y);  dt l^2 / (2 c0 h^2)
     double chi_inf;
