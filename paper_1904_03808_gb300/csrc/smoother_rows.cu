@@ -155,6 +155,10 @@ struct RowCols {
 
 // Finest level: the structured 19-point operator (scaled Eq. 30).
 struct FineRowsOp {
+    // the residual adds its right-hand side last: added to the neighbour sums,
+    // which are of the size of d0 x, it loses digits that their cancellation
+    // would leave it
+    static constexpr bool kLateRhs = true;
     Fine<float> f;
     // right-hand side of window rows 1 .. R-2 with the z-neighbour terms
     // folded in (L, H: the lower and upper neighbour planes, B: b rows 1..R-2)
@@ -223,6 +227,7 @@ struct FineRowsOp {
 // and the pairs to the left (whose O is x - 1 of E) and right (whose E is
 // x + 1 of O).
 struct CoarseRowsOp {
+    static constexpr bool kLateRhs = false;
     Coarse<float> c;
     __device__ __forceinline__ static float2 pair(const float *A, const RowCols &q, int row,
                                                   int comp, int x2) {
@@ -467,7 +472,11 @@ __global__ void __launch_bounds__(MODE == kRows    ? kPersMaxNx / 2
         const bool mine = !WIN || (t >= kPersHalo / 2 && t < hn - kPersHalo / 2 && gx < gnx);
         // right-hand side with the z-neighbour terms folded in
         float r[3][2][R];
-        op.template fold<R>(r, Zs0 + sL * plane_f, Zs0 + sH * plane_f, Bs, q);
+        if constexpr (RES && OP::kLateRhs)
+            op.template fold_with<R>(
+                r, Zs0 + sL * plane_f, Zs0 + sH * plane_f, [](int, int, int) { return 0.f; }, q);
+        else
+            op.template fold<R>(r, Zs0 + sL * plane_f, Zs0 + sH * plane_f, Bs, q);
         float P[3][2][R];
 #pragma unroll
         for (int c = 0; c < 3; c++)
@@ -496,13 +505,19 @@ __global__ void __launch_bounds__(MODE == kRows    ? kPersMaxNx / 2
                 for (int c = 0; c < 3; c++) x[c] = P[c][0][jj];
                 op.centre(x, cx);
 #pragma unroll
-                for (int c = 0; c < 3; c++) res[c][0][jj] = num[c] - cx[c];
+                for (int c = 0; c < 3; c++) {
+                    res[c][0][jj] = num[c] - cx[c];
+                    if constexpr (OP::kLateRhs) res[c][0][jj] += Bs[q.at(jj - 1, c, q.xe)];
+                }
                 op.template numer<1, R>(P, r, Ps, q, jj, num);
 #pragma unroll
                 for (int c = 0; c < 3; c++) x[c] = P[c][1][jj];
                 op.centre(x, cx);
 #pragma unroll
-                for (int c = 0; c < 3; c++) res[c][1][jj] = num[c] - cx[c];
+                for (int c = 0; c < 3; c++) {
+                    res[c][1][jj] = num[c] - cx[c];
+                    if constexpr (OP::kLateRhs) res[c][1][jj] += Bs[q.at(jj - 1, c, q.xo)];
+                }
             }
             if (RR) {
                 // full weighting R = T^T (weight 1 at offset 0, 1/2 at +-1 per
