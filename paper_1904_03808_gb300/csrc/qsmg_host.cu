@@ -457,12 +457,20 @@ mg_status sweeps_colour(mg_ctx *ctx, int l, const T *b, T *x, int sweeps, bool d
     return MG_OK;
 }
 
+// Sizes a two-phase sweep takes: it deals rows and columns in pairs and planes
+// of alternating parity to its phases, and stores whole planes out of place.
+// The coarsest level, which the cycles solve but mg_smooth takes, may have odd
+// sizes: there the colour launches update x in place and leave the last plane,
+// row or column of an odd size as it was.
+bool even_sizes(const Dims &d) { return ((d.nx | d.ny | d.nz) & 1) == 0; }
+
 // FP64: row strips in two launches a sweep where the rows fit, ping-ponging
 // with the level's residual buffer, else colour launches
 template <typename T>
 mg_status sweeps(mg_ctx *ctx, int l, const T *b, T *x, int n, bool descending) {
     const Dims &d = ctx->L[l];
-    if (!strip_fits<T>(d, l == 0)) return sweeps_colour<T>(ctx, l, b, x, n, descending);
+    if (!even_sizes(d) || !strip_fits<T>(d, l == 0))
+        return sweeps_colour<T>(ctx, l, b, x, n, descending);
     T *a = x, *o = ctx->r64[l];
     for (int s = 0; s < n; s++) {
         if (l == 0)
@@ -488,12 +496,13 @@ mg_status sweeps(mg_ctx *ctx, int l, const T *b, T *x, int n, bool descending) {
 //    launch against 4 x 13 us at 128^2 planes);
 //  - on arrays that are not 16-byte aligned (a caller's, through mg_smooth),
 //    unless the strips take the level: they and the colour launches read
-//    single words, the row strips copy 16 bytes and the tiles pairs.
+//    single words, the row strips copy 16 bytes and the tiles pairs;
+//  - on odd sizes, whose rows the tiles would load at misaligned pairs.
 template <>
 mg_status sweeps<float>(mg_ctx *ctx, int l, const float *b, float *x, int n, bool descending) {
     const Dims &d = ctx->L[l];
     const bool odd = (((uintptr_t)b | (uintptr_t)x) & 15) != 0;
-    const bool colour = (ctx->opts.flags & MG_FLAG_COLOUR_PASSES) ||
+    const bool colour = (ctx->opts.flags & MG_FLAG_COLOUR_PASSES) || !even_sizes(d) ||
                         (l > 0 && (long)d.nx * d.ny >= 128L * 128L && !coarse_rows_fit(d)) ||
                         (odd && !(strip_fits<float>(d, l == 0) && !(l == 0 && ctx->has_sync)));
     if (!colour) return sweeps_tiled(ctx, l, b, x, n, descending);
