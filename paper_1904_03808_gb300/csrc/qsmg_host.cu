@@ -1248,19 +1248,27 @@ mg_status qs_explicit_step(mg_ctx *ctx, qs_state *state, double dt, double rho, 
     const size_t nc = (size_t)d.nx * d.ny * d.nz, nv = corner_count(d);
     const StepParams p = step_params(ctx, dt);
     // steps alternate between the state's arrays and the context's step
-    // scratch (sig_star, chi_tmp, rhs); an odd count is copied back at the end
+    // scratch (sig_star, chi_tmp, rhs).  After an odd number of them, all that
+    // were asked for or those before a failed launch, the last complete state is
+    // in the scratch and is copied back.
     double *sig[2] = {state->sigma, ctx->sig_star}, *chi[2] = {state->chi, ctx->chi_tmp},
            *v[2] = {state->v, ctx->rhs};
-    for (int n = 0; n < nsteps; n++) {
-        const int i = n & 1, o = 1 - i;
+    const auto step = [&](int i, int o) -> mg_status {
         CK(explicit_stress(p, v[i], sig[i], chi[i], sig[o], ctx->dpl, ctx->sbar, ctx->st));
         CK(chi_update(p, sig[i], chi[i], ctx->dpl, ctx->sbar, chi[o], ctx->st));
         CK(explicit_velocity(p, rho, kappa, v[i], sig[i], v[o], ctx->st));
         CK(wall_fill(wall_params(ctx, state->t + dt), v[o], ctx->st));
+        return MG_OK;
+    };
+    mg_status s = MG_OK;
+    int n = 0;
+    for (; n < nsteps; n++) {
+        s = step(n & 1, 1 - (n & 1));
+        if (s != MG_OK) break;
         state->t += dt;
         state->step += 1;
     }
-    if (nsteps & 1) {
+    if (n & 1) {
         CK(cudaMemcpyAsync(state->sigma, ctx->sig_star, 6 * nc * sizeof(double),
                            cudaMemcpyDeviceToDevice, ctx->st));
         CK(cudaMemcpyAsync(state->chi, ctx->chi_tmp, nc * sizeof(double),
@@ -1269,7 +1277,7 @@ mg_status qs_explicit_step(mg_ctx *ctx, qs_state *state, double dt, double rho, 
                            ctx->st));
     }
     CK(cudaStreamSynchronize(ctx->st));
-    return MG_OK;
+    return s;
 }
 
 // ------------------------------------------------------------ components
