@@ -243,16 +243,22 @@ struct NormBuf {
     unsigned *count;
 };
 // exponent e of the power of two 2^e <= sqrt(s2) < 2^(e+1) up to rounding, by
-// which a residual of squared norm s2 is scaled for FP32; 0 if s2 is zero,
-// subnormal or not finite
+// which a residual of squared norm s2 is scaled for FP32; 0 if s2 is zero or
+// not finite.  A subnormal s2 (a norm below 1.5e-154) keeps its exponent: with
+// 0 the FP32 copy would vanish and the refinement stall.
 __host__ __device__ inline int norm_exponent(double s2) {
     union {
         double d;
         long long i;
     } u;
     u.d = s2;
-    const int ex = (int)((u.i >> 52) & 0x7ff);
-    return ex == 0 || ex == 0x7ff ? 0 : (ex - 1023) >> 1;
+    int ex = (int)((u.i >> 52) & 0x7ff);
+    if (ex == 0x7ff || s2 == 0.0) return 0;
+    if (ex == 0) {
+        u.d = s2 * 18014398509481984.0;  // 2^54
+        ex = (int)((u.i >> 52) & 0x7ff) - 54;
+    }
+    return (ex - 1023) >> 1;
 }
 long norm_blocks(const Dims &d);
 // r = b - A x (interior), r walls zero

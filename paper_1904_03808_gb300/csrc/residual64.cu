@@ -63,12 +63,14 @@ __device__ void finish_sum(double acc, int block, int blocks, const NormBuf &nb,
 }
 
 // float(r 2^-e) by exponent arithmetic (no FP64 multiplication); values whose
-// exponent leaves the normal range vanish in FP32 anyway
+// exponent falls below the normal range vanish in FP32 anyway, those above it
+// are infinite
 __device__ __forceinline__ float scaled32(double r, int e) {
     const int hi = __double2hiint(r), ex = (hi >> 20) & 0x7ff;
     if (ex == 0x7ff) return (float)r;
     if (ex - e <= 0 || ex == 0) return 0.0f;
-    return (float)__hiloint2double(hi - (e << 20), __double2loint(r));
+    if (ex - e >= 0x7ff) return __int_as_float(hi < 0 ? 0xff800000 : 0x7f800000);
+    return (float)__hiloint2double(hi - e * (1 << 20), __double2loint(r));
 }
 
 enum { kStore = 0, kNorm = 1 };
