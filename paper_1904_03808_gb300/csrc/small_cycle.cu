@@ -265,14 +265,16 @@ struct Walker {
         }
     }
 
-    // r = right-hand side of plane k minus the dz = +-1 terms, at own nodes
+    // r = right-hand side of plane k (RES: zero) minus the dz = +-1 terms, at
+    // own nodes
+    template <bool RES = false>
     __device__ __forceinline__ void fold(const Coarse<T> &c, const T *b, const T *lo, const T *hi,
                                          T (&r)[NODES][NC]) const {
         T *U = sm + g.scratch, *V = U + g.plmax;
 #pragma unroll
         for (int u = 0; u < NODES; u++) {
             if (node[u].colour < 0) continue;
-            T up[NC], vp[NC], bp[NC];
+            T up[NC], vp[NC], bp[NC] = {};
             const int o = node[u].r[1] + node[u].c[1] + comp[u];
             if constexpr (COMP)
                 z_row_c(c, lo, hi, node[u], comp[u], r[u][0], up[0], vp[0]);
@@ -280,7 +282,7 @@ struct Walker {
                 z_row(c, lo, hi, node[u], r[u], up, vp);
             put(U + o, up);
             put(V + o, vp);
-            get(b + o, bp);
+            if (!RES) get(b + o, bp);
 #pragma unroll
             for (int a = 0; a < NC; a++) r[u][a] = bp[a] - r[u][a];
         }
@@ -393,8 +395,10 @@ struct Walker {
 #pragma unroll 1
             for (int k = k0; k < k1; k++) {
                 T r[NODES][NC];
-                const T *P = own(l, L.x, k);
-                fold(c, own(l, L.b, k), P - L.pl, P + L.pl, r);
+                const T *P = own(l, L.x, k), *B = own(l, L.b, k);
+                // the right-hand side last: it would lose digits to the
+                // neighbour sums, which cancel with the centre term first
+                fold<true>(c, B, P - L.pl, P + L.pl, r);
                 sync_act();
 #pragma unroll
                 for (int u = 0; u < NODES; u++) {
@@ -402,11 +406,12 @@ struct Walker {
                     T o[NC];
                     in_plane(c, P, u, o);
                     const int q = node[u].r[1] + node[u].c[1] + comp[u];
-                    T x[NC];
+                    T x[NC], b[NC];
                     get(P + q, x);
+                    get(B + q, b);
 #pragma unroll
                     for (int a = 0; a < NC; a++)
-                        o[a] = r[u][a] - (o[a] + c.cd[comp[u] + a][0] * x[a]);
+                        o[a] = (r[u][a] - (o[a] + c.cd[comp[u] + a][0] * x[a])) + b[a];
                     put(R + q, o);
                 }
                 sync_act();

@@ -155,10 +155,6 @@ struct RowCols {
 
 // Finest level: the structured 19-point operator (scaled Eq. 30).
 struct FineRowsOp {
-    // the residual adds its right-hand side last: added to the neighbour sums,
-    // which are of the size of d0 x, it loses digits that their cancellation
-    // would leave it
-    static constexpr bool kLateRhs = true;
     Fine<float> f;
     // right-hand side of window rows 1 .. R-2 with the z-neighbour terms
     // folded in (L, H: the lower and upper neighbour planes, B: b rows 1..R-2)
@@ -167,6 +163,12 @@ struct FineRowsOp {
                                          const float *Bs, const RowCols &q) const {
         auto bv = [&](int jj, int c, int e) { return Bs[q.at(jj - 1, c, e ? q.xo : q.xe)]; };
         fold_with<R>(r, Ls, Hs, bv, q);
+    }
+    // the z-neighbour terms alone
+    template <int R>
+    __device__ __forceinline__ void fold_z(float (&r)[3][2][R], const float *Ls, const float *Hs,
+                                           const RowCols &q) const {
+        fold_with<R>(r, Ls, Hs, [](int, int, int) { return 0.f; }, q);
     }
     // the same with the right-hand side of window row jj, component c, node
     // e (0: E, 1: O) given by bv(jj, c, e)
@@ -227,20 +229,14 @@ struct FineRowsOp {
 // and the pairs to the left (whose O is x - 1 of E) and right (whose E is
 // x + 1 of O).
 struct CoarseRowsOp {
-    static constexpr bool kLateRhs = false;
     Coarse<float> c;
     __device__ __forceinline__ static float2 pair(const float *A, const RowCols &q, int row,
                                                   int comp, int x2) {
         return *reinterpret_cast<const float2 *>(&A[q.at(row, comp, x2)]);
     }
-    // row by row: row y contributes A to its own right-hand side, U to the row
-    // above it and V to the row below, each formed from four columns of that
-    // row only (z_row in small_cycle.cu has the algebra), so a row's z sums and
-    // differences are loaded and formed once instead of for three rows
     template <int R>
     __device__ __forceinline__ void fold(float (&r)[3][2][R], const float *Ls, const float *Hs,
                                          const float *Bs, const RowCols &q) const {
-        const int xl = q.xom - 1, xr = q.xep;  // first columns of the left / right pairs
 #pragma unroll
         for (int jj = 1; jj < R - 1; jj++)
 #pragma unroll
@@ -249,6 +245,25 @@ struct CoarseRowsOp {
                 r[a][0][jj] = b2.x;
                 r[a][1][jj] = b2.y;
             }
+        subtract_z<R>(r, Ls, Hs, q);
+    }
+    template <int R>
+    __device__ __forceinline__ void fold_z(float (&r)[3][2][R], const float *Ls, const float *Hs,
+                                           const RowCols &q) const {
+#pragma unroll
+        for (int jj = 1; jj < R - 1; jj++)
+#pragma unroll
+            for (int a = 0; a < 3; a++) r[a][0][jj] = r[a][1][jj] = 0.f;
+        subtract_z<R>(r, Ls, Hs, q);
+    }
+    // row by row: row y contributes A to its own right-hand side, U to the row
+    // above it and V to the row below, each formed from four columns of that
+    // row only (z_row in small_cycle.cu has the algebra), so a row's z sums and
+    // differences are loaded and formed once instead of for three rows
+    template <int R>
+    __device__ __forceinline__ void subtract_z(float (&r)[3][2][R], const float *Ls,
+                                               const float *Hs, const RowCols &q) const {
+        const int xl = q.xom - 1, xr = q.xep;  // first columns of the left / right pairs
 #pragma unroll
         for (int jj = 0; jj < R; jj++) {
             // z sums and differences at columns x_E - 1, x_E, x_O, x_O + 1
@@ -470,11 +485,13 @@ __global__ void __launch_bounds__(MODE == kRows    ? kPersMaxNx / 2
         // this thread's columns in the grid; its pair is stored if in the tile
         const int gx = col0(s) - (WIN ? kPersHalo : 0) + 2 * t;
         const bool mine = !WIN || (t >= kPersHalo / 2 && t < hn - kPersHalo / 2 && gx < gnx);
-        // right-hand side with the z-neighbour terms folded in
+        // right-hand side with the z-neighbour terms folded in; the residual adds
+        // its right-hand side last: added to the neighbour sums, which are of the
+        // size of the centre term, it loses digits that their cancellation would
+        // leave it
         float r[3][2][R];
-        if constexpr (RES && OP::kLateRhs)
-            op.template fold_with<R>(
-                r, Zs0 + sL * plane_f, Zs0 + sH * plane_f, [](int, int, int) { return 0.f; }, q);
+        if constexpr (RES)
+            op.template fold_z<R>(r, Zs0 + sL * plane_f, Zs0 + sH * plane_f, q);
         else
             op.template fold<R>(r, Zs0 + sL * plane_f, Zs0 + sH * plane_f, Bs, q);
         float P[3][2][R];
@@ -505,19 +522,15 @@ __global__ void __launch_bounds__(MODE == kRows    ? kPersMaxNx / 2
                 for (int c = 0; c < 3; c++) x[c] = P[c][0][jj];
                 op.centre(x, cx);
 #pragma unroll
-                for (int c = 0; c < 3; c++) {
-                    res[c][0][jj] = num[c] - cx[c];
-                    if constexpr (OP::kLateRhs) res[c][0][jj] += Bs[q.at(jj - 1, c, q.xe)];
-                }
+                for (int c = 0; c < 3; c++)
+                    res[c][0][jj] = (num[c] - cx[c]) + Bs[q.at(jj - 1, c, q.xe)];
                 op.template numer<1, R>(P, r, Ps, q, jj, num);
 #pragma unroll
                 for (int c = 0; c < 3; c++) x[c] = P[c][1][jj];
                 op.centre(x, cx);
 #pragma unroll
-                for (int c = 0; c < 3; c++) {
-                    res[c][1][jj] = num[c] - cx[c];
-                    if constexpr (OP::kLateRhs) res[c][1][jj] += Bs[q.at(jj - 1, c, q.xo)];
-                }
+                for (int c = 0; c < 3; c++)
+                    res[c][1][jj] = (num[c] - cx[c]) + Bs[q.at(jj - 1, c, q.xo)];
             }
             if (RR) {
                 // full weighting R = T^T (weight 1 at offset 0, 1/2 at +-1 per

@@ -208,7 +208,7 @@ __global__ void __launch_bounds__(NT, 2)
             l[a] = lo[q + a * g.cs];
             h[a] = hi[q + a * g.cs];
             p[a] = __ldg(own + q + a * g.cs);
-            r[a] = __ldg(bk + q + a * g.cs);
+            r[a] = RES ? T(0) : __ldg(bk + q + a * g.cs);
         }
 #pragma unroll
         for (int a = 0; a < 3; a++) {
@@ -240,7 +240,10 @@ __global__ void __launch_bounds__(NT, 2)
             const long q = (long)y * nx + gcol(i, hx, split);
 #pragma unroll
             for (int a = 0; a < 3; a++) {
-                out[q + a * g.cs] = o[a] - op.c.cd[a][0] * P[jj * w + x0 + a];
+                // the right-hand side last: it would lose digits to the
+                // neighbour sums, which cancel with the centre term first
+                out[q + a * g.cs] = (o[a] - op.c.cd[a][0] * P[jj * w + x0 + a]) +
+                                    __ldg(bk + q + a * g.cs);
                 if (k == 1) vout[q + a * g.cs] = T(0);
                 if (k + 1 == g.nz) vout[q + a * g.cs + (long)g.nz * g.ps] = T(0);
             }

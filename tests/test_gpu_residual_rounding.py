@@ -1,0 +1,73 @@
+"""Residuals add their right-hand side after the neighbour sums have cancelled
+against the centre term, so that a right-hand side much smaller than the terms of
+A x keeps its digits.
+
+With x = 1 everywhere every node forms the same sum s (zero up to rounding), and
+r = fl(b - s): r - b varies by no more than one rounding of |b| + |s|, eps (|b| +
+|s|), with |s| read off as the mean of b - r.  Added to the neighbour sums first, b
+would be rounded at their size, 2^17 times larger here.  The restriction (weights
+of sum 8, six additions) is held to 8 (1 + 3) such roundings against the FP64
+restriction of b."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+import oracle as O  # noqa: E402
+from paper_1904_03808_gb300 import MG_MIXED, Context, inputs as I  # noqa: E402
+
+MU, K = I.TABLE1["mu"], I.TABLE1["K"]
+SMALL = 2.0 ** -17
+# strips (64, 32, 20 columns and fewer), one thread a node (odd sizes below
+# 40), persistent rows with a fused restriction (256 and 128 columns)
+SHAPES = [(64, 64, 64), (40, 40, 40), (256, 64, 64)]
+
+
+@pytest.fixture(params=SHAPES, ids=str)
+def ctx(request):
+    c = Context(*request.param, 2e-2 / request.param[0], K, MU, precision=MG_MIXED)
+    yield c
+    c.close()
+
+
+def _arrays(ctx, l, dtype):
+    nx, ny, nz = ctx.level_dims(l)
+    rng = np.random.default_rng(l)
+    b = (SMALL * rng.uniform(-1, 1, (3, nz + 1, ny, nx))).astype(dtype)
+    bg = torch.from_numpy(b).cuda()
+    return b.astype(np.float64), bg, torch.ones_like(bg)
+
+
+def _coarse_levels(ctx):
+    return range(1, ctx.levels - 1)
+
+
+def _check(r, b, eps):
+    e = r.cpu().numpy().astype(np.float64)[:, 1:-1] - b[:, 1:-1]
+    s = np.abs(e.mean(axis=(1, 2, 3)))
+    assert (np.ptp(e, axis=(1, 2, 3)) <= eps * (SMALL + 2 * s)).all()
+
+
+@pytest.mark.parametrize("dtype", [np.float64, np.float32])
+def test_coarse_residual(ctx, dtype):
+    f = ctx.residual if dtype == np.float64 else ctx.residual32
+    for l in _coarse_levels(ctx):
+        b, bg, x = _arrays(ctx, l, dtype)
+        r = torch.empty_like(bg)
+        f(l, bg, x, r)
+        _check(r, b, np.finfo(dtype).eps)
+
+
+def test_coarse_restricted_residual(ctx):
+    for l in _coarse_levels(ctx):
+        b, bg, x = _arrays(ctx, l, np.float32)
+        nx, ny, nz = ctx.level_dims(l + 1)
+        bc = torch.zeros((3, nz + 1, ny, nx), dtype=torch.float32, device="cuda")
+        ctx.residual_restrict32(l, bg, x, bc)
+        got = bc.cpu().numpy().astype(np.float64)
+        e = (got - O.restrict(b))[:, 2:-2]
+        if e.size:
+            s = np.abs(e.mean(axis=(1, 2, 3))) / 8
+            spread = np.ptp(e, axis=(1, 2, 3))
+            assert (spread <= 32 * 2.0 ** -23 * (SMALL + 2 * s)).all(), l
