@@ -179,17 +179,19 @@ __global__ void __launch_bounds__(NT, 2)
         double Pn, Qn;
         pq(k + 1, Pn, Qn);
         const double Cn = Pn + Qn;
+        // the neighbour sums cancel with the centre term first; the right-hand
+        // side, added to them, would lose digits
         double o[3];
-        o[0] = fma(lp, u[own - 1] + u[own + 1], fma(-d0, uc[0], bn[0])) +
-               ((u[own - PX] + u[own + PX]) + (um[0] + un[0]));
-        o[1] = fma(lp, v[own - PX] + v[own + PX], fma(-d0, uc[1], bn[1])) +
-               ((v[own - 1] + v[own + 1]) + (um[1] + un[1]));
-        o[2] = fma(lp, um[2] + un[2], fma(-d0, uc[2], bn[2])) +
-               ((w[own - 1] + w[own + 1]) + (w[own - PX] + w[own + PX]));
+        o[0] = fma(-d0, uc[0], fma(lp, u[own - 1] + u[own + 1],
+                                   (u[own - PX] + u[own + PX]) + (um[0] + un[0])));
+        o[1] = fma(-d0, uc[1], fma(lp, v[own - PX] + v[own + PX],
+                                   (v[own - 1] + v[own + 1]) + (um[1] + un[1])));
+        o[2] = fma(-d0, uc[2], fma(lp, um[2] + un[2],
+                                   (w[own - 1] + w[own + 1]) + (w[own - PX] + w[own + PX])));
         __syncthreads();
-        o[0] += kq * (A[ty][tx + 2] - A[ty][tx]);
-        o[1] += kq * (B[ty + 2][tx] - B[ty][tx]);
-        o[2] += kq * (Cn - Cm);
+        o[0] = fma(kq, A[ty][tx + 2] - A[ty][tx], o[0]) + bn[0];
+        o[1] = fma(kq, B[ty + 2][tx] - B[ty][tx], o[1]) + bn[1];
+        o[2] = fma(kq, Cn - Cm, o[2]) + bn[2];
         if (act) {
             const long row = (long)k * ps + (long)j * nx;
 #pragma unroll

@@ -71,3 +71,11 @@ def test_coarse_restricted_residual(ctx):
             s = np.abs(e.mean(axis=(1, 2, 3))) / 8
             spread = np.ptp(e, axis=(1, 2, 3))
             assert (spread <= 32 * 2.0 ** -23 * (SMALL + 2 * s)).all(), l
+
+
+@pytest.mark.parametrize("dtype", [np.float64, np.float32])
+def test_finest_residual(ctx, dtype):
+    b, bg, x = _arrays(ctx, 0, dtype)
+    r = torch.empty_like(bg)
+    (ctx.residual if dtype == np.float64 else ctx.residual32)(0, bg, x, r)
+    _check(r, b, np.finfo(dtype).eps)
