@@ -138,7 +138,12 @@ cudaError_t gs_colour_coarse(const Dims &d, const Coarse<float> &c, const float 
 // smoother_rows.cu 6.8, 15.4).
 constexpr int kStripFineNx = 96, kStripCoarseNx = 64;
 // From 128 nodes a row on the persistent strips are faster (160x80x80 step 9.75
-// against 10.03 ms).
+// against 10.03 ms) where they take the level: planes of fewer than 9 rows, and
+// rows that are no multiple of 4 (of 8 beyond 256), stay on the strips of any
+// length that fits shared memory.  Ten V-cycles from 128x8x8 take 4.3 ms so
+// against 5.9 with the tile kernel, from 260x16x16 7.9 against 10.8; us a sweep
+// of these finest levels 12 and 16 against 20 and 25, of a 128x8x8 coarse one
+// 12 against 21.
 constexpr int kStripFineNx32 = 126, kStripCoarseNx32 = 126;
 cudaError_t strip_init();
 template <typename T>

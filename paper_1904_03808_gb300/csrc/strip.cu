@@ -354,10 +354,10 @@ cudaError_t strip_init() {
 
 template <typename T>
 bool strip_fits(const Dims &d, bool finest) {
-    const int most = sizeof(T) == 8 ? (finest ? kStripFineNx : kStripCoarseNx)
-                                    : (finest ? kStripFineNx32 : kStripCoarseNx32);
     const size_t node = 3 * sizeof(T) * (finest ? 3 : 6);
-    return d.nx <= most && d.nx % 2 == 0 && d.ny % 2 == 0 && strip_rows(d, node, d.nz / 2) > 0;
+    if (d.nx % 2 || d.ny % 2 || strip_rows(d, node, d.nz / 2) == 0) return false;
+    if (sizeof(T) == 8) return d.nx <= (finest ? kStripFineNx : kStripCoarseNx);
+    return d.nx <= (finest ? kStripFineNx32 : kStripCoarseNx32) || !coarse_rows_fit(d);
 }
 
 template <typename T>
