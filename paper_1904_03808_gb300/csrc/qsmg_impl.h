@@ -137,14 +137,14 @@ cudaError_t gs_colour_coarse(const Dims &d, const Coarse<float> &c, const float 
 // (tile kernel 13.4-13.8); fine 64^3 6.4, 96^3 10.6 (row kernels of
 // smoother_rows.cu 6.8, 15.4).
 constexpr int kStripFineNx = 96, kStripCoarseNx = 64;
-// From 128 nodes a row on the persistent strips are faster (160x80x80 step 9.75
-// against 10.03 ms) where they take the level: planes of fewer than 9 rows, and
+// The persistent strips are faster on FP32 rows of 128 nodes and more (160x80x80
+// step 9.75 against 10.03 ms) and on large finest levels of shorter ones
+// (fine_rows_fit), where they take the level: planes of fewer than 9 rows, and
 // rows that are no multiple of 4 (of 8 beyond 256), stay on the strips of any
 // length that fits shared memory.  Ten V-cycles from 128x8x8 take 4.3 ms so
 // against 5.9 with the tile kernel, from 260x16x16 7.9 against 10.8; us a sweep
 // of these finest levels 12 and 16 against 20 and 25, of a 128x8x8 coarse one
 // 12 against 21.
-constexpr int kStripFineNx32 = 126, kStripCoarseNx32 = 126;
 cudaError_t strip_init();
 template <typename T>
 bool strip_fits(const Dims &d, bool finest);
@@ -200,6 +200,8 @@ cudaError_t residual_fine_rows(const Dims &d, const Fine<float> &f, const float 
 // block stencil); cudaErrorNotSupported when it does not apply.
 // coarse_rows_fit: whether a level of these dimensions takes it.
 bool coarse_rows_fit(const Dims &d);
+// the same for the finest level
+bool fine_rows_fit(const Dims &d);
 cudaError_t gs_sweep_coarse_rows(const Dims &d, const Coarse<float> &c, const float *b,
                                  const float *vin, float *vout, bool descending, cudaStream_t s);
 // coarse FP32 residual and restriction without storing the residual (part:

@@ -1198,6 +1198,24 @@ bool coarse_rows_fit(const Dims &d) {
     return d.nx >= 128 && rows_p_shape(d, sms);
 }
 
+// On the finest level they also take rows of 64 to 126 nodes, unless a phase's
+// tiles fill less than half of the resident CTAs or leave a second round of them
+// more than half empty: these CTAs are then too few to hide their copies, and
+// strip.cu's larger blocks of smaller strips are faster.  Ten V-cycles, rows
+// against strips in ms, with tiles a phase over resident CTAs:
+//   64^3 0.29: 6.62, 6.24       64x80x80 0.46: 6.75, 6.62   64x128x64 0.58: 7.16, 7.38
+//   96x64x64 0.58: 6.88, 7.12   80^3 0.92: 7.76, 8.11       64x128x112 1.01: 9.63, 10.05
+//   96x128x64 1.16: 10.38, 10.11  96^3 1.26: 10.32, 9.95    112x128x112 2.03: 15.71, 16.82
+//   64x160x160 1.78: 13.61, 15.31 96x160x160 3.6: 19.56, 21.29  64x256x256 4.5: 27.7, 32.4
+bool fine_rows_fit(const Dims &d) {
+    int sms = 0;
+    if (d.nx < 64 || !rows_p_shape(d, sms)) return false;
+    if (d.nx >= 128) return true;
+    const long tiles = (long)((d.ny + kPersTY - 1) / kPersTY) * (d.nz / 2);
+    const long slots = pers_slots(d.nx, sms);
+    return 2 * tiles >= slots && !(10 * tiles > 11 * slots && 2 * tiles < 3 * slots);
+}
+
 // coarse-level FP32 sweep with the persistent row-strip kernel (natural
 // column order), or cudaErrorNotSupported
 cudaError_t gs_sweep_coarse_rows(const Dims &d, const Coarse<float> &c, const float *b,

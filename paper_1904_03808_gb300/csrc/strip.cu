@@ -357,7 +357,7 @@ bool strip_fits(const Dims &d, bool finest) {
     const size_t node = 3 * sizeof(T) * (finest ? 3 : 6);
     if (d.nx % 2 || d.ny % 2 || strip_rows(d, node, d.nz / 2) == 0) return false;
     if (sizeof(T) == 8) return d.nx <= (finest ? kStripFineNx : kStripCoarseNx);
-    return d.nx <= (finest ? kStripFineNx32 : kStripCoarseNx32) || !coarse_rows_fit(d);
+    return finest ? !fine_rows_fit(d) : !coarse_rows_fit(d);
 }
 
 template <typename T>

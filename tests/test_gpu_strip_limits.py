@@ -18,6 +18,9 @@ LAM = I.lame_lambda(K, MU)
 # 256/128, 260/130; few rows (4 to 8) and, for the persistent rows, ten and more
 SHAPES = [(96, 20, 16), (98, 8, 8), (126, 8, 8), (128, 8, 8), (128, 20, 16), (132, 16, 16),
           (252, 16, 16), (256, 16, 16), (256, 32, 32), (260, 16, 16)]
+# finest levels below 128 columns: tiles enough for the persistent rows (80^3,
+# 64x128x64, 112x64x64), too few (64^3) and a second round of few (96^3)
+SHAPES += [(80, 80, 80), (64, 128, 64), (112, 64, 64), (64, 64, 64), (96, 96, 96)]
 
 
 @pytest.mark.parametrize("shape", SHAPES)
