@@ -48,21 +48,19 @@ namespace {
 //   z_1 = (L1+H1) + kq (D2(y+1) - D2(y-1)),
 //   z_2 = lp (L2+H2) + kq ((D0(x+1) - D0(x-1)) + (D1(y+1) - D1(y-1))),
 // with D = H - L, streamed row by row so each plane value is loaded once.
-// numerators of the node of x-parity E at window row jj: the folded
-// right-hand side r plus the in-plane neighbour terms, from the own column
-// values P and the far-side neighbour column X[c * sc + row * sr + xn]
-// (shared memory); the Gauss-Seidel update is numerator / d0, the residual
-// numerator - d0 x
+// m, p: the in-plane neighbours of the node of x-parity E at window row jj in
+// columns x - 1 and x + 1, by component and row (jj-1, jj, jj+1), from the own
+// column values P and the far-side neighbour column X[c * sc + row * sr + xn]
+// (shared memory); component 2 enters only through row jj
 template <int E, int R>
-__device__ __forceinline__ void rows_numer(const float (&P)[3][2][R], float r0, float r1,
-                                           float r2, const float *X, int sc, int sr, int xn,
-                                           int jj, const Fine<float> &f, float num[3]) {
-    float m[3][3], p[3][3];  // [component][row jj-1, jj, jj+1] at x-1 and x+1
+__device__ __forceinline__ void rows_columns(const float (&P)[3][2][R], const float *X, int sc,
+                                             int sr, int xn, int jj, float (&m)[3][3],
+                                             float (&p)[3][3]) {
 #pragma unroll
     for (int q = 0; q < 3; q++)
 #pragma unroll
         for (int c = 0; c < 3; c++) {
-            if (q != 1 && c == 2) continue;  // comp 2 enters only through row jj
+            if (q != 1 && c == 2) continue;
             const float own = P[c][1 - E][jj - 1 + q];
             const float nb = X[c * sc + (jj - 1 + q) * sr + xn];
             if (E == 0) {
@@ -73,12 +71,46 @@ __device__ __forceinline__ void rows_numer(const float (&P)[3][2][R], float r0, 
                 p[c][q] = nb;
             }
         }
+}
+
+// numerators of that node: the folded right-hand side r plus the in-plane
+// neighbour terms; the Gauss-Seidel update is numerator / d0
+template <int E, int R>
+__device__ __forceinline__ void rows_numer(const float (&P)[3][2][R], float r0, float r1,
+                                           float r2, const float *X, int sc, int sr, int xn,
+                                           int jj, const Fine<float> &f, float num[3]) {
+    float m[3][3], p[3][3];
+    rows_columns<E, R>(P, X, sc, sr, xn, jj, m, p);
     const float lp = f.lp, kq = f.kq;
     num[0] = r0 + lp * (m[0][1] + p[0][1]) + (P[0][E][jj - 1] + P[0][E][jj + 1]) +
              kq * (p[1][2] - p[1][0] - m[1][2] + m[1][0]);
     num[1] = r1 + lp * (P[1][E][jj - 1] + P[1][E][jj + 1]) + (m[1][1] + p[1][1]) +
              kq * (p[0][2] - p[0][0] - m[0][2] + m[0][0]);
     num[2] = r2 + (m[2][1] + p[2][1]) + (P[2][E][jj - 1] + P[2][E][jj + 1]);
+}
+
+// -A x at that node, r0 .. r2 its z-neighbour terms.  d0 = 2 lp + 4: each pair of
+// neighbours gives up its share 2 x of the centre term before it is weighted and
+// added, so that no sum of the size of d0 x is rounded.
+template <int E, int R>
+__device__ __forceinline__ void rows_minus_ax(const float (&P)[3][2][R], float r0, float r1,
+                                              float r2, const float *X, int sc, int sr, int xn,
+                                              int jj, const Fine<float> &f, float out[3]) {
+    float m[3][3], p[3][3];
+    rows_columns<E, R>(P, X, sc, sr, xn, jj, m, p);
+    const float lp = f.lp, kq = f.kq;
+    float dx[3], dy[3];
+#pragma unroll
+    for (int c = 0; c < 3; c++) {
+        const float x = P[c][E][jj];
+        dx[c] = fmaf(-2.f, x, m[c][1] + p[c][1]);
+        dy[c] = fmaf(-2.f, x, P[c][E][jj - 1] + P[c][E][jj + 1]);
+    }
+    const float dz0 = fmaf(-2.f, P[0][E][jj], r0), dz1 = fmaf(-2.f, P[1][E][jj], r1),
+                dz2 = fmaf(-2.f * lp, P[2][E][jj], r2);
+    out[0] = fmaf(kq, p[1][2] - p[1][0] - m[1][2] + m[1][0], fmaf(lp, dx[0], dy[0] + dz0));
+    out[1] = fmaf(kq, p[0][2] - p[0][0] - m[0][2] + m[0][0], fmaf(lp, dy[1], dx[1] + dz1));
+    out[2] = (dx[2] + dy[2]) + dz2;
 }
 
 // ------------------------------------------------------------------------
@@ -211,13 +243,17 @@ struct FineRowsOp {
         rows_numer<E, R>(P, r[0][E][jj], r[1][E][jj], r[2][E][jj], X, q.nx, 3 * q.nx,
                          E == 0 ? q.xom : q.xep, jj, f, num);
     }
+    // -A x, r the z-neighbour terms alone
+    template <int E, int R>
+    __device__ __forceinline__ void minus_ax(const float (&P)[3][2][R], const float (&r)[3][2][R],
+                                             const float *X, const RowCols &q, int jj,
+                                             float out[3]) const {
+        rows_minus_ax<E, R>(P, r[0][E][jj], r[1][E][jj], r[2][E][jj], X, q.nx, 3 * q.nx,
+                            E == 0 ? q.xom : q.xep, jj, f, out);
+    }
     __device__ __forceinline__ void solve(const float num[3], float out[3]) const {
 #pragma unroll
         for (int a = 0; a < 3; a++) out[a] = num[a] * f.dinv;
-    }
-    __device__ __forceinline__ void centre(const float x[3], float out[3]) const {
-#pragma unroll
-        for (int a = 0; a < 3; a++) out[a] = f.d0 * x[a];
     }
 };
 
@@ -340,9 +376,13 @@ struct CoarseRowsOp {
 #pragma unroll
         for (int a = 0; a < 3; a++) out[a] = c.dinv[a] * num[a];
     }
-    __device__ __forceinline__ void centre(const float x[3], float out[3]) const {
+    template <int E, int R>
+    __device__ __forceinline__ void minus_ax(const float (&P)[3][2][R], const float (&r)[3][2][R],
+                                             const float *X, const RowCols &q, int jj,
+                                             float out[3]) const {
+        numer<E, R>(P, r, X, q, jj, out);
 #pragma unroll
-        for (int a = 0; a < 3; a++) out[a] = c.cd[a][0] * x[a];
+        for (int a = 0; a < 3; a++) out[a] -= c.cd[a][0] * P[a][E][jj];
     }
 };
 
@@ -509,28 +549,20 @@ __global__ void __launch_bounds__(MODE == kRows    ? kPersMaxNx / 2
                 }
             }
         if (RES) {
-            // residual of the tile rows 1 .. TY: numerator - centre block x
+            // residual of the tile rows 1 .. TY
             // (with RR rows 1 .. TY + 1, i.e. y0 - 1 .. y0 + TY - 1: the fine
             // rows of the strip's coarse rows)
             constexpr int NR = RR ? TY + 2 : TY + 1;
             float res[3][2][NR];
 #pragma unroll
             for (int jj = 1; jj < NR; jj++) {
-                float num[3], x[3], cx[3];
-                op.template numer<0, R>(P, r, Ps, q, jj, num);
+                float ax[3];
+                op.template minus_ax<0, R>(P, r, Ps, q, jj, ax);
 #pragma unroll
-                for (int c = 0; c < 3; c++) x[c] = P[c][0][jj];
-                op.centre(x, cx);
+                for (int c = 0; c < 3; c++) res[c][0][jj] = ax[c] + Bs[q.at(jj - 1, c, q.xe)];
+                op.template minus_ax<1, R>(P, r, Ps, q, jj, ax);
 #pragma unroll
-                for (int c = 0; c < 3; c++)
-                    res[c][0][jj] = (num[c] - cx[c]) + Bs[q.at(jj - 1, c, q.xe)];
-                op.template numer<1, R>(P, r, Ps, q, jj, num);
-#pragma unroll
-                for (int c = 0; c < 3; c++) x[c] = P[c][1][jj];
-                op.centre(x, cx);
-#pragma unroll
-                for (int c = 0; c < 3; c++)
-                    res[c][1][jj] = (num[c] - cx[c]) + Bs[q.at(jj - 1, c, q.xo)];
+                for (int c = 0; c < 3; c++) res[c][1][jj] = ax[c] + Bs[q.at(jj - 1, c, q.xo)];
             }
             if (RR) {
                 // full weighting R = T^T (weight 1 at offset 0, 1/2 at +-1 per

@@ -79,3 +79,17 @@ def test_finest_residual(ctx, dtype):
     r = torch.empty_like(bg)
     (ctx.residual if dtype == np.float64 else ctx.residual32)(0, bg, x, r)
     _check(r, b, np.finfo(dtype).eps)
+
+
+@pytest.mark.parametrize("value", [1.1, 0.7, 1.3, 0.9])
+def test_finest_residual_of_a_constant_field(ctx, value):
+    """FP32 persistent rows: every pair of neighbours gives up its share of the
+    centre term before it is weighted, so a constant field has no residual in u and
+    v, and in w at most the rounding of the weighted z pair, 2 lp x."""
+    nx, ny, nz = ctx.level_dims(0)
+    x = torch.full((3, nz + 1, ny, nx), value, dtype=torch.float32, device="cuda")
+    r = torch.empty_like(x)
+    ctx.residual32(0, torch.zeros_like(x), x, r)
+    lp = np.float32((I.lame_lambda(K, MU) + 2 * MU) / MU)
+    assert not r[:2].any()
+    assert float(r[2].abs().max()) <= 0.5 * np.spacing(np.float32(2 * lp * value))
