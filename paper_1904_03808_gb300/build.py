@@ -15,9 +15,8 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 OUT_DIR = os.path.join(HERE, "_build")
 LIB = os.path.join(OUT_DIR, "libqsmg.so")
-SOURCES = ["mg_kernels.cu", "smoother_fast.cu", "smoother_rows.cu", "small_cycle.cu",
-           "strip.cu", "residual64.cu", "step_kernels.cu", "qsmg_host.cu",
-           "static_scratch.cu"]
+SOURCES = ["mg_kernels.cu", "smoother_rows.cu", "small_cycle.cu", "strip.cu", "residual64.cu",
+           "step_kernels.cu", "qsmg_host.cu", "static_scratch.cu"]
 PROBE = "peak_probe.cu"
 PROBE_LIB = os.path.join(OUT_DIR, "libqsmg_peak.so")
 HEADERS = ["qsmg_impl.h", os.path.join("..", "..", "include", "qsmg.h")]

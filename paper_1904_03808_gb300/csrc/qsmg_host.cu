@@ -410,10 +410,11 @@ mg_status gs_pass(mg_ctx *ctx, int l, const T *b, T *x, int colour) {
     return MG_OK;
 }
 
-// FP32 sweeps on level l with the tiled two-phase kernels, ping-ponging
+// FP32 sweeps on level l with the two-phase kernels, ping-ponging
 // between x and the level's partner buffer (whose wall planes are made equal
 // to x's; the solver's own level arrays and partners all keep zero walls)
-mg_status sweeps_tiled(mg_ctx *ctx, int l, const float *b, float *x, int sweeps, bool descending) {
+mg_status sweeps_two_phase(mg_ctx *ctx, int l, const float *b, float *x, int sweeps,
+                           bool descending) {
     const Dims &d = ctx->L[l];
     float *a = x, *o = ctx->xs32[l];
     if (x != ctx->x32[l]) {
@@ -427,10 +428,10 @@ mg_status sweeps_tiled(mg_ctx *ctx, int l, const float *b, float *x, int sweeps,
     }
     for (int s = 0; s < sweeps; s++) {
         if (l == 0)
-            CK(gs_sweep_fine_tiled(d, ctx->f32, b, a, o, descending, ctx->st, ctx->split0,
-                                   ctx->has_sync ? &ctx->sync : nullptr));
+            CK(gs_sweep_fine32(d, ctx->f32, b, a, o, descending, ctx->st, ctx->split0,
+                               ctx->has_sync ? &ctx->sync : nullptr));
         else
-            CK(gs_sweep_coarse_tiled(d, ctx->c32[l], b, a, o, descending, ctx->st));
+            CK(gs_sweep_coarse32(d, ctx->c32[l], b, a, o, descending, ctx->st));
         float *t = a;
         a = o;
         o = t;
@@ -490,23 +491,19 @@ mg_status sweeps(mg_ctx *ctx, int l, const T *b, T *x, int n, bool descending) {
     return MG_OK;
 }
 
-// FP32: the two-phase kernels (strips, persistent row strips, tiles), except
-//  - on large coarse levels without row strips, where the 27-point tile kernel
-//    (128 registers, 2 CTAs per SM) loses to colour launches (71 us per phase
-//    launch against 4 x 13 us at 128^2 planes);
-//  - on arrays that are not 16-byte aligned (a caller's, through mg_smooth),
-//    unless the strips take the level: they and the colour launches read
-//    single words, the row strips copy 16 bytes and the tiles pairs;
-//  - on odd sizes, whose rows the tiles would load at misaligned pairs.
+// FP32: the two-phase kernels (strips, persistent row strips), except on
+//  - odd sizes;
+//  - arrays that are not 16-byte aligned (a caller's, through mg_smooth), unless
+//    the strips take the level: they and the colour launches read single words,
+//    the row strips copy 16 bytes.
 template <>
 mg_status sweeps<float>(mg_ctx *ctx, int l, const float *b, float *x, int n, bool descending) {
     const Dims &d = ctx->L[l];
-    const bool odd = (((uintptr_t)b | (uintptr_t)x) & 15) != 0;
-    const bool colour = (ctx->opts.flags & MG_FLAG_COLOUR_PASSES) || !even_sizes(d) ||
-                        (l > 0 && (long)d.nx * d.ny >= 128L * 128L && !coarse_rows_fit(d)) ||
-                        (odd && !(strip_fits<float>(d, l == 0) && !(l == 0 && ctx->has_sync)));
-    if (!colour) return sweeps_tiled(ctx, l, b, x, n, descending);
-    return sweeps_colour<float>(ctx, l, b, x, n, descending);
+    const bool aligned = (((uintptr_t)b | (uintptr_t)x) & 15) == 0;
+    const bool two_phase = !(ctx->opts.flags & MG_FLAG_COLOUR_PASSES) && even_sizes(d) &&
+                           (aligned || strip_fits<float>(d, l == 0));
+    return two_phase ? sweeps_two_phase(ctx, l, b, x, n, descending)
+                     : sweeps_colour<float>(ctx, l, b, x, n, descending);
 }
 
 // queue one timed event pair for the next drain

@@ -133,18 +133,16 @@ cudaError_t gs_colour_coarse(const Dims &d, const Coarse<float> &c, const float 
 // repeated work of a strip outweighs its fewer, longer launches (226 us a sweep
 // at 128^3 against 218 us for eight colour launches; at 64^3 38 against 60 us);
 // 64-wide coarse rows fill half an SM's shared memory (75 against 115 us a 64^3
-// sweep).  FP32, us a phase launch: coarse 64^3 7.8, 80x40x40 7.4, 48^3 6.0
-// (tile kernel 13.4-13.8); fine 64^3 6.4, 96^3 10.6 (row kernels of
-// smoother_rows.cu 6.8, 15.4).
+// sweep).
 constexpr int kStripFineNx = 96, kStripCoarseNx = 64;
-// The persistent strips are faster on FP32 rows of 128 nodes and more (160x80x80
-// step 9.75 against 10.03 ms) and on large finest levels of shorter ones
-// (fine_rows_fit), where they take the level: planes of fewer than 9 rows, and
-// rows that are no multiple of 4 (of 8 beyond 256), stay on the strips of any
-// length that fits shared memory.  Ten V-cycles from 128x8x8 take 4.3 ms so
-// against 5.9 with the tile kernel, from 260x16x16 7.9 against 10.8; us a sweep
-// of these finest levels 12 and 16 against 20 and 25, of a 128x8x8 coarse one
-// 12 against 21.
+// FP32: every level that the persistent row strips do not take or are slower on
+// (coarse_rows_fit, fine_rows_fit): coarse rows below 128 nodes, small finest
+// levels, planes of fewer than 9 rows, and rows that are no multiple of 4 (of 8
+// beyond 256).  us a phase launch, with the 27-point tile kernel that took these
+// coarse levels before: 64^3 7.8, 80x40x40 7.4, 48^3 6.0 (13.4-13.8); us a sweep
+// of a 96x208x208 level 107 and of a 112x160x128 one 78, 140 and 87 as eight
+// colour launches.  Ten V-cycles from 128x8x8 take 4.3 ms, 5.9 with a tile kernel
+// of the finest operator, from 260x16x16 7.9 and 10.8.
 cudaError_t strip_init();
 template <typename T>
 bool strip_fits(const Dims &d, bool finest);
@@ -220,19 +218,18 @@ struct SweepSync {
 bool fused_sweep_sizes(const Dims &d, long &naflag);
 // FP32 finest-level sweep vin -> vout with the row-strip kernels: the fused
 // one-launch sweep when sync is given and the grid suits it, else the two
-// phase launches; cudaErrorNotSupported when the rows are too long for them
+// phase launches; cudaErrorNotSupported when they do not take the rows or arrays
 cudaError_t gs_sweep_fine_rows(const Dims &d, const Fine<float> &f, const float *b,
                                const float *vin, float *vout, bool descending, cudaStream_t s,
                                int split, const SweepSync *sync = nullptr);
-// tiled FP32 finest-level sweep vin -> vout (two phase launches); split:
-// the arrays are in parity-split column order
-cudaError_t gs_sweep_fine_tiled(const Dims &d, const Fine<float> &f, const float *b,
-                                const float *vin, float *vout, bool descending, cudaStream_t s,
-                                int split = 0, const SweepSync *sync = nullptr);
-
-// tiled FP32 coarse-level sweep vin -> vout (27-point block stencil)
-cudaError_t gs_sweep_coarse_tiled(const Dims &d, const Coarse<float> &c, const float *b,
-                                  const float *vin, float *vout, bool descending, cudaStream_t s);
+// FP32 sweeps vin -> vout of any level of even sizes (strips or persistent rows;
+// vout's wall planes must hold the walls); split: the arrays are in parity-split
+// column order
+cudaError_t gs_sweep_fine32(const Dims &d, const Fine<float> &f, const float *b, const float *vin,
+                            float *vout, bool descending, cudaStream_t s, int split = 0,
+                            const SweepSync *sync = nullptr);
+cudaError_t gs_sweep_coarse32(const Dims &d, const Coarse<float> &c, const float *b,
+                              const float *vin, float *vout, bool descending, cudaStream_t s);
 
 // r = b - A x (interior), r walls zero
 cudaError_t residual_fine(const Dims &d, const Fine<float> &f, const float *b, const float *x,

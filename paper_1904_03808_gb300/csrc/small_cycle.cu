@@ -12,7 +12,7 @@
 //   - an update is stored (FP64: an updated plane is copied) through distributed
 //     shared memory to the halos that mirror it too, and a cluster barrier (0.2 us measured, against
 //     1.2 us for a grid-wide one) takes the place of a launch boundary;
-//   - a sweep is the two phases of smoother_fast.cu, planes of one k-parity
+//   - a sweep is the two phases of strip.cu, planes of one k-parity
 //     and then of the other: the dz = +-1 part of the 27-point operator is
 //     folded into the right-hand side, then the 4 in-plane colours run on the
 //     plane, so every node sees the neighbour values of the sequential order.

@@ -3,8 +3,7 @@
 // coarse levels of rows >= 128 nodes (27-point block stencil, Eq. 36), and
 // the residuals of those levels.
 //
-// One 8-colour sweep runs as two phase launches, as in smoother_fast.cu:
-// the planes of one k-parity (4 in-plane colours each, reading the old
+// One 8-colour sweep runs as two phase launches, as in strip.cu: the planes of one k-parity (4 in-plane colours each, reading the old
 // z-neighbour planes), then the planes of the other parity (reading the
 // first phase's output).  A CTA owns whole rows of a plane where they have at
 // most 512 nodes, so the periodic x direction needs no halo, and tiles of

@@ -6,17 +6,21 @@
 // bound by the number of full-lane FP64 instructions and by how evenly they
 // are dealt to the 608 schedulers.  Eight colour launches of one thread a node
 // leave most schedulers idle on levels of 64^3 and below and evaluate every
-// sum of a node from scratch.  Here a sweep is two launches (planes of one
-// k-parity, then of the other, as in smoother_fast.cu); a CTA owns TY rows of
-// a plane:
+// sum of a node from scratch.  Here, as in smoother_rows.cu, a sweep is two
+// launches: colours 0-3 (colour (i&1) + 2 (j&1) + 4 (k&1)) live on the even
+// planes, 4-7 on the odd ones, and the stencil couples a plane only to its two
+// neighbours, so the planes of one k-parity are updated in the order of their 4
+// colours from the old neighbour planes, then the others from the new ones:
+// every node sees the values of eight colour passes, and v is read and written
+// about twice a sweep.  A CTA owns TY rows of a plane:
 //   - the sums S = up + down and differences D = up - down of the two
 //     neighbour planes are formed once per node and shared;
 //   - coarse levels: the dz = +-1 part is applied row by row (small_cycle.cu
 //     has the same form), 96 FP64 instructions a node instead of 154;
 //   - the 4 in-plane colours run on shared rows, lanes packed by colour.
 // FP32 takes the same kernel, a node a thread, on levels too small for the
-// persistent row strips (smoother_rows.cu): what it saves there is the repeated
-// evaluation of the z sums, which the tile kernel did in every pass.
+// persistent row strips (smoother_rows.cu) or of rows these do not take: the z
+// sums are evaluated once instead of in every pass.
 // Measured per phase launch in FP64 (before: four colour launches): fine 32^3 6.3 us
 // (29), 64^3 19 us (30), coarse 32^3 9.5 us (57), 64^3 37.6 us (57).  What
 // bounds it now: at 64^3 two waves of 256 strips on 152 SMs, at 32^3 the
@@ -374,6 +378,23 @@ template <typename T>
 cudaError_t residual_strip(const Dims &d, const Coarse<T> &c, const T *b, const T *x, T *r,
                            cudaStream_t s) {
     return launch<0, true>(d, CoarseStrip<T>{c}, b, x, x, x, r, 1, d.nz - 1, s, 0);
+}
+
+// FP32: the persistent rows where they take the level, else the strips (which a
+// caller's arrays at any word suit); every level of even sizes that mg_setup
+// accepts suits one of them
+cudaError_t gs_sweep_fine32(const Dims &d, const Fine<float> &f, const float *b, const float *vin,
+                            float *vout, bool descending, cudaStream_t s, int split,
+                            const SweepSync *sync) {
+    if (!sync && strip_fits<float>(d, true))
+        return gs_sweep_strip(d, f, b, vin, vin, vout, descending, s, split);
+    return gs_sweep_fine_rows(d, f, b, vin, vout, descending, s, split, sync);
+}
+cudaError_t gs_sweep_coarse32(const Dims &d, const Coarse<float> &c, const float *b,
+                              const float *vin, float *vout, bool descending, cudaStream_t s) {
+    if (strip_fits<float>(d, false))
+        return gs_sweep_strip(d, c, b, vin, vin, vout, descending, s);
+    return gs_sweep_coarse_rows(d, c, b, vin, vout, descending, s);
 }
 
 #define INSTANTIATE(T)                                                                           \
