@@ -587,14 +587,15 @@ cudaError_t restrict_z(const Dims &fine, const float *part, float *bc, cudaStrea
 template <typename T>
 static cudaError_t prolong_t(const Dims &f, const T *xc, T *x, cudaStream_t s, int split) {
     const Dims c = make_dims(f.nx / 2, f.ny / 2, f.nz / 2);
-    if (sizeof(T) == 8 || (long)c.nx * c.ny * c.nz <= kProlongSplit) {
-        const int nt = lin_threads((long)c.nx * c.ny, 3L * c.nz);
-        const dim3 grid((c.nx * c.ny + nt - 1) / nt, c.nz, 3);
-        k_prolong_c<T><<<grid, nt, 0, s>>>(f, c, magic(c.nx, (long)c.nx * c.ny), xc, x, split);
-    } else {
-        k_prolong<T><<<node_grid(c.nx, c.ny, c.nz), kBlock, 0, s>>>(f, c, xc, x, split);
-    }
     count_launch();
+    if constexpr (sizeof(T) == 4)
+        if ((long)c.nx * c.ny * c.nz > kProlongSplit) {
+            k_prolong<T><<<node_grid(c.nx, c.ny, c.nz), kBlock, 0, s>>>(f, c, xc, x, split);
+            return cudaGetLastError();
+        }
+    const int nt = lin_threads((long)c.nx * c.ny, 3L * c.nz);
+    const dim3 grid((c.nx * c.ny + nt - 1) / nt, c.nz, 3);
+    k_prolong_c<T><<<grid, nt, 0, s>>>(f, c, magic(c.nx, (long)c.nx * c.ny), xc, x, split);
     return cudaGetLastError();
 }
 cudaError_t prolong_add(const Dims &fine, const double *xc, double *x, cudaStream_t s) {

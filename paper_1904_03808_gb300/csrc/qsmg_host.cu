@@ -2,6 +2,7 @@
 // hierarchy set-up (Galerkin coarse operators, dense coarsest inverse),
 // V-cycle and solve orchestration (FP64, and FP32 cycles inside FP64
 // iterative refinement), the projection step, and the component entry points.
+#include <limits.h>
 #include <math.h>
 #include <stdarg.h>
 #include <stdio.h>
@@ -29,13 +30,12 @@ void set_err(const char *fmt, ...) {
 constexpr int kMaxLev = 16;
 constexpr int kMaxCoarse = 3072;
 constexpr int kProfSlots = 64;
-// Top levels of at most this many nodes run their V-cycles in one cluster of
-// 16 SMs.  FP32: whatever fits its shared memory (up to about 60000 nodes) is
-// faster there than in separate launches.  FP64: with 2 operations a clock and
-// SM, 16 SMs take longer over a 16^3 level than row strips on the whole chip
-// (64^3 gradient 68.1 against 65.1 ms with the limit at 8192 and 1000 nodes),
-// not over an 8^3 one.
-constexpr long kSmallNodes64 = 2048, kSmallNodes32 = 100000;
+// Top levels of at most this many nodes run their FP64 V-cycles in one cluster
+// of 16 SMs: with 2 operations a clock and SM, these take longer over a 16^3
+// level than row strips on the whole chip (64^3 gradient 68.1 against 65.1 ms
+// with the limit at 8192 and 1000 nodes), not over an 8^3 one.  In FP32 whatever
+// a plan takes (small_plan: up to 32x32x48 nodes) is faster there.
+constexpr long kSmallNodes64 = 2048;
 constexpr int kMaxInner = 10;  // cap on FP32 V-cycles per refinement step
 
 // n FP32 V-cycles (from e = 0) captured once and replayed; the event pairs
@@ -1163,7 +1163,7 @@ mg_status mg_setup(const mg_grid *grid, const mg_moduli *moduli, const mg_bc *bc
         if (ctx->top32 < 0 && !(f & MG_FLAG_COLOUR_PASSES) &&
             !(l == 0 && (f & (MG_FLAG_FUSED_SWEEP | MG_FLAG_UNFUSED_TRANSFERS))) &&
             small_plan(ctx->L + l, ctx->c32 + l, ctx->nlev - l, ctx->ncoarse, ctx->Ainv,
-                       opts->nu1, opts->nu2, kSmallNodes32, ctx->s32))
+                       opts->nu1, opts->nu2, LONG_MAX, ctx->s32))
             ctx->top32 = l;
     }
     if (ctx->top32 == 0) ctx->split0 = 0;  // its arrays are in natural order

@@ -611,8 +611,8 @@ void configure(const SmallPlan<T> &g, cudaLaunchConfig_t &cfg, cudaLaunchAttribu
 // plane (FP32: nodes, FP64: node components) and `nodes` of them go to a
 // thread.  Few threads leave each more registers, which hold a level's
 // constants and node offsets across its phases (16^3 step: 796 us with 128 of
-// them against 870 with 64; 80 x 40 x 40 and 48^3 levels' planes of 800 and 576
-// nodes gain 1 and 2% of a step from bounds of 832 and 640 instead of 1024); on
+// them against 870 with 64; steps whose top level here has planes of 40 x 20 and
+// 24 x 24 nodes gain 1 and 2% from bounds of 832 and 640 instead of 1024); on
 // 32 x 32 planes 512 threads with two nodes each also pass barriers sooner
 // (64^3 solve 2.83 against 2.92 ms), on the smaller ones one node a thread
 // stays faster.
@@ -640,14 +640,13 @@ template <>
 const std::vector<SmallKernel<double>> &small_kernels() {
     static const std::vector<SmallKernel<double>> k = {
         {k_small_cycle<double, 1, 256>, 256, 1},
-        {k_small_cycle<double, 1, 768>, 768, 1},
-        {k_small_cycle<double, kMaxNodes, 512>, 512 * kMaxNodes, kMaxNodes}};
+        {k_small_cycle<double, 1, 768>, 768, 1}};
     return k;
 }
 
 // shared-memory layout of the plan; false if it does not fit
 template <typename T>
-bool small_layout(const Dims *d, const Coarse<T> *op, int nlev, bool pad, SmallPlan<T> &g) {
+bool small_layout(const Dims *d, const Coarse<T> *op, int nlev, SmallPlan<T> &g) {
     long off = 0;
     constexpr int N = kNode<T>;
     // nodes a shared-memory wavefront serves: eight of 16 bytes in FP32, the
@@ -672,9 +671,9 @@ bool small_layout(const Dims *d, const Coarse<T> *op, int nlev, bool pad, SmallP
             L.mnh = magic(L.np / 4);
             // two rows of a colour apart, as if its lanes went on in one row
             if (N == 4)
-                while (pad && (2 * (L.w / N) - L.hx) % unit > 1) L.w += N;
+                while ((2 * (L.w / N) - L.hx) % unit > 1) L.w += N;
             else
-                while (pad && (2 * L.w - N * L.hx) % unit > 1) L.w++;
+                while ((2 * L.w - N * L.hx) % unit > 1) L.w++;
         }
         L.pl = L.ny * L.w;
         if (l + 1 < nlev) L.pl = (L.pl + 3) & ~3;  // planes are copied 16 bytes at a time
@@ -710,9 +709,11 @@ bool small_layout(const Dims *d, const Coarse<T> *op, int nlev, bool pad, SmallP
 }  // namespace
 
 // The plan for levels d[0 .. nlev-1] (d[nlev-1] solved densely), or false if
-// they do not suit the kernel: their planes must fit the cluster's shared
-// memory, with at most `max_nodes` nodes on the top level (beyond it, the
-// whole chip is faster than 16 SMs).
+// they do not suit the kernel: at most kSmallCoarse unknowns on the coarsest
+// level (a CTA takes every 16th row of its dense solve), planes that fit the
+// cluster's shared memory and its threads (up to 32x32x48 nodes, planes of up to
+// 2560), and at most `max_nodes` nodes on the top level (beyond it, the whole
+// chip is faster than 16 SMs).
 template <typename T>
 bool small_plan(const Dims *d, const Coarse<T> *op, int nlev, int ncoarse, const double *Ainv,
                 int nu1, int nu2, long max_nodes, SmallPlan<T> &g) {
@@ -724,8 +725,7 @@ bool small_plan(const Dims *d, const Coarse<T> *op, int nlev, int ncoarse, const
     g.nu2 = nu2;
     g.ncoarse = ncoarse;
     g.Ainv = Ainv;
-    // with the bank-conflict-free row pitch if that fits, else packed rows
-    if (!small_layout(d, op, nlev, true, g) && !small_layout(d, op, nlev, false, g)) return false;
+    if (!small_layout(d, op, nlev, g)) return false;
     const int np = g.lev[0].np * (sizeof(T) == 8 ? 3 : 1);  // FP64: a thread a component
     g.nodes = 0;
     for (const SmallKernel<T> &k : small_kernels<T>()) {
