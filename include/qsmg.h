@@ -106,8 +106,10 @@ typedef struct {
  *                 observed V-cycle contraction.
  *   flags         0 or an OR of: MG_FLAG_COLOUR_PASSES runs FP32 sweeps as
  *                 eight colour launches instead of the two-phase kernels
- *                 (row strips, whole planes, tiles); MG_FLAG_NO_GRAPH issues the FP32 inner cycles as
- *                 plain launches instead of replaying a CUDA graph captured
+ *                 (row strips, persistent rows) and the one-launch V-cycles
+ *                 of the small levels; MG_FLAG_NO_GRAPH issues the FP32 inner
+ *                 cycles, and the levels below the finest of an FP64 V-cycle,
+ *                 as plain launches instead of replaying CUDA graphs captured
  *                 at their first use; MG_FLAG_FUSED_SWEEP runs each
  *                 finest-level FP32 sweep as one cooperative launch (both
  *                 k-parities, with ready flags between neighbouring row
@@ -116,7 +118,7 @@ typedef struct {
  *                 kept for comparison); MG_FLAG_UNFUSED_TRANSFERS runs the
  *                 finest-level FP32 residual and its restriction as two passes
  *                 with the residual stored instead of one fused pass (kept
- *                 for comparison); MG_FLAG_ADVECT_STRESS adds to the
+ *                 for comparison; coarse levels stay fused); MG_FLAG_ADVECT_STRESS adds to the
  *                 intermediate stress of Eq. (27) the advection term
  *                 -(v.grad) sigma of the general constitutive law (section 2),
  *                 sigma* -= dt (u.grad) sigma^n with u the mean of each cell's
@@ -250,8 +252,9 @@ mg_status mg_residual32(mg_ctx *ctx, int level, const float *b, const float *x, 
 
 /* bc = T^T (b - A_level x) in FP32 (level -> level + 1): the residual and its
  * restriction (section 3.6), as the mixed-precision V-cycle computes them.
- * On the finest level, where its row-strip kernel takes the grid, the two
- * are fused and the residual is never stored: the kernel applies the x and y
+ * Where the persistent row-strip kernel takes the level (16 columns and more
+ * on the finest one, 128 and more on a coarse one, in planes of 9 rows and
+ * more), the two are fused and the residual is never stored: the kernel applies the x and y
  * parts of the full weighting to each tile's residual and a second kernel
  * the z part.  b, x: (3, nz+1, ny, nx) of the level, natural column order;
  * bc: the next level's (3, nz/2+1, ny/2, nx/2), wall planes not written.
@@ -261,7 +264,9 @@ mg_status mg_residual_restrict32(mg_ctx *ctx, int level, const float *b, const f
                                  float *bc);
 
 /* nsweeps Gauss-Seidel sweeps on level `level`, colours 0..7 if
- * descending == 0 else 7..0; FP64 (precision 0) or FP32 arrays (precision 1). */
+ * descending == 0 else 7..0; FP64 (precision 0) or FP32 arrays (precision 1).
+ * On the coarsest level, which the cycles solve directly and whose sizes may be
+ * odd, the last plane, row or column of an odd size is left as it is. */
 mg_status mg_smooth(mg_ctx *ctx, int level, const void *b, void *x, int nsweeps, int descending,
                     int precision);
 

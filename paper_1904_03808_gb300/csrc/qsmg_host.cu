@@ -343,7 +343,6 @@ mg_status prof_drain(mg_ctx *ctx) {
 
 // ---------------------------------------------------------------- norms
 
-// ||r||^2 from the partial sums of the last reduction kernel
 // the fused sweep's error word (set when a bounded wait for a neighbouring
 // tile gave up), read after the stream has drained; cleared when reported
 mg_status sync_error(mg_ctx *ctx) {

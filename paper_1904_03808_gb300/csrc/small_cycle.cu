@@ -17,8 +17,8 @@
 //     folded into the right-hand side, then the 4 in-plane colours run on the
 //     plane, so every node sees the neighbour values of the sequential order.
 //     The halos written in a phase are not those read in it;
-//   - one thread a node in FP32, one a node component in FP64 (or up to
-//     kMaxNodes of them on planes larger than a CTA).
+//   - one thread a node in FP32 (up to kMaxNodes of them on the largest
+//     planes), one a node component in FP64.
 // Levels start from x = 0 below the top, so the first phase of their first
 // pre-sweep has no neighbour planes to fold.  Every level's operator, the
 // finest included, is used in its parity-class form (Coarse<T>).

@@ -1,11 +1,12 @@
 // smoother_rows.cu -- persistent row-strip Gauss-Seidel sweep phases (FP32) for
 // the finest level (structured 19-point operator of the scaled Eq. 30) and for
 // coarse levels of rows >= 128 nodes (27-point block stencil, Eq. 36), and
-// the residuals of those levels.
+// the residuals of those levels; coarse_rows_fit and fine_rows_fit say which
+// levels take it.
 //
-// One 8-colour sweep runs as two phase launches, as in strip.cu: the planes of one k-parity (4 in-plane colours each, reading the old
-// z-neighbour planes), then the planes of the other parity (reading the
-// first phase's output).  A CTA owns whole rows of a plane where they have at
+// One 8-colour sweep runs as two phase launches, as in strip.cu: the planes of
+// one k-parity (4 in-plane colours each, reading the old z-neighbour planes),
+// then the planes of the other parity (reading the first phase's output).  A CTA owns whole rows of a plane where they have at
 // most 512 nodes, so the periodic x direction needs no halo, and tiles of
 // longer rows with 8 halo columns a side.  k_gs_rows_p copies the rows of
 // each tile into shared memory with cp.async while the other CTAs on the SM
@@ -46,7 +47,9 @@ namespace {
 //   z_0 = (L0+H0) + kq (D2(x+1) - D2(x-1)),
 //   z_1 = (L1+H1) + kq (D2(y+1) - D2(y-1)),
 //   z_2 = lp (L2+H2) + kq ((D0(x+1) - D0(x-1)) + (D1(y+1) - D1(y-1))),
-// with D = H - L, streamed row by row so each plane value is loaded once.
+// with D = H - L, from the z-neighbour planes' rows jj-1, jj and jj+1 in shared
+// memory.
+
 // m, p: the in-plane neighbours of the node of x-parity E at window row jj in
 // columns x - 1 and x + 1, by component and row (jj-1, jj, jj+1), from the own
 // column values P and the far-side neighbour column X[c * sc + row * sr + xn]
