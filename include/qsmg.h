@@ -252,11 +252,11 @@ mg_status mg_residual32(mg_ctx *ctx, int level, const float *b, const float *x, 
 
 /* bc = T^T (b - A_level x) in FP32 (level -> level + 1): the residual and its
  * restriction (section 3.6), as the mixed-precision V-cycle computes them.
- * Where the persistent row-strip kernel takes the level (16 columns and more
- * on the finest one, 128 and more on a coarse one, in planes of 9 rows and
- * more), the two are fused and the residual is never stored: the kernel applies the x and y
- * parts of the full weighting to each tile's residual and a second kernel
- * the z part.  b, x: (3, nz+1, ny, nx) of the level, natural column order;
+ * Where the persistent row-strip kernel takes the level (a multiple of 4
+ * columns, of 8 beyond 256; 16 and more on the finest level, 128 and more on a
+ * coarse one; 9 rows and more), the two are fused and the residual is never
+ * stored: the kernel applies the x and y parts of the full weighting to each
+ * tile's residual and a second kernel the z part.  b, x: (3, nz+1, ny, nx) of the level, natural column order;
  * bc: the next level's (3, nz/2+1, ny/2, nx/2), wall planes not written.
  * Uses the solver's own FP32 buffers (must not overlap a solve on the same
  * context).  Errors: MG_ERR_ARG (null array, no coarser level), MG_ERR_CUDA. */
