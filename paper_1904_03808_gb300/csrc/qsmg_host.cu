@@ -1165,6 +1165,7 @@ mg_status mg_setup(const mg_grid *grid, const mg_moduli *moduli, const mg_bc *bc
                        opts->nu1, opts->nu2, LONG_MAX, ctx->s32))
             ctx->top32 = l;
     }
+    ctx->s32.fine = ctx->top32 == 0;
     if (ctx->top32 == 0) ctx->split0 = 0;  // its arrays are in natural order
     *out = ctx;
     return MG_OK;

@@ -169,6 +169,7 @@ struct SmallLevel {
 template <typename T>
 struct SmallPlan {
     int nlev, nu1, nu2, ncoarse;
+    int fine;  // the top level is the grid's finest
     int plmax, scratch;  // the largest plane; offset of the scratch
     int threads, nodes;  // threads of a CTA, nodes of a plane a thread may own
     const void *kernel;

@@ -102,18 +102,21 @@ __device__ __forceinline__ int col_of(const SmallLevel &L, int i) {
 //   A(y) + U(y - 1) + V(y + 1)
 // to row y, each of A, U, V three components formed from columns x - 1, x,
 // x + 1 of one row only: 46 operations a node instead of 116.
-template <typename T>
-__device__ __forceinline__ void z_row(const Coarse<T> &c, const T *lo, const T *hi, const Node &n,
-                                      T A[3], T U[3], T V[3]) {
+// SHARES: of S - 2 p, p the node between up and down (plane_residual_at).
+template <bool SHARES, typename T>
+__device__ __forceinline__ void z_row(const Coarse<T> &c, const T *lo, const T *P, const T *hi,
+                                      const Node &n, T A[3], T U[3], T V[3]) {
     T S[3][3], D[3][3];  // [column][component]
 #pragma unroll
     for (int x = 0; x < 3; x++) {
-        T l[3], h[3];
+        T l[3], h[3], p[3];
         load3(lo + n.r[1] + n.c[x], l);
         load3(hi + n.r[1] + n.c[x], h);
+        if (SHARES) load3(P + n.r[1] + n.c[x], p);
 #pragma unroll
         for (int a = 0; a < 3; a++) {
             S[x][a] = h[a] + l[a];
+            if (SHARES) S[x][a] -= T(2) * p[a];
             D[x][a] = h[a] - l[a];
         }
     }
@@ -151,6 +154,33 @@ __device__ __forceinline__ void plane_at(const Coarse<T> &c, const T *P, const N
             if (x != 1 || y != 1) load3(P + n.r[y] + n.c[x], v[y][x]);
     auto u = [&](int b, int dx, int dy) -> T { return v[dy + 1][dx + 1][b]; };
     coarse_plane_terms(c, u, o);
+}
+
+// A x at node n of plane P but for z_row's terms of S - 2 p.  The rows of A sum to
+// zero, so the centre term is the shares of the 26 others: with S - 2 p above,
+// each class of in-plane neighbours has the sum of its weights over the three
+// planes and gives up its share of the centre before it is weighted, and no sum of
+// the size of the centre term is rounded.  (A sweep rounds such sums, and a
+// residual that rounds the same ones does not see what its fixed point lost.)
+template <typename T>
+__device__ __forceinline__ void plane_residual_at(const Coarse<T> &c, const T *P, const Node &n,
+                                                  T o[3]) {
+    T v[3][3][3];  // [row][column][component]
+#pragma unroll
+    for (int y = 0; y < 3; y++)
+#pragma unroll
+        for (int x = 0; x < 3; x++) load3(P + n.r[y] + n.c[x], v[y][x]);
+#pragma unroll
+    for (int a = 0; a < 3; a++) {
+        const T p = v[1][1][a];
+        const T sx = (v[1][0][a] + v[1][2][a]) - T(2) * p, sy = (v[0][1][a] + v[2][1][a]) - T(2) * p;
+        const T sd = ((v[0][0][a] + v[2][2][a]) + (v[0][2][a] + v[2][0][a])) - T(4) * p;
+        o[a] = (c.cd[a][1] + T(2) * c.cd[a][5]) * sx + (c.cd[a][2] + T(2) * c.cd[a][6]) * sy +
+               (c.cd[a][3] + T(2) * c.cd[a][7]) * sd;
+    }
+    const T g = c.g[2][0] + T(2) * c.g[2][1];
+    o[0] += g * ((v[2][2][1] - v[0][2][1]) - (v[2][0][1] - v[0][0][1]));
+    o[1] += g * ((v[2][2][0] - v[0][2][0]) - (v[2][0][0] - v[0][0][0]));
 }
 
 // Component a alone of z_row and of plane_at: in FP64 a warp instruction takes
@@ -265,11 +295,12 @@ struct Walker {
         }
     }
 
-    // r = right-hand side of plane k (RES: zero) minus the dz = +-1 terms, at
-    // own nodes
-    template <bool RES = false>
-    __device__ __forceinline__ void fold(const Coarse<T> &c, const T *b, const T *lo, const T *hi,
-                                         T (&r)[NODES][NC]) const {
+    // r = right-hand side of plane P (RES: zero) minus the dz = +-1 terms (SHARES:
+    // less their shares of the centre term), at own nodes
+    template <bool RES = false, bool SHARES = false>
+    __device__ __forceinline__ void fold(const Coarse<T> &c, const T *b, const T *P,
+                                         T (&r)[NODES][NC], int pl) const {
+        const T *lo = P - pl, *hi = P + pl;
         T *U = sm + g.scratch, *V = U + g.plmax;
 #pragma unroll
         for (int u = 0; u < NODES; u++) {
@@ -279,7 +310,7 @@ struct Walker {
             if constexpr (COMP)
                 z_row_c(c, lo, hi, node[u], comp[u], r[u][0], up[0], vp[0]);
             else
-                z_row(c, lo, hi, node[u], r[u], up, vp);
+                z_row<SHARES>(c, lo, P, hi, node[u], r[u], up, vp);
             put(U + o, up);
             put(V + o, vp);
             if (!RES) get(b + o, bp);
@@ -344,7 +375,7 @@ struct Walker {
                             if (node[u].colour >= 0)
                                 get(b + node[u].r[1] + node[u].c[1] + comp[u], r[u]);
                     } else {
-                        fold(c, b, P - pl, P + pl, r);
+                        fold(c, b, P, r, pl);
                     }
                     // colours (F,F), (1-F,F), (F,1-F), (1-F,1-F) in (x, y) parity
 #pragma unroll 1
@@ -390,6 +421,8 @@ struct Walker {
         const SmallLevel &L = g.lev[l], &C = g.lev[l + 1];
         const Coarse<T> &c = g.op[l];
         const int nc3 = 3 * C.np, k0 = first(l), k1 = last(l);
+        // on the finest level, whose residual limits what the cycles reach
+        const bool shares = !COMP && g.fine && l == 0;
         T *R = sm + g.scratch;  // in place of U
         if (tid < act)
 #pragma unroll 1
@@ -398,20 +431,28 @@ struct Walker {
                 const T *P = own(l, L.x, k), *B = own(l, L.b, k);
                 // the right-hand side last: it would lose digits to the
                 // neighbour sums, which cancel with the centre term first
-                fold<true>(c, B, P - L.pl, P + L.pl, r);
+                if (shares)
+                    fold<true, true>(c, B, P, r, L.pl);
+                else
+                    fold<true>(c, B, P, r, L.pl);
                 sync_act();
 #pragma unroll
                 for (int u = 0; u < NODES; u++) {
                     if (node[u].colour < 0) continue;
-                    T o[NC];
-                    in_plane(c, P, u, o);
+                    T o[NC], b[NC];
                     const int q = node[u].r[1] + node[u].c[1] + comp[u];
-                    T x[NC], b[NC];
-                    get(P + q, x);
+                    if (shares) {
+                        if constexpr (!COMP) plane_residual_at(c, P, node[u], o);
+                    } else {
+                        T x[NC];
+                        in_plane(c, P, u, o);
+                        get(P + q, x);
+#pragma unroll
+                        for (int a = 0; a < NC; a++) o[a] += c.cd[comp[u] + a][0] * x[a];
+                    }
                     get(B + q, b);
 #pragma unroll
-                    for (int a = 0; a < NC; a++)
-                        o[a] = (r[u][a] - (o[a] + c.cd[comp[u] + a][0] * x[a])) + b[a];
+                    for (int a = 0; a < NC; a++) o[a] = (r[u][a] - o[a]) + b[a];
                     put(R + q, o);
                 }
                 sync_act();

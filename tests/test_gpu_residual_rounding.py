@@ -93,3 +93,24 @@ def test_finest_residual_of_a_constant_field(ctx, value):
     lp = np.float32((I.lame_lambda(K, MU) + 2 * MU) / MU)
     assert not r[:2].any()
     assert float(r[2].abs().max()) <= 0.5 * np.spacing(np.float32(2 * lp * value))
+
+
+@pytest.mark.parametrize("shape", [(24, 24, 24), (32, 32, 32), (32, 32, 40), (32, 32, 48)])
+def test_floor_of_the_cluster_cycle(shape):
+    """Ten FP32 cycles of four and four sweeps, whole grid in one cluster, towards
+    the linear profile that the moving walls leave: a sweep rounds a node's sum and
+    its quotient, two units; the eight sweeps after a residual leave 16, the
+    cycles before them, contracting below one half, at most as many again."""
+    nx, ny, nz = shape
+    ctx = Context(*shape, 2e-2 / nx, K, MU, precision=MG_MIXED, nu1=4, nu2=4, max_cycles=1,
+                  inner_cycles=10)
+    z = torch.linspace(-1, 1, nz + 1, dtype=torch.float64, device="cuda")[:, None, None]
+    v = torch.zeros((3, nz + 1, ny, nx), dtype=torch.float64, device="cuda")
+    want = v.clone()
+    for a, c in enumerate((1.1, 0.7, 0.9)):
+        want[a] = c * z
+        v[a, 0], v[a, nz] = -c, c
+    ctx.solve(torch.zeros_like(v), v, tol=0.0)
+    err = torch.linalg.vector_norm(v - want) / torch.linalg.vector_norm(want)
+    assert float(err) <= 32 * 2.0 ** -24
+    ctx.close()
